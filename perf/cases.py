@@ -35,8 +35,8 @@ def listed():
         _star("star100", n=100, depth=20, regions=2, width=8, n_t=10, marginal=12, zstrings=64, shots=10000),
         # the largest single circuit: 20736 variants of a 500-wire body, 4^8 cut terms
         _star("star500", n=500, depth=30, regions=4, width=1, n_t=16, marginal=16, zstrings=0, shots=16384),
-        # a wide contraction in BF16 (tensor cores): 4^6 cut terms, 2^12 hub outputs, an odd qubit count
-        _star("star301_bf16", n=301, depth=24, regions=3, width=2, n_t=9, marginal=15, zstrings=0, shots=8192,
+        # a wide contraction in BF16 (tensor cores): 4^8 cut terms, 2^9 hub outputs, an odd qubit count
+        _star("star301_bf16", n=301, depth=24, regions=4, width=2, n_t=9, marginal=13, zstrings=0, shots=4096,
               precision="bf16"),
         # a VQE sweep: many deep, narrow circuits in one plan, cuts searched, launch shapes tuned
         dict(name="vqe300x64", kind="vqe", n=300, rounds=5, circuits=64, marginal=10, zstrings=8, shots=5000,
