@@ -53,6 +53,8 @@ struct ccs_ctx_s {
 };
 
 cudaStream_t ccs::c_stream(ccs_ctx c) { return c->stream; }
+int ccs::c_device(ccs_ctx c) { return c->device; }
+int ccs::c_sm_count(ccs_ctx c) { return c->sm_count; }
 
 namespace {
 enum Stage { ST_CLIFFORD = 0, ST_SAMPLE = 1, ST_STATEVEC = 2, ST_FOLD = 3, ST_RECOMB = 4, ST_OPERANDS = 5, ST_N = 6 };
@@ -104,6 +106,12 @@ cudaMemPool_t lib_pool(int device) {
     g_pools[device] = pool;
   }
   return g_pools[device];
+}
+
+void trim_pool(int device) {   // hand the pool's unused memory back
+  if (device < 0 || device >= kMaxPoolDevices) return;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (g_pools[device]) cudaMemPoolTrimTo(g_pools[device], 0);
 }
 
 void* dalloc(ccs_ctx c, size_t bytes) {
@@ -276,25 +284,33 @@ struct Staging {
     if (items.empty()) return true;
     char* d = A.get<char>(total);
     if (!d) return false;
-    // the previous copy out of the staging buffer must be done before reuse
-    // (waits for that copy only, not for other work on the stream)
-    if (!upload_wait(c)) return false;
-    if (c->pinned_bytes < total) {
-      if (c->pinned) cudaFreeHost(c->pinned);
-      c->pinned = nullptr;
-      c->pinned_bytes = 0;
-      if (cudaMallocHost(&c->pinned, total) != cudaSuccess) return false;
-      c->pinned_bytes = total;
-    }
+    if (!reserve(c, total)) return false;
     for (auto& it : items) {
       if (it.bytes) std::memcpy(c->pinned + it.off, it.src, it.bytes);
       *it.out = d + it.off;
     }
-    if (cudaMemcpyAsync(d, c->pinned, total, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) return false;
-    if (!c->upload_ev && cudaEventCreateWithFlags(&c->upload_ev, cudaEventDisableTiming) != cudaSuccess) return false;
-    if (cudaEventRecord(c->upload_ev, c->stream) != cudaSuccess) return false;
-    c->upload_pending = true;
+    return send(c, d, total) == cudaSuccess;
+  }
+  // The pinned buffer with room for `bytes`: the previous copy out of it must
+  // be done before reuse (waits for that copy only, not for other work on the
+  // stream).
+  static bool reserve(ccs_ctx c, size_t bytes) {
+    if (!upload_wait(c)) return false;
+    if (c->pinned_bytes < bytes) {
+      if (c->pinned) cudaFreeHost(c->pinned);
+      c->pinned = nullptr;
+      c->pinned_bytes = 0;
+      if (cudaMallocHost(&c->pinned, bytes) != cudaSuccess) return false;
+      c->pinned_bytes = bytes;
+    }
     return true;
+  }
+  static cudaError_t send(ccs_ctx c, void* dst, size_t bytes) {
+    cudaError_t e = cudaMemcpyAsync(dst, c->pinned, bytes, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && !c->upload_ev) e = cudaEventCreateWithFlags(&c->upload_ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(c->upload_ev, c->stream);
+    if (e == cudaSuccess) c->upload_pending = true;
+    return e;
   }
   static bool upload_wait(ccs_ctx c) {
     if (!c->upload_pending) return true;
@@ -303,6 +319,20 @@ struct Staging {
     return true;
   }
 };
+
+}  // namespace
+
+void* ccs::pool_alloc(ccs_ctx c, size_t bytes) {
+  void* p = nullptr;
+  cudaMemPool_t pool = lib_pool(c->device);
+  const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, c->stream) : cudaMallocAsync(&p, bytes, c->stream);
+  return e == cudaSuccess ? p : nullptr;
+}
+void ccs::pool_trim(int device) { trim_pool(device); }
+char* ccs::stage_reserve(ccs_ctx c, size_t bytes) { return Staging::reserve(c, bytes) ? c->pinned : nullptr; }
+cudaError_t ccs::stage_send(ccs_ctx c, void* dst, size_t bytes) { return Staging::send(c, dst, bytes); }
+
+namespace {
 
 template <class T>
 bool upload(ccs_ctx c, Allocs& A, const std::vector<T>& h, T** out) {
@@ -448,7 +478,7 @@ static int learned_pick(ccs_ctx c, const Problem& P, const std::vector<CutCandid
   ccs_graph_batch b{goff.back(), nc, X.data(), rowptr.data(), col.data(), val.data(), valt.data(), goff.data(),
                     glob.data()};
   std::vector<float> pred(nc);
-  if (mpnn_predict(c->cut_model, &b, pred.data()) != CCS_OK) return fail(c, CCS_ERR_CUDA, "cut model forward");
+  if (mpnn_predict(c, c->cut_model, &b, pred.data()) != CCS_OK) return fail(c, CCS_ERR_CUDA, "cut model forward");
   *pick = idx[std::min_element(pred.begin(), pred.end()) - pred.begin()];
   return CCS_OK;
 }
@@ -541,10 +571,7 @@ void ccs_destroy(ccs_ctx c) {
   if (c->side) cudaStreamDestroy(c->side);
   if (c->pinned) cudaFreeHost(c->pinned);
   if (c->upload_ev) cudaEventDestroy(c->upload_ev);
-  if (c->own_alloc && !c->host_only && c->device >= 0 && c->device < kMaxPoolDevices) {
-    std::lock_guard<std::mutex> lk(g_pool_mu);   // hand the pool's unused memory back
-    if (g_pools[c->device]) cudaMemPoolTrimTo(g_pools[c->device], 0);
-  }
+  if (c->own_alloc && !c->host_only) trim_pool(c->device);
   delete c;
 }
 

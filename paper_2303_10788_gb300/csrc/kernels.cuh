@@ -296,7 +296,18 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
                              float* scratch, double* marg_out, double* zexp_out, cudaStream_t s);
 // context stream; learned scorer helpers (mpnn.cu, features.cpp)
 cudaStream_t c_stream(ccs_ctx c);
-int mpnn_predict(ccs_mpnn n, const ccs_graph_batch* b, float* pred);
+int c_sm_count(ccs_ctx c);
+int c_device(ccs_ctx c);
+// Memory of one call: from the library's stream-ordered pool of the context's
+// device, on its stream (released with cudaFreeAsync on that stream; NULL on
+// failure).  pool_trim hands the pool's unused memory back to the driver.
+void* pool_alloc(ccs_ctx c, size_t bytes);
+void pool_trim(int device);
+// The context's pinned staging buffer, free to be written (the previous copy
+// out of it is done), and the copy of its first `bytes` to the device.
+char* stage_reserve(ccs_ctx c, size_t bytes);
+cudaError_t stage_send(ccs_ctx c, void* dst, size_t bytes);
+int mpnn_predict(ccs_ctx c, ccs_mpnn n, const ccs_graph_batch* b, float* pred);
 int featurize(const Problem& p, const std::vector<ccs_cut>& cuts, std::vector<float>& x, std::vector<int>& rowptr,
               std::vector<int>& col, std::vector<float>& val, std::vector<float>& val_t, std::vector<float>& glob,
               std::string& err);
