@@ -346,6 +346,13 @@ bool upload(ccs_ctx c, Allocs& A, const std::vector<T>& h, T** out) {
 
 }  // namespace
 
+// Tree contractions: a problem's steps but the last run in one CTA up to this
+// many multiply-adds (512 threads, a few microseconds; a level launched on its
+// own costs about as much), and the doubles of intermediate tensors a plan may
+// hold (512 MB; a problem beyond that is summed directly).
+constexpr double kTreeSmallWork = 1 << 16;
+constexpr long long kTreeTmpMax = 1ll << 26;
+
 struct ccs_plan_s {
   ccs_ctx ctx = nullptr;
   bool host_only = false;
@@ -387,7 +394,12 @@ struct ccs_plan_s {
   long long n_qrows = 0;            // operand-row flags of the Clifford hubs
   bool stitch_ok = true;            // every Clifford hub has at most 4 quantum outputs
   bool tableau_fits = true;         // every Clifford fragment's whole tableau fits in shared memory
-  bool all_star = true;
+  bool all_star = true;             // no problem is summed over its whole cut index for every output
+  std::vector<GStep> gsteps;        // tree contractions (problems that are no stars)
+  std::vector<FoldSet> tree_levels;
+  int* d_tree_small = nullptr;
+  int n_tree_small = 0;
+  long long n_gtmp = 0;             // doubles of their intermediate tensors
   ~ccs_plan_s() { A.release(); }
 };
 
@@ -435,6 +447,109 @@ struct ccs_res_s {
     A.release();
   }
 };
+
+// Order of a tree contraction (a problem with no fragment on every cut): the
+// fragment tensors are contracted pair by pair, disjoint pairs in one level
+// (levels follow each other, so fewer levels are fewer launches), cheapest
+// pairs first; a pair much dearer than the level's cheapest one waits unless
+// it is small in itself.  Steps are appended in level order; false when the
+// intermediate tensors would exceed `cap` doubles in total.
+namespace {
+struct GNode {
+  bool tmp;
+  long long off;
+  int zoff, level;
+  std::vector<int> cuts;       // open cuts, digit order
+  std::vector<int> marg;       // output bits, bit order
+};
+
+bool plan_tree(const std::vector<Frag>& frags, const Problem& P, const std::vector<FragDev>& fdev, int frag0,
+               int problem, long long cap, std::vector<GStep>& steps, std::vector<int>& levels, long long& tmp_len,
+               int& z_len) {
+  std::vector<GNode> nodes;
+  long long z = 0;
+  for (size_t l = 0; l < P.frag_ids.size(); ++l) {
+    const Frag& f = frags[P.frag_ids[l]];
+    GNode nd{false, fdev[frag0 + l].T_off, (int)z, 0, f.slots, f.marg_pos};
+    z += 1ll << (2 * f.slots.size());
+    nodes.push_back(nd);
+  }
+  const size_t first_step = steps.size();
+  const long long tmp0 = tmp_len;
+  struct Pair { double cost; int a, b, shared; };
+  for (int level = 0; nodes.size() > 1; ++level) {
+    std::vector<Pair> pairs;
+    for (int a = 0; a < (int)nodes.size(); ++a)
+      for (int b = a + 1; b < (int)nodes.size(); ++b) {
+        int sh = 0;
+        for (int c : nodes[a].cuts) sh += (int)std::count(nodes[b].cuts.begin(), nodes[b].cuts.end(), c);
+        const int open = (int)(nodes[a].cuts.size() + nodes[b].cuts.size()) - 2 * sh;
+        const int lg = (int)(nodes[a].marg.size() + nodes[b].marg.size()) + 2 * open + 2 * sh;
+        // tensors without a common cut (an outer product) only when nothing else is left
+        pairs.push_back(Pair{std::ldexp(1.0, lg) * (sh ? 1.0 : 1e18), a, b, sh});
+      }
+    std::stable_sort(pairs.begin(), pairs.end(), [](const Pair& x, const Pair& y) { return x.cost < y.cost; });
+    const double limit = std::max(16.0 * pairs.front().cost, 4096.0);
+    std::vector<char> used(nodes.size(), 0);
+    std::vector<GNode> next;
+    for (const Pair& pr : pairs) {
+      if (used[pr.a] || used[pr.b] || pr.cost > limit) continue;
+      if (pr.shared == 0 && !next.empty()) continue;
+      used[pr.a] = used[pr.b] = 1;
+      const GNode &A = nodes[pr.a], &B = nodes[pr.b];
+      GStep g{};
+      g.problem = problem;
+      g.a_tmp = A.tmp;
+      g.b_tmp = B.tmp;
+      g.a_off = A.off;
+      g.b_off = B.off;
+      g.za = A.zoff;
+      g.zb = B.zoff;
+      g.ma = (int)A.marg.size();
+      g.mb = (int)B.marg.size();
+      g.na = (int)A.cuts.size();
+      g.nb = (int)B.cuts.size();
+      GNode C{true, 0, 0, 0, {}, A.marg};
+      C.marg.insert(C.marg.end(), B.marg.begin(), B.marg.end());
+      for (int j = 0; j < g.na; ++j) {
+        const auto it = std::find(B.cuts.begin(), B.cuts.end(), A.cuts[j]);
+        if (it == B.cuts.end()) {
+          g.a_free[g.fa++] = (uint8_t)j;
+          C.cuts.push_back(A.cuts[j]);
+        } else {
+          g.a_sh[g.ns] = (uint8_t)j;
+          g.b_sh[g.ns++] = (uint8_t)(it - B.cuts.begin());
+        }
+      }
+      for (int j = 0; j < g.nb; ++j)
+        if (std::find(A.cuts.begin(), A.cuts.end(), B.cuts[j]) == A.cuts.end()) {
+          g.b_free[g.fb++] = (uint8_t)j;
+          C.cuts.push_back(B.cuts[j]);
+        }
+      g.last = nodes.size() == 2;
+      if (g.last) {
+        for (size_t j = 0; j < C.marg.size(); ++j) g.pos[j] = (uint8_t)C.marg[j];
+      } else {
+        const int lg = (int)C.marg.size() + 2 * (g.fa + g.fb);
+        if (lg > 40) return false;
+        C.off = g.out_off = tmp_len;
+        C.zoff = g.zo = (int)std::min<long long>(z, 1 << 30);
+        tmp_len += 1ll << lg;
+        z += 1ll << (2 * (g.fa + g.fb));
+        if (tmp_len - tmp0 > cap) return false;
+      }
+      steps.push_back(g);
+      levels.push_back(level);
+      next.push_back(std::move(C));
+    }
+    for (size_t i = 0; i < nodes.size(); ++i)
+      if (!used[i]) next.push_back(std::move(nodes[i]));
+    nodes.swap(next);
+  }
+  z_len = z <= kZTree ? (int)z : 0;
+  return steps.size() > first_step;
+}
+}  // namespace
 
 // Score up to 16 candidate cut sets with the learned model; index of the
 // smallest predicted time.
@@ -931,6 +1046,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       if (f.role == 1 && !f.clifford) { fidx_hn.push_back(fi); tp_hn.push_back(tp_hn.back() + t); }
       if (f.role == 2) { fidx_o.push_back(fi); tp_o.push_back(tp_o.back() + t); }
     }
+    std::vector<int> tree_level, tree_small;   // launch level of every step (-1: in the small problems' CTA)
     for (auto& P : plan->problems) {
       ProblemDev d{};
       d.k = (int)P.cuts.size();
@@ -945,10 +1061,32 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       plan->n_zexp += d.nz;
       plan->out_prefix.push_back(plan->n_marg);
       plan->z_prefix.push_back(plan->n_zexp);
-      if (P.hub < 0) {          // not a star: the general contraction over all fragment tensors
-        plan->all_star = false;
+      if (P.hub < 0) {          // not a star: fragment tensors contracted pair by pair
         d.general = 1;
         d.K = 1ll << (2 * d.k);
+        const size_t g0 = plan->gsteps.size();
+        const long long tmp0 = plan->n_gtmp;
+        if (plan_tree(plan->frags, P, plan->fdev, f0, (int)plan->pdev.size(), kTreeTmpMax - plan->n_gtmp, plan->gsteps,
+                      tree_level, plan->n_gtmp, d.g_zlen)) {
+          d.g_first = (int)g0;
+          d.g_count = (int)(plan->gsteps.size() - g0);
+          // few multiply-adds in all steps but the last: one CTA runs them
+          double work = 0.0;
+          for (size_t i = g0; i + 1 < plan->gsteps.size(); ++i) {
+            const GStep& g = plan->gsteps[i];
+            work += std::ldexp(1.0, g.ma + g.mb + 2 * (g.fa + g.fb + g.ns));
+          }
+          if (work <= kTreeSmallWork) {
+            tree_small.push_back((int)plan->pdev.size());
+            for (size_t i = g0; i + 1 < plan->gsteps.size(); ++i) tree_level[i] = -1;
+          }
+        } else {                // summed directly
+          plan->gsteps.resize(g0);
+          tree_level.resize(g0);
+          plan->n_gtmp = tmp0;
+          d.g_zlen = 0;
+          plan->all_star = false;
+        }
       }
       if (P.hub >= 0) {
         const int m_hub = plan->fdev[f0 + P.hub].m;
@@ -1060,6 +1198,27 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       plan->pdev.push_back(d);
     }
 
+    // the tree contractions' launches: one per level over all problems, the last steps together at the end
+    std::vector<std::vector<int>> tree_sets;
+    for (size_t i = 0; i < plan->gsteps.size(); ++i)
+      if (!plan->gsteps[i].last && tree_level[i] >= 0) {
+        if ((int)tree_sets.size() <= tree_level[i]) tree_sets.resize(tree_level[i] + 1);
+        tree_sets[tree_level[i]].push_back((int)i);
+      }
+    if (!plan->gsteps.empty()) {
+      tree_sets.emplace_back();
+      for (size_t i = 0; i < plan->gsteps.size(); ++i)
+        if (plan->gsteps[i].last) tree_sets.back().push_back((int)i);
+    }
+    std::vector<std::vector<long long>> tree_prefix(tree_sets.size(), std::vector<long long>{0});
+    for (size_t l = 0; l < tree_sets.size(); ++l)
+      for (int i : tree_sets[l]) {
+        const GStep& g = plan->gsteps[i];
+        tree_prefix[l].push_back(tree_prefix[l].back() + (1ll << (g.ma + g.mb + 2 * (g.fa + g.fb))));
+      }
+    std::vector<int*> d_tree_ids(tree_sets.size());
+    std::vector<long long*> d_tree_prefix(tree_sets.size());
+
     // the scratch holds every problem's R operand first, then the split-K partials
     plan->r_total = (plan->r_total + 3) & ~3ll;
     for (auto& d : plan->pdev) d.part_off += plan->r_total;
@@ -1103,8 +1262,21 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     st.add(plan->out_prefix, &plan->d_out_prefix);
     st.add(plan->z_prefix, &plan->d_z_prefix); st.add(plan->r_prefix, &plan->d_r_prefix);
     st.add(plan->blk_prefix, &plan->d_blk_prefix); st.add(plan->direct_items, &plan->d_direct_items);
+    GStep* dgs = nullptr;
+    if (!plan->gsteps.empty()) {
+      st.add(plan->gsteps, &dgs); st.add(tree_small, &plan->d_tree_small);
+      for (size_t l = 0; l < tree_sets.size(); ++l) {
+        st.add(tree_sets[l], &d_tree_ids[l]);
+        st.add(tree_prefix[l], &d_tree_prefix[l]);
+      }
+    }
     bool ok = st.commit(c, plan->A);
     if (!ok) { return fail(c, CCS_ERR_OOM, "plan upload failed"); }
+    plan->dp.gsteps = dgs;
+    plan->n_tree_small = (int)tree_small.size();
+    for (size_t l = 0; l < tree_sets.size(); ++l)
+      plan->tree_levels.push_back(FoldSet{d_tree_ids[l], d_tree_prefix[l], (int)tree_sets[l].size(),
+                                          tree_prefix[l].back()});
     dp.frags = dfr; dp.cops = dco; dp.nops = dno; dp.moments = dmo; dp.wires = dwi; dp.zoffs = dzo;
     dp.items_cliff = dic; dp.items_nc = din; dp.nc_basis_chunk = plan->nc_basis_chunk;
     dp.n_items_cliff = (int)items_c.size(); dp.n_items_nc = (int)items_nc.size();
@@ -1418,6 +1590,7 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
       d.rowbasis = r->A.get<unsigned long long>(std::max<long long>((long long)kRowBasisWords * p->dp.n_cliff_frags, 1));
       d.zimg = r->A.get<unsigned long long>(std::max<long long>(p->n_zimg, 1));
       d.pbasis = r->A.get<uint32_t>(std::max<long long>(p->n_pbasis, 1));
+      d.gtmp = r->A.get<double>(std::max<long long>(p->n_gtmp, 1));
 
       d.status = r->A.get<unsigned>(4);
       r->scratch = r->A.get<float>(std::max<long long>(p->r_total + p->part_total, 1));
@@ -1438,7 +1611,7 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
         r->rt_scratch = r->A.get<uint16_t>(p->rt_total);
       }
       if (!d.spaces || !d.dist || !d.qnz || !d.zval || !d.T || !d.TQ || !d.marg || !d.zexp || !d.work || !d.status ||
-          !d.body || !d.rowbasis || !d.zimg || !d.fragcnt || !d.pbasis ||
+          !d.body || !d.rowbasis || !d.zimg || !d.fragcnt || !d.pbasis || !d.gtmp ||
           !r->scratch || (p->rt_total && (!d.TQh || !r->rt_scratch))) {
         return fail(c, CCS_ERR_OOM, "result allocation failed");
       }
@@ -1583,7 +1756,8 @@ int ccs_recombine(ccs_ctx c, ccs_plan p, ccs_res r, const ccs_recomb_opts* opts,
                    p->d_direct_items, (int)p->direct_items.size(), (int)p->direct_stage_floats, p->chain,
                    p->d_r_prefix, p->d_blk_prefix, p->d_out_prefix, p->d_z_prefix, p->max_tile_smem,
                    p->pdev.data(), (int)p->pdev.size(), r->rt_scratch, tc ? 1 : 0, stitched ? 1 : 0, KRange{0, -1},
-                   p->all_star ? 0 : 1};
+                   p->all_star ? 0 : 1, p->tree_levels.data(), (int)p->tree_levels.size(), p->d_tree_small,
+                   p->n_tree_small};
     if (opts && (opts->k_lo || opts->k_hi)) {
       if (opts->k_hi && opts->k_hi <= opts->k_lo) return fail(c, CCS_ERR_INVALID_ARG, "empty cut-index range");
       if (opts->k_lo > (1ull << 62) || opts->k_hi > (1ull << 62)) return fail(c, CCS_ERR_INVALID_ARG, "bad range");
@@ -1998,7 +2172,8 @@ extern "C" int ccs_recombine_noalloc(ccs_ctx c, ccs_plan p, ccs_res r, int preci
                    p->d_direct_items, (int)p->direct_items.size(), (int)p->direct_stage_floats, p->chain,
                    p->d_r_prefix, p->d_blk_prefix, p->d_out_prefix, p->d_z_prefix, p->max_tile_smem,
                    p->pdev.data(), (int)p->pdev.size(), nullptr, 0, r->ep.mode == CCS_STITCH ? 1 : 0,
-                   KRange{0, -1}, p->all_star ? 0 : 1};
+                   KRange{0, -1}, p->all_star ? 0 : 1, p->tree_levels.data(), (int)p->tree_levels.size(), p->d_tree_small,
+                   p->n_tree_small};
     e = launch_recombine(p->dp, r->dr, precision, rz, scratch, marginal_out, zexp_out, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "recombine kernel");
     return CCS_OK;

@@ -71,11 +71,30 @@ struct ProblemDev {
   // the first leaf contracted while streaming (FP32, full range, dense rows):
   // its G1 = 4^s1 cut-digit rows per group against its table (N1 outputs),
   // then the other leaves' product table Rrest[group][NR] (NR = N / N1)
+  int g_first, g_count;    // general problems: the range of the tree contraction's steps (0: summed directly)
+  int g_zlen;              // doubles of the Z-string tensors of that tree (0: too many, summed directly)
   int fact, fl1, G1, N1, NR;
   long long fl1_T_off;     // T_off of that leaf (its table T'[x1][g1])
   int ndig1, ndigr;
   int dig1[kMaxCuts], digr[kMaxCuts];   // cut positions of the leaf's digits / of the other digits
 };
+
+// One pairwise step of a tree contraction (problems with no fragment on every
+// cut): out[oA | oB << ma][PA' | PB' << 2 fa] = sum over the ns shared cut
+// digits of A[oA][PA] B[oB][PB].  A and B are fragment tensors T_f (float,
+// index into DevRes::T) or earlier results (double, index into DevRes::gtmp);
+// the last step of a problem (fa = fb = 0) writes the marginal.
+struct GStep {
+  int problem, last;
+  int a_tmp, b_tmp;                 // 1: in gtmp
+  int ma, mb, fa, fb, ns;           // marginal bits; free and shared cut digits
+  int na, nb;                       // digits of A's and of B's index (fa + ns, fb + ns)
+  int za, zb, zo;                   // offsets of A, B and the result among the Z-string tensors (no marginal bits)
+  long long a_off, b_off, out_off;
+  uint8_t a_free[kMaxCuts], a_sh[kMaxCuts], b_free[kMaxCuts], b_sh[kMaxCuts];   // digit positions
+  uint8_t pos[kMaxMarginal];        // last step: output bit of every marginal bit of A, then of B
+};
+constexpr int kZTree = 1024;        // doubles of Z-string tensors a tree contraction stages per string
 
 // Device views of a plan + result.
 struct DevPlan {
@@ -105,6 +124,7 @@ struct DevPlan {
   int img_words_max;          // most Z-image words of one fragment
   const ProblemDev* problems;
   int n_problems;
+  const GStep* gsteps;         // tree contraction steps of the general problems
   const CliffordOp* prep_ops;  // 4
   const CliffordOp* basis_ops; // 3
   const float* prep_mats;      // 4 x 8
@@ -125,6 +145,7 @@ struct DevRes {
   float* T;
   float* TQ;               // contraction operands: Q for hubs, T' for the other fragments
   uint16_t* TQh;           // bf16 copy of the hubs' Q (tensor-core path), may be null
+  double* gtmp;            // tree contractions: the intermediate tensors
   double* marg;
   double* zexp;
   uint8_t* qnz;            // stitched results: per Clifford hub operand row, 1 unless identically zero
@@ -290,7 +311,11 @@ struct RecombSizes {
   int stitched;                  // 1: Clifford hubs' operand rows flagged in DevRes::qnz (zero rows
                                  //    of streamed problems are neither written nor read)
   KRange krange;                 // the cut-index terms summed ({0, -1}: all)
-  int has_general;               // 1: some problem is not a star
+  int has_general;               // 1: some problem is not a star and has no tree contraction
+  const FoldSet* tree_levels;    // host array: the tree contractions' steps (fidx), one launch each; the last
+  int n_tree_levels;             //    step of every problem is in the final entry
+  const int* tree_small;         // device list: problems whose steps but the last run in one CTA each
+  int n_tree_small;
 };
 cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, const RecombSizes& z,
                              float* scratch, double* marg_out, double* zexp_out, cudaStream_t s);
