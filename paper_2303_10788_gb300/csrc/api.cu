@@ -2033,10 +2033,10 @@ int ccs_ml_correct(ccs_ctx c, ccs_plan p, ccs_res r, int which) {
           i16_hub = i16_hub || mf.i16;
           mf.index = (int)recs.size();
           mf.blk0 = G.blocks;
-          mf.ev_off = floats;
-          floats += nb * Dm;
-          mf.vec_off = floats;
-          floats += nb * 2 * Dm * Dm;   // complex64 eigenvectors
+          auto up4 = [](long long x) { return (x + 3) & ~3ll; };    // 16-byte vectors
+          mf.ev_off = up4(floats);
+          mf.vec_off = up4(mf.ev_off + nb * Dm);
+          floats = mf.vec_off + nb * 2 * Dm * Dm;   // complex64 eigenvectors
           mf.total = (double)(1ll << F.qin);
           recs.push_back(mf);
           G.blocks += nb;
@@ -2076,7 +2076,7 @@ int ccs_ml_correct(ccs_ctx c, ccs_plan p, ccs_res r, int which) {
       return CCS_OK;
     }
     cudaError_t e = launch_ml_correct(p->dp, r->dr, mc.d_frags, mc.n_frags, mc.groups.data(), (int)mc.groups.size(),
-                                      mc.scratch, mc.theta, c->stream);
+                                      mc.scratch, mc.theta, c->stream, SideStream{c->side, c->fork_ev, c->join_ev});
     if (e != cudaSuccess) return cuda_fail(c, e, "correction kernels");
     if (mc.i16_hub) r->dr.hub_i16 = 0;   // the corrected hub operands are FP32 now
     if (mc.leaves.nf &&

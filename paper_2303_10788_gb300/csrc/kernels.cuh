@@ -269,11 +269,17 @@ struct MlGroup {
   int d, first, count;     // cut slots; range of MlFrag records
   long long blocks;        // sum of 2^m over them
 };
+// A second stream with the events that fork it from and join it to the main one.
+struct SideStream {
+  cudaStream_t stream;
+  cudaEvent_t fork, join;
+};
 // Eigendecomposition of every block, the threshold per fragment, and the
 // rebuilt T_f (and hub operands); d <= 6.  `scratch` holds the eigenvalues
 // and eigenvectors, `theta` one double per record.
 cudaError_t launch_ml_correct(const DevPlan& p, const DevRes& r, const MlFrag* d_frags, int n_frags,
-                              const MlGroup* groups, int n_groups, float* scratch, double* theta, cudaStream_t s);
+                              const MlGroup* groups, int n_groups, float* scratch, double* theta, cudaStream_t s,
+                              const SideStream& side);
 constexpr int kMlMaxSlots = 6;
 
 // Contraction operands of star problems: Q of each hub from its variant data
