@@ -1250,12 +1250,72 @@ __device__ __forceinline__ uint32_t space_point(const uint32_t (*tbl)[256], uint
 
 // A full-rank space in canonical form (pivots = lowest bits, reduced, offset
 // with every pivot bit clear) has the identity basis and a zero offset, so a
-// shot's outcome is its coefficient bits; checked, not assumed.
+// shot's outcome is its coefficient bits; checked, not assumed.  One warp, a
+// basis vector per lane (one thread reading them in turn took as long as a
+// hundred shots of the whole CTA).
 __device__ __forceinline__ bool space_is_identity(const SpaceRec& sp, int rank, int nA) {
-  if (rank != nA || sp.off != 0u) return false;
-  for (int j = 0; j < rank; ++j)
-    if (sp.basis[j] != (1u << j)) return false;
-  return true;
+  const int j = (int)threadIdx.x & 31;
+  const bool ok = j >= rank || sp.basis[j] == (1u << j);
+  return __all_sync(0xffffffffu, ok) && rank == nA && sp.off == 0u;
+}
+
+// All shots of a hub variant whose outcome is its coefficient bits, counted
+// in shared memory: byte, 16-bit or 32-bit counters.  The field's place in
+// its word, its word's byte address and its increment come from one shift, one
+// mask and one wrapping shift each, with no masked copy of the field.
+template <int CB>
+__device__ __forceinline__ void count_field(uint32_t* hist, uint32_t w, int sh, uint32_t cmask) {
+  if (CB == 32) {
+    const uint32_t at = (sh >= 2 ? w >> (sh - 2) : w << 2) & (cmask << 2);
+    atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(hist) + at), 1u);
+  } else {
+    const uint32_t f = w >> sh;
+    const uint32_t at = CB == 8 ? f & (cmask & ~3u) : (f << 1) & ((cmask << 1) & ~3u);
+    atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(hist) + at),
+              __funnelshift_l(0u, 1u, CB == 8 ? f << 3 : f << 4));     // 1 << (shift mod 32)
+  }
+}
+template <int CB>
+__device__ __forceinline__ void count_outcome(uint32_t* hist, uint32_t y) {
+  if (CB == 32) atomicAdd(hist + y, 1u);
+  else if (CB == 16) atomicAdd(hist + (y >> 1), 1u << ((y & 1u) << 4));
+  else atomicAdd(hist + (y >> 2), 1u << ((y & 3u) << 3));
+}
+template <int CB, int L>
+__device__ __forceinline__ void count_identity(uint32_t* hist, uint32_t shots, uint4 ctr, const PhiloxKeys& K,
+                                               uint32_t cmask) {
+  constexpr int S = L == 1 ? 4 : L == 2 ? 2 : 1, WB = 32 / S;
+  for (uint32_t g = threadIdx.x; (unsigned long long)(4 * S) * g < shots; g += blockDim.x) {
+    ctr.x = g;
+    const uint4 o = philox4x32_10(ctr, K);
+    const uint32_t w4[4] = {o.x, o.y, o.z, o.w};
+    if ((unsigned long long)(4 * S) * (g + 1) <= shots) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < S; ++h) count_field<CB>(hist, w4[j], h * WB, cmask);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < S; ++h)
+          if ((4 * g + j) * S + h < shots) count_field<CB>(hist, w4[j], h * WB, cmask);
+    }
+  }
+}
+// All shots of a hub variant (rank <= 16) into its histogram.
+template <int CB>
+__device__ __forceinline__ void count_shots(uint32_t* hist, bool ident, int rank, const uint32_t (*tbl)[256],
+                                            uint32_t off, uint32_t shots, uint4 ctr, const PhiloxKeys& K) {
+  const uint32_t cmask = (1u << rank) - 1u;
+  if (ident) {
+    if (rank <= 8) count_identity<CB, 1>(hist, shots, ctr, K, cmask);
+    else count_identity<CB, 2>(hist, shots, ctr, K, cmask);
+  } else if (rank <= 8) {
+    for_shots<1>(0u, shots, ctr, K, cmask, [&](uint32_t c) { count_outcome<CB>(hist, space_point<1>(tbl, off, c)); });
+  } else {
+    for_shots<2>(0u, shots, ctr, K, cmask, [&](uint32_t c) { count_outcome<CB>(hist, space_point<2>(tbl, off, c)); });
+  }
 }
 
 // Calls fn with the lookups a rank needs as a compile-time constant.
@@ -1391,7 +1451,7 @@ __device__ __forceinline__ void hub_pair_out_packed(unsigned (&p)[16], const int
 // p = lo + 2^16 hi with |lo|, |hi| <= shots < 2^15 at every stage keeps both
 // lanes recoverable (the low lane's borrow is undone when the pair is
 // written), and the variant's sign masks (bits < Q) pick by a select tree.
-template <int Q>
+template <int Q, bool WIDE>
 __device__ __forceinline__ void hub16_readout(const uint32_t* __restrict__ hist2, int m, int M, const int* s_czD,
                                               const int* s_czS, int nz, float* QT, int16_t* QH, float inv) {
   constexpr int NB = 1 << Q;
@@ -1399,7 +1459,15 @@ __device__ __forceinline__ void hub16_readout(const uint32_t* __restrict__ hist2
     const int o = 2 * o2;
     unsigned p[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) p[b] = hist2[((uint32_t)o | ((uint32_t)b << m)) >> 1];
+    for (int b = 0; b < NB; ++b) {
+      const uint32_t y = (uint32_t)o | ((uint32_t)b << m);
+      if (WIDE) {
+        const uint2 c = *reinterpret_cast<const uint2*>(hist2 + y);
+        p[b] = c.x + (c.y << 16);
+      } else {
+        p[b] = hist2[y >> 1];
+      }
+    }
 #pragma unroll
     for (int h = 1; h < NB; h <<= 1)
 #pragma unroll
@@ -1439,33 +1507,26 @@ __device__ __forceinline__ void hub16_readout(const uint32_t* __restrict__ hist2
 // the block before reading them.
 __device__ __forceinline__ void hub_variant_rows(const FragDev& F, int v, int* s_czD, int* s_czS, int* s_nzm) {
   if (threadIdx.x >= 32) return;
-  int beta[kMaxCuts], zpos[kMaxCuts], zout[kMaxCuts];
-  int nz, zm;
-  int t = v;
-  for (int i = 0; i < F.qin; ++i) t /= 4;
-  for (int j = 0; j < F.qout; ++j) { beta[j] = t % 3; t /= 3; }
-  int Dbase = 0, fixed_mask = 0;
-  nz = 0;
-  zm = 0;
+  unsigned pb = 0;                       // basis digits, two bits per quantum output
+  for (int j = 0, t = v >> (2 * F.qin); j < F.qout; ++j, t /= 3) pb |= (unsigned)(t % 3) << (2 * j);
+  int D = 0, smask = 0, nz = 0, zm = 0;
   for (int j = 0; j < F.n_slots; ++j) {
     const int code = F.slot_code[j], idx = code & 255;
+    const int beta = (int)(pb >> (2 * idx)) & 3;
     if ((code >> 8) == 0) {
-      int u = v;
-      for (int i = 0; i < idx; ++i) u /= 4;
-      Dbase |= (u % 4) << (2 * j);
-    } else if (beta[idx] == 2) {
-      zpos[nz] = j;
-      zout[nz++] = idx;
+      D |= ((v >> (2 * idx)) & 3) << (2 * j);
+    } else if (beta == 2) {              // the lane's choice of I or Z
+      const int pick = ((int)threadIdx.x >> nz) & 1;
+      D |= (pick * 3) << (2 * j);
+      smask |= pick << idx;
       zm |= 1 << idx;
+      ++nz;
     } else {
-      Dbase |= (beta[idx] == 0 ? 1 : 2) << (2 * j);
-      fixed_mask |= 1 << idx;
+      D |= (beta + 1) << (2 * j);        // X basis -> X, Y basis -> Y
+      smask |= 1 << idx;
     }
   }
   if ((int)threadIdx.x < (1 << nz)) {
-    int D = Dbase, smask = fixed_mask;
-    for (int i = 0; i < nz; ++i)
-      if ((threadIdx.x >> i) & 1) { D |= 3 << (2 * zpos[i]); smask |= 1 << zout[i]; }
     s_czD[threadIdx.x] = D;
     s_czS[threadIdx.x] = smask;
   }
@@ -1483,51 +1544,43 @@ __device__ __forceinline__ void hub_variant_rows(const FragDev& F, int v, int* s
 // for every P_out with beta(P_out) = the variant's bases, written to the
 // transposed store Q^T.  Dense counts are written only when kept for
 // inspection.
+// WIDE: 32-bit counters, where they overflow 16 bits (shots > 65535) and for
+// histograms of at most 2^kWideMeas outcomes, where the halved address and
+// increment arithmetic is worth more than the shared memory.
+constexpr int kWideMeas = 11;
+template <bool WIDE>
 __global__ void __launch_bounds__(512) sample_hub_kernel(DevPlan P, DevRes R, EvalParams E, const int2* items,
-                                                         int keep_counts, int wide, int hist_words) {
+                                                         int keep_counts, int hist_words) {
   extern __shared__ __align__(16) uint32_t hist2[];
   __shared__ uint32_t tbl[3][256];
-  __shared__ FragDev sF;
   __shared__ int s_czD[16], s_czS[16], s_nzm[2], s_ident;
   const int2 it = items[blockIdx.x];
-  {
-    const int* src = reinterpret_cast<const int*>(P.frags + it.x);
-    int* dst = reinterpret_cast<int*>(&sF);
-    for (int i = threadIdx.x; i < (int)(sizeof(FragDev) / 4); i += blockDim.x) dst[i] = src[i];
+  {   // zero the histogram (the plan's widest, so that nothing waits for the variant's record), 16 bytes per store
+    uint4* h4 = reinterpret_cast<uint4*>(hist2);
+    for (int i = threadIdx.x; i < hist_words / 4; i += blockDim.x) h4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 4 * (hist_words / 4) + threadIdx.x; i < hist_words; i += blockDim.x) hist2[i] = 0u;
   }
-  __syncthreads();
-  const FragDev& F = sF;
+  const FragDev& F = P.frags[it.x];
   const int v = it.y, nA = F.nA;
   const SpaceRec& sp = R.spaces[F.space_off + v];
   const int rank = sp.rank;
   const uint32_t off = sp.off;
-  if (threadIdx.x == 32) s_ident = space_is_identity(sp, rank, nA) ? 1 : 0;
+  if ((threadIdx.x >> 5) == 1) {
+    const bool id = space_is_identity(sp, rank, nA);
+    if (threadIdx.x == 32) s_ident = id ? 1 : 0;
+  }
   if (F.qout <= 4) hub_variant_rows(F, v, s_czD, s_czS, s_nzm);   // warp 0: at most 16 rows
   __syncthreads();
-  if (!s_ident) build_tables(tbl, sp, rank);   // a full-rank space needs no lookup tables
-  const int nwords = wide ? (1 << nA) : ((1 << nA) > 1 ? (1 << (nA - 1)) : 1);
-  {   // zero the histogram, 16 bytes per store
-    uint4* h4 = reinterpret_cast<uint4*>(hist2);
-    for (int i = threadIdx.x; i < nwords / 4; i += blockDim.x) h4[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = 4 * (nwords / 4) + threadIdx.x; i < nwords; i += blockDim.x) hist2[i] = 0u;
-  }
-  __syncthreads();
   const bool ident = s_ident != 0;
-  const uint32_t cmask = rank >= 32 ? 0xffffffffu : ((1u << rank) - 1u);
-  {
-    const uint4 ctr = make_uint4(0u, (uint32_t)v, (uint32_t)F.findex, (uint32_t)F.problem);
-    by_rank(rank, [&](auto lk) {
-      constexpr int L = decltype(lk)::value;
-      for_shots<L>(0u, E.shots, ctr, E.keys, cmask, [&](uint32_t c) {
-        const uint32_t y = ident ? c : space_point<L>(tbl, off, c);   // full rank: the coefficient bits
-        if (wide) atomicAdd(&hist2[y], 1u);
-        else atomicAdd(&hist2[y >> 1], 1u << ((y & 1u) << 4));
-      });
-    });
+  if (!ident) {                          // a full-rank space needs no lookup tables
+    build_tables(tbl, sp, rank);
+    __syncthreads();
   }
+  count_shots<WIDE ? 32 : 16>(hist2, ident, rank, tbl, off, E.shots,
+                              make_uint4(0u, (uint32_t)v, (uint32_t)F.findex, (uint32_t)F.problem), E.keys);
   __syncthreads();
   auto count = [&](uint32_t y) -> uint32_t {
-    return wide ? hist2[y] : (hist2[y >> 1] >> ((y & 1u) << 4)) & 0xffffu;
+    return WIDE ? hist2[y] : (hist2[y >> 1] >> ((y & 1u) << 4)) & 0xffffu;
   };
   if (keep_counts) {
     uint32_t* g = R.counts + F.counts_off + ((long long)v << nA);
@@ -1536,10 +1589,10 @@ __global__ void __launch_bounds__(512) sample_hub_kernel(DevPlan P, DevRes R, Ev
   // Q is stored transposed, Q^T[D][o] (o fastest), so each D of the variant
   // is one coalesced row of 2^m floats.
   const int m = F.m, M = 1 << m, nb = 1 << F.qout;
-  const float inv = (float)E.inv_shots;
+  const float inv = R.hub_scale;
   float* QT = R.TQ + F.T_off;
   int16_t* QH = R.hub_i16 ? reinterpret_cast<int16_t*>(R.TQ + F.T_off) : nullptr;
-  if (!wide && m >= 1 && F.qout <= 4 && E.shots <= (1u << 26)) {
+  if ((!WIDE || E.shots <= 32767u) && m >= 1 && F.qout <= 4 && E.shots <= (1u << 26)) {
     // Pairs of outputs (o, o+1) share the packed counter words.  Per pair,
     // a 16-point Walsh-Hadamard transform over the output bits gives the
     // signed sum for every sign mask at once; each thread parks it in its
@@ -1553,11 +1606,11 @@ __global__ void __launch_bounds__(512) sample_hub_kernel(DevPlan P, DevRes R, Ev
       // fits a signed 16-bit lane: the counter word (outputs o, o+1) is
       // transformed as is, two outputs per SIMD add
       switch (F.qout) {
-        case 0: hub16_readout<0>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
-        case 1: hub16_readout<1>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
-        case 2: hub16_readout<2>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
-        case 3: hub16_readout<3>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
-        default: hub16_readout<4>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
+        case 0: hub16_readout<0, WIDE>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
+        case 1: hub16_readout<1, WIDE>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
+        case 2: hub16_readout<2, WIDE>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
+        case 3: hub16_readout<3, WIDE>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
+        default: hub16_readout<4, WIDE>(hist2, m, M, s_czD, s_czS, nz, QT, QH, inv); break;
       }
     } else
     for (int o2 = threadIdx.x; o2 < (M >> 1); o2 += blockDim.x) {
@@ -1645,18 +1698,20 @@ __global__ void __launch_bounds__(512) sample_hub_kernel(DevPlan P, DevRes R, Ev
 }
 
 // Readout of a byte-counter histogram into the variant's operand rows,
-// specialised on ZM, the quantum outputs measured in the Z basis.  Row cz
-// of the variant needs S(o, cz) = sum_b (-1)^(b . smask_cz) count(o, b) with
-// smask_cz = the X/Y-basis outputs (whose outcome always flips the sign)
+// specialised on Q, the quantum outputs, and ZM, those measured in the Z basis.
+// Row cz of the variant needs S(o, cz) = sum_b (-1)^(b . smask_cz) count(o, b)
+// with smask_cz = the X/Y-basis outputs (whose outcome always flips the sign)
 // plus the Z outputs selected by cz.  So the bins are first summed over the
 // X/Y bits with their fixed signs (F over the Z bits), then a Walsh-Hadamard
-// transform over the Z bits gives every row at once: 16 - 2^nz + nz 2^nz
-// adds instead of a full 16-point transform.  Four outputs o..o+3 share a
-// counter word; each half is processed as two 16-bit lanes of one 32-bit
-// integer (signed lane sums stay below 2^15 in magnitude, so plain integer
-// adds keep the lanes separable).  Returns the thread's sum of all counter
-// bytes read (the caller compares the block's total with the shots: a byte
-// that wrapped makes it smaller).
+// transform over the Z bits gives every row at once: 2^Q - 2^nz + nz 2^nz
+// adds instead of a full transform.  Four outputs o..o+3 share a counter word
+// and all the adds work on whole words: where no byte exceeds 15 and no
+// output's bins sum beyond 127 (both checked), every partial sum fits a signed
+// byte lane, and one bias at the end separates the lanes.  Other words are
+// split into 16-bit lanes first (sums of 16 bytes stay below 2^15).  V words
+// (4 V outputs) per thread and pass: one store of 8 V bytes per row.  Returns
+// the thread's sum of all counter bytes read (the caller compares the block's
+// total with the shots: a byte that wrapped makes it smaller).
 __host__ __device__ constexpr int popc4(int x) { return (x & 1) + ((x >> 1) & 1) + ((x >> 2) & 1) + ((x >> 3) & 1); }
 __host__ __device__ constexpr int pext4(int b, int zm) {
   int r = 0, k = 0;
@@ -1665,58 +1720,121 @@ __host__ __device__ constexpr int pext4(int b, int zm) {
   return r;
 }
 
-template <int ZM>
-__device__ __forceinline__ unsigned hub8_readout(const uint32_t* __restrict__ h32, int m, int M, int nb,
-                                                 const int* s_czD, float* __restrict__ QT, int16_t* __restrict__ QH,
-                                                 float inv) {
+// F[i] over the Z bits from the words x[b] (2^Q of them), then the transform.
+template <int ZM, int Q>
+__device__ __forceinline__ void hub8_rows(const uint32_t (&x)[1 << Q], uint32_t (&F)[1 << popc4(ZM)]) {
   constexpr int NR = 1 << popc4(ZM);
-  unsigned tot = 0;
-  for (int q = threadIdx.x; q < (M >> 2); q += blockDim.x) {
-    const int o = 4 * q;
-    uint32_t w[16];
 #pragma unroll
-    for (int b = 0; b < 16; ++b) w[b] = b < nb ? h32[((uint32_t)o | ((uint32_t)b << m)) >> 2] : 0u;
+  for (int i = 0; i < NR; ++i) F[i] = 0u;
 #pragma unroll
-    for (int b = 0; b < 16; ++b) tot = __dp4a(w[b], 0x01010101u, tot);
-    uint32_t W[NR][2];     // per row: outputs (o, o+1) and (o+2, o+3) as int16 pairs
+  for (int b = 0; b < (1 << Q); ++b) {
+    if (popc4(b & ~ZM & 15) & 1) F[pext4(b, ZM)] -= x[b];
+    else F[pext4(b, ZM)] += x[b];
+  }
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      int F[NR];
+  for (int h = 1; h < NR; h <<= 1)
 #pragma unroll
-      for (int i = 0; i < NR; ++i) F[i] = 0;
-#pragma unroll
-      for (int b = 0; b < 16; ++b) {     // outputs o + 2 half, o + 2 half + 1 as 16-bit lanes
-        const int x = (int)__byte_perm(w[b], 0u, half ? 0x4342 : 0x4140);
-        if (popc4(b & ~ZM & 15) & 1) F[pext4(b, ZM)] -= x;
-        else F[pext4(b, ZM)] += x;
+    for (int i = 0; i < NR; ++i)
+      if (!(i & h)) {
+        const uint32_t a = F[i], c = F[i | h];
+        F[i] = a + c;
+        F[i | h] = a - c;
       }
+}
+
+// Two bytes of x sign-extended to 16 bits (prmt's sign-replicating selectors,
+// which __byte_perm masks off).
+template <unsigned SEL>
+__device__ __forceinline__ uint32_t sext_bytes(uint32_t x) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "n"(SEL));
+  return r;
+}
+
+template <int ZM, int Q, int V>
+__device__ __forceinline__ unsigned hub8_readout(const uint32_t* __restrict__ h32, int m, int M, const int* s_czD,
+                                                 float* __restrict__ QT, int16_t* __restrict__ QH, float inv) {
+  constexpr int NR = 1 << popc4(ZM), NB = 1 << Q;
+  unsigned tot = 0;
+  for (int q = threadIdx.x; q < M / (4 * V); q += blockDim.x) {
+    const int o = 4 * V * q;
+    uint32_t w[V][NB];
 #pragma unroll
-      for (int h = 1; h < NR; h <<= 1)
+    for (int b = 0; b < NB; ++b) {
+      const uint32_t* src = h32 + (((uint32_t)o | ((uint32_t)b << m)) >> 2);
+      if (V == 2) {
+        const uint2 t = *reinterpret_cast<const uint2*>(src);
+        w[0][b] = t.x;
+        w[V - 1][b] = t.y;
+      } else {
+        w[0][b] = *src;
+      }
+    }
+    uint32_t W[NR][2 * V];     // per row: pairs of outputs as int16
 #pragma unroll
-        for (int i = 0; i < NR; ++i)
-          if (!(i & h)) {
-            const int a = F[i], c = F[i | h];
-            F[i] = a + c;
-            F[i | h] = a - c;
-          }
-      // F = lo + 2^16 hi with |lo|, |hi| <= 16 x 255: the int16 pair word is
-      // F plus the borrow its low lane took from the high one
+    for (int u = 0; u < V; ++u) {
+      uint32_t any = 0u, sum = 0u, F[NR];
 #pragma unroll
-      for (int i = 0; i < NR; ++i) W[i][half] = (uint32_t)F[i] + (((uint32_t)F[i] & 0x8000u) << 1);
+      for (int b = 0; b < NB; ++b) { any |= w[u][b]; sum += w[u][b]; }
+      if (((any & 0xf0f0f0f0u) | (sum & 0x80808080u)) == 0u) {
+        tot = __dp4a(sum, 0x01010101u, tot);
+        hub8_rows<ZM, Q>(w[u], F);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          const uint32_t x = (F[i] + 0x80808080u) ^ 0x80808080u;      // four signed bytes
+          W[i][2 * u] = sext_bytes<0x9180>(x);                        // as int16 pairs
+          W[i][2 * u + 1] = sext_bytes<0xb3a2>(x);
+        }
+      } else {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) tot = __dp4a(w[u][b], 0x01010101u, tot);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {     // two outputs as 16-bit lanes
+          uint32_t x[NB];
+#pragma unroll
+          for (int b = 0; b < NB; ++b) x[b] = __byte_perm(w[u][b], 0u, half ? 0x4342 : 0x4140);
+          hub8_rows<ZM, Q>(x, F);
+          // F = lo + 2^16 hi with |lo|, |hi| <= 16 x 255: the int16 pair word is
+          // F plus the borrow its low lane took from the high one
+#pragma unroll
+          for (int i = 0; i < NR; ++i) W[i][2 * u + half] = F[i] + ((F[i] & 0x8000u) << 1);
+        }
+      }
     }
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
       const long long idx = (long long)s_czD[i] * M + o;
-      if (QH) {
+      if (QH && V == 2) {
+        *reinterpret_cast<uint4*>(QH + idx) = make_uint4(W[i][0], W[i][1], W[i][2 * V - 2], W[i][2 * V - 1]);
+      } else if (QH) {
         *reinterpret_cast<uint2*>(QH + idx) = make_uint2(W[i][0], W[i][1]);
       } else {
-        const int v[4] = {(int)(short)(W[i][0] & 0xffffu), (int)(short)(W[i][0] >> 16),
-                          (int)(short)(W[i][1] & 0xffffu), (int)(short)(W[i][1] >> 16)};
-        put4(QT, nullptr, idx, v, inv);
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+          const int v[4] = {(int)(short)(W[i][2 * u] & 0xffffu), (int)(short)(W[i][2 * u] >> 16),
+                            (int)(short)(W[i][2 * u + 1] & 0xffffu), (int)(short)(W[i][2 * u + 1] >> 16)};
+          put4(QT, nullptr, idx + 4 * u, v, inv);
+        }
       }
     }
   }
   return tot;
+}
+// The Z-basis pattern as a compile-time constant.
+template <int Q, int V>
+__device__ __forceinline__ unsigned hub8_readout_any(int zm, const uint32_t* __restrict__ h32, int m, int M,
+                                                     const int* s_czD, float* __restrict__ QT, int16_t* __restrict__ QH,
+                                                     float inv) {
+  switch (zm & ((1 << Q) - 1)) {
+#define CCS_HUB8_CASE(z) \
+  case z: return hub8_readout<(z) & ((1 << Q) - 1), Q, V>(h32, m, M, s_czD, QT, QH, inv);
+    CCS_HUB8_CASE(0) CCS_HUB8_CASE(1) CCS_HUB8_CASE(2) CCS_HUB8_CASE(3)
+    CCS_HUB8_CASE(4) CCS_HUB8_CASE(5) CCS_HUB8_CASE(6) CCS_HUB8_CASE(7)
+    CCS_HUB8_CASE(8) CCS_HUB8_CASE(9) CCS_HUB8_CASE(10) CCS_HUB8_CASE(11)
+    CCS_HUB8_CASE(12) CCS_HUB8_CASE(13) CCS_HUB8_CASE(14) CCS_HUB8_CASE(15)
+#undef CCS_HUB8_CASE
+    default: return 0u;
+  }
 }
 
 // --- the hub sampler with byte counters (three CTAs per SM) ---------------
@@ -1735,32 +1853,36 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 2 : 3) sample_hub8_kernel(DevP
                                                                           int hist_words) {
   extern __shared__ __align__(16) uint32_t h32[];
   __shared__ uint32_t tbl[3][256];
-  __shared__ FragDev sF;
   __shared__ int s_czD[16], s_czS[16], s_nzm[2];
   __shared__ unsigned s_tot;
   __shared__ int s_ident;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int2 it = items[blockIdx.x];
-  {
-    const int* src = reinterpret_cast<const int*>(P.frags + it.x);
-    int* dst = reinterpret_cast<int*>(&sF);
-    for (int i = tid; i < (int)(sizeof(FragDev) / 4); i += nt) dst[i] = src[i];
+  {   // zero the histogram (the plan's widest, so that nothing waits for the variant's record), 16 bytes per store
+    uint4* h4 = reinterpret_cast<uint4*>(h32);
+    for (int i = tid; i < hist_words / 4; i += nt) h4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 4 * (hist_words / 4) + tid; i < hist_words; i += nt) h32[i] = 0u;
   }
   if (tid == 0) s_tot = 0u;
-  __syncthreads();
-  const FragDev& F = sF;
+  const FragDev& F = P.frags[it.x];
   const int v = it.y, nA = F.nA, m = F.m, M = 1 << m, nb = 1 << F.qout;
   const SpaceRec& sp = R.spaces[F.space_off + v];
   const int rank = sp.rank;
   const uint32_t off = sp.off;
-  if (tid == 32) s_ident = space_is_identity(sp, rank, nA) ? 1 : 0;
+  if ((tid >> 5) == 1) {
+    const bool id = space_is_identity(sp, rank, nA);
+    if (tid == 32) s_ident = id ? 1 : 0;
+  }
   // the variant's operand rows: one D and sign mask per Z-basis choice
   hub_variant_rows(F, v, s_czD, s_czS, s_nzm);
   __syncthreads();
   const bool ident = s_ident != 0;
-  if (!ident) build_tables(tbl, sp, rank);   // a full-rank space needs no lookup tables
-  const uint32_t cmask = rank >= 32 ? 0xffffffffu : ((1u << rank) - 1u);
-  const float inv = (float)E.inv_shots;
+  if (!ident) {                              // a full-rank space needs no lookup tables
+    build_tables(tbl, sp, rank);
+    __syncthreads();
+  }
+  const uint32_t cmask = (1u << rank) - 1u;
+  const float inv = R.hub_scale;
   float* QT = R.TQ + F.T_off;
   int16_t* QH = R.hub_i16 ? reinterpret_cast<int16_t*>(R.TQ + F.T_off) : nullptr;
   const int wstride = E.shots <= 32767u ? 0 : 33;    // only the unpacked transform parks values
@@ -1768,37 +1890,29 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 2 : 3) sample_hub8_kernel(DevP
   uint32_t* gcount = R.counts + F.counts_off + ((long long)v << nA);
   bool narrow = (unsigned long long)E.shots <= (64ull << rank);
   if (narrow) {
-    {   // zero the histogram, 16 bytes per store
-      uint4* h4 = reinterpret_cast<uint4*>(h32);
-      for (int i = tid; i < (1 << nA) / 16; i += nt) h4[i] = make_uint4(0u, 0u, 0u, 0u);
-      for (int i = 4 * ((1 << nA) / 16) + tid; i < (1 << nA) / 4; i += nt) h32[i] = 0u;
-    }
-    __syncthreads();
-    const uint4 ctr = make_uint4(0u, (uint32_t)v, (uint32_t)F.findex, (uint32_t)F.problem);
-    by_rank(rank, [&](auto lk) {
-      constexpr int L = decltype(lk)::value;
-      if (ident)        // full rank: the outcome is the coefficient bits (no table lookup)
-        for_shots<L>(0u, E.shots, ctr, E.keys, cmask,
-                     [&](uint32_t c) { atomicAdd(&h32[c >> 2], 1u << ((c & 3u) << 3)); });
-      else
-        for_shots<L>(0u, E.shots, ctr, E.keys, cmask, [&](uint32_t c) {
-          const uint32_t y = space_point<L>(tbl, off, c);
-          atomicAdd(&h32[y >> 2], 1u << ((y & 3u) << 3));
-        });
-    });
+    count_shots<8>(h32, ident, rank, tbl, off, E.shots,
+                   make_uint4(0u, (uint32_t)v, (uint32_t)F.findex, (uint32_t)F.problem), E.keys);
     __syncthreads();
     if (keep_counts)
       for (uint32_t y = tid; y < (1u << nA); y += nt) gcount[y] = (h32[y >> 2] >> ((y & 3u) << 3)) & 0xffu;
     unsigned tot = 0;
-    switch (s_nzm[1]) {
-#define CCS_HUB8_CASE(z) \
-  case z: tot = hub8_readout<z>(h32, m, M, nb, s_czD, QT, QH, inv); break;
-      CCS_HUB8_CASE(0) CCS_HUB8_CASE(1) CCS_HUB8_CASE(2) CCS_HUB8_CASE(3)
-      CCS_HUB8_CASE(4) CCS_HUB8_CASE(5) CCS_HUB8_CASE(6) CCS_HUB8_CASE(7)
-      CCS_HUB8_CASE(8) CCS_HUB8_CASE(9) CCS_HUB8_CASE(10) CCS_HUB8_CASE(11)
-      CCS_HUB8_CASE(12) CCS_HUB8_CASE(13) CCS_HUB8_CASE(14) CCS_HUB8_CASE(15)
-#undef CCS_HUB8_CASE
-      default: break;
+    const int zm = s_nzm[1];
+    if (M >= 8) {
+      switch (F.qout) {
+        case 0: tot = hub8_readout_any<0, 2>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        case 1: tot = hub8_readout_any<1, 2>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        case 2: tot = hub8_readout_any<2, 2>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        case 3: tot = hub8_readout_any<3, 2>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        default: tot = hub8_readout_any<4, 2>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+      }
+    } else {
+      switch (F.qout) {
+        case 0: tot = hub8_readout_any<0, 1>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        case 1: tot = hub8_readout_any<1, 1>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        case 2: tot = hub8_readout_any<2, 1>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        case 3: tot = hub8_readout_any<3, 1>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+        default: tot = hub8_readout_any<4, 1>(zm, h32, m, M, s_czD, QT, QH, inv); break;
+      }
     }
     tot = __reduce_add_sync(0xffffffffu, tot);
     if ((tid & 31) == 0) atomicAdd(&s_tot, tot);
@@ -1945,14 +2059,15 @@ cudaError_t launch_sample_hub(const DevPlan& p, const DevRes& r, const EvalParam
     kern<<<n_items, t8, smem, s>>>(p, r, e, items, keep_counts, hist_words); note_launch();
     return cudaGetLastError();
   }
-  const int wide = e.shots > 0xffffu ? 1 : 0;     // 32-bit counters when 16 bits could overflow
+  const bool wide = e.shots > 0xffffu || max_nA <= kWideMeas;
   const int hist_words = wide ? (1 << max_nA) : ((1 << max_nA) > 1 ? (1 << (max_nA - 1)) : 1);
   // packed counters, then 33 ints per thread for the transform of the 16-bit path
   threads = threads >= 512 ? 512 : threads >= 256 ? 256 : 128;
   const size_t smem = (size_t)4 * hist_words + (wide ? 0 : (size_t)threads * (e.shots <= 32767u ? 0 : 33) * 4);
-  cudaError_t err = cudaFuncSetAttribute(sample_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = wide ? sample_hub_kernel<true> : sample_hub_kernel<false>;
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  sample_hub_kernel<<<n_items, threads, smem, s>>>(p, r, e, items, keep_counts, wide, hist_words); note_launch();
+  kern<<<n_items, threads, smem, s>>>(p, r, e, items, keep_counts, hist_words); note_launch();
   return cudaGetLastError();
 }
 
