@@ -380,13 +380,20 @@ def _ncu_traffic(kernel, workload):
 E2E_WORKERS = 8     # host threads serving end-to-end steps, one step at a time each
 
 
+def hub_counters(hub_threads):
+    """Counter width of the hub sampler from ccs_get_tuning's CTA size (16-bit
+    stands for the 32-bit counters of narrow hubs too)."""
+    return "16-bit" if hub_threads > 0 else "4-bit" if hub_threads == -128 else "8-bit"
+
+
 def stage_kernel(st, precision, tuning=None, ws=None, prob_infos=None):
     """The kernel that stands for a stage (its longest launch): the hub
     sampler the autotuner picked (byte or 16-bit counters); the contraction
     of wide hub operands (the first-leaf streaming GEMM, or tcgen05 in BF16)
     or of small stars (leaf by leaf); the body kernel for the Clifford stage."""
     if st == "sample":
-        return "sample_hub_kernel" if (tuning or {}).get("hub_counters") == "16-bit" else "sample_hub8_kernel"
+        return {"16-bit": "sample_hub_kernel", "4-bit": "sample_hub4_kernel"}.get(
+            (tuning or {}).get("hub_counters"), "sample_hub8_kernel")
     if st == "recombine":
         wide = False
         for x, infos in zip(ws or [], prob_infos or []):
@@ -641,7 +648,7 @@ def run_ours(args, rank, world, local_rank):
     d2h = 8 * sum((1 << len(x.marginal)) + len(x.zstrings) for x in ws)
 
     pk, pk_kind = peaks()
-    tune_info = {"hub_counters": "8-bit" if tuning[3] < 0 else "16-bit", "variant_path": bool(tuning[4])}
+    tune_info = {"hub_counters": hub_counters(tuning[3]), "variant_path": bool(tuning[4])}
     roofs = stage_rooflines(stage, ws, prob_infos, pk, pk_kind, args.precision, args.workload, tune_info)
     roof = dict(roofs[dom], stage=dom, kernel=stage_kernel(dom, args.precision, tune_info, ws, prob_infos))
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -659,7 +666,7 @@ def run_ours(args, rank, world, local_rank):
                                                           " (CUDA-core FMA, FP64 across splits)"),
                        "tuning": {"threads": tuning[0], "words_per_op": tuning[1], "shots_per_cta": tuning[2],
                                   "hub_threads": abs(tuning[3]),
-                                  "hub_counters": "8-bit" if tuning[3] < 0 else "16-bit",
+                                  "hub_counters": hub_counters(tuning[3]),
                                   "path": "per-variant simulation" if tuning[4] else "shared bodies + screen",
                                   "autotuned": tune}},
             "circuits_per_s": world * len(ws) * args.steps / t_tot,

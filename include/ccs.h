@@ -214,8 +214,9 @@ typedef struct {
   int32_t per_variant_body; /* 1: simulate each variant's whole gate sequence; 0 (default):
                               evolve each Clifford fragment's shared body once and derive
                               every variant from it (same tableaus bit for bit) */
-  int32_t hub_sampler;     /* star hubs' sampler: 0 automatic (or autotuned), 1 16-bit
-                              counters, 2 byte counters with an exact 16-bit recount where
+  int32_t hub_sampler;     /* star hubs' sampler: 0 automatic (or autotuned; 4-bit counters
+                              for sparse histograms), 1 16-bit counters (32-bit for hubs
+                              of at most 11 measured bits), 2 byte counters with an exact 16-bit recount where
                               a byte could overflow, 256 threads per CTA, 3 the same with 512
                               (2 and 3 used only if every hub has >= 2 marginal bits, <= 4
                               quantum outputs, |A| <= 16); same counts */
@@ -241,7 +242,7 @@ void ccs_res_free(ccs_res res);
 /* Launch shape in use for a result (after autotuning, if any): threads per
  * tableau CTA, 64-row words of one fused op per thread, shots per sampling
  * CTA, threads per fused hub-sampler CTA (negative: the byte-counter
- * sampler with that many threads), and the evaluation path (1: every
+ * sampler with that many threads, or at -128 the 4-bit-counter one), and the evaluation path (1: every
  * Clifford variant simulates its whole circuit, which the autotuner picks
  * for small plans when it is faster, or which per_variant_body asks for;
  * 0: shared bodies and the outcome-space screen).  Both paths give the same

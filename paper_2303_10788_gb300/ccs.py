@@ -463,7 +463,7 @@ def ccs_ml_correct(ctx, plan, res, which=CCS_ML_SAMPLED):
 
 def ccs_get_tuning(ctx, res):
     """(threads per tableau CTA, words per op per thread, shots per sampling CTA,
-    threads per hub-sampler CTA (negative: byte counters), 1 if every variant
+    threads per hub-sampler CTA (negative: byte counters, -128: 4-bit ones), 1 if every variant
     simulates its whole circuit else 0)."""
     t, wpo, spc, hub, vp = C.c_int(), C.c_int(), C.c_int(), C.c_int(), C.c_int()
     ctx.check(lib().ccs_get_tuning(ctx.h, res.h, C.byref(t), C.byref(wpo), C.byref(spc), C.byref(hub),

@@ -388,6 +388,7 @@ struct ccs_plan_s {
   int2* d_items_plain = nullptr;    // other Clifford variants (sampler -> counts)
   int n_items_hub = 0, n_items_plain = 0, max_hub_nA = 0;
   bool hub_bytes_ok = true;         // every hub fits the byte-counter sampler
+  int min_hub_nA = 99, min_hub_m = 99;   // narrowest hub's measured bits, marginal bits
   long long n_counts_plain = 0;     // counts of non-hub Clifford fragments come first
   long long n_dist_nc = 0;          // distributions of statevector fragments come first
   long long n_dist_stitch = 0;      // ... then non-hub Clifford fragments (all a stitched evaluation needs)
@@ -424,7 +425,9 @@ struct ccs_res_s {
   int cliff_words = 1;        // words per op per thread in the tableau kernel
   int sample_spc = 4096;
   int hub_threads = 512;      // threads of the fused hub sampler CTA (either counter width)
-  bool hub_bytes = false;     // use the byte-counter hub sampler (64 KB of counters at |A| = 16)
+  bool hub_bytes = false;     // use the byte-counter hub sampler (64 KB of counters at |A| = 16; at 128
+                              // threads the 4-bit-counter one, while it applies)
+  int2* nibble_list = nullptr;   // variants the 4-bit counters leave to the byte counters
   bool variant_path = false;  // autotuned: every variant simulates its whole circuit (small plans)
   float* scratch = nullptr;   // recombination: R operand + split-K partials
   uint16_t* rt_scratch = nullptr;   // bf16 R'^T of tensor-core-eligible problems
@@ -1025,6 +1028,8 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       if (f.role == 1) {
         items_hub.push_back(it);
         plan->max_hub_nA = std::max(plan->max_hub_nA, f.nA);
+        plan->min_hub_nA = std::min(plan->min_hub_nA, f.nA);
+        plan->min_hub_m = std::min(plan->min_hub_m, f.m);
         if (f.m < 2 || f.qout > 4 || f.nA > 16) plan->hub_bytes_ok = false;
       }
       else items_plain.push_back(it);
@@ -1337,6 +1342,14 @@ int ccs_cut_candidates(ccs_ctx c, const ccs_problem* q, const ccs_cut_opts* opts
 // fold) on the side stream, forked after the memsets and joined at the end.
 // With profiling on, everything runs on the context stream so each stage's
 // events bracket one kernel.
+// The 4-bit-counter hub sampler pays for sparse histograms: every hub has at
+// most four shots per outcome (at full rank), eight outputs per counter word,
+// and int16 operand rows.
+static bool nibble_ok(ccs_plan p, unsigned shots) {
+  return p->hub_bytes_ok && p->n_items_hub > 0 && p->min_hub_m >= 3 && shots <= 32767u &&
+         (unsigned long long)shots <= (4ull << p->min_hub_nA);
+}
+
 static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
   cudaStream_t s = c->stream;
   const EvalParams& e = r->ep;
@@ -1391,7 +1404,7 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
       stage_begin(c, ST_SAMPLE);
       if ((err = launch_sample_hub(dp, r->dr, e, p->d_items_hub, p->n_items_hub, p->max_hub_nA, r->hub_threads,
                                    e.keep_tableaus, p->hub_bytes_ok && r->hub_bytes,
-                                   s)) != cudaSuccess)
+                                   nibble_ok(p, e.shots) ? r->nibble_list : nullptr, c->sm_count, s)) != cudaSuccess)
         return cuda_fail(c, err, "hub sample kernel");
       if ((err = launch_sample(dp, r->dr, e, p->d_items_plain, p->n_items_plain, r->sample_spc, 256, s)) !=
           cudaSuccess)
@@ -1466,7 +1479,7 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
   const int threads_c[] = {128, 256, 512};
   const int words_c[] = {1, 2, 4, 8};
   const int spc_c[] = {1024, 2048, 4096, 8192};
-  const int hub_c[] = {128, 512, 256, 512};  // 16-bit counters, then byte counters
+  const int hub_c[] = {128, 512, 256, 512, 128};  // 16-bit counters, byte counters, 4-bit counters
   const int max_w = 2 * ((max_n + 63) / 64);
   const bool sampled = r->ep.mode == CCS_SAMPLED;
   int rc = CCS_OK;
@@ -1490,9 +1503,10 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
   }
   r->sample_spc = bs;
   bool bb = r->hub_bytes;
-  for (int hi = 0; sampled && p->n_items_hub && hi < 4 && rc == CCS_OK; ++hi) {
+  for (int hi = 0; sampled && p->n_items_hub && hi < 5 && rc == CCS_OK; ++hi) {
     const bool bytes = hi >= 2;
     if (bytes && !p->hub_bytes_ok) continue;
+    if (hi == 4 && !nibble_ok(p, r->ep.shots)) continue;
     r->hub_bytes = bytes;
     r->hub_threads = hub_c[hi];
     if ((rc = time_it(&ms)) == CCS_OK && ms < best) { best = ms; bh = hub_c[hi]; bb = bytes; }
@@ -1604,7 +1618,9 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
         // small hub CTAs when a variant has few shots and few outputs (more CTAs per SM);
         // byte counters when the histogram would otherwise fill an SM's shared memory
         r->hub_bytes = p->hub_bytes_ok && p->max_hub_nA >= 13;
-        r->hub_threads = r->hub_bytes ? 256 : (p->max_hub_nA <= 12 && opts->shots <= 4096) ? 128 : 512;
+        r->hub_threads = r->hub_bytes && nibble_ok(p, opts->shots) ? 128
+                         : r->hub_bytes                            ? 256
+                         : (p->max_hub_nA <= 12 && opts->shots <= 4096) ? 128 : 512;
       }
       if (p->rt_total) {
         d.TQh = r->A.get<uint16_t>(p->n_T);
@@ -1640,6 +1656,11 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
         r->dist_len = need;
         drop_graph();
       }
+    }
+    if (opts->mode == CCS_SAMPLED && nibble_ok(p, opts->shots) && !r->nibble_list) {
+      r->nibble_list = r->A.get<int2>(p->n_items_hub);
+      if (!r->nibble_list) return fail(c, CCS_ERR_OOM, "sampler list allocation failed");
+      drop_graph();
     }
     if (opts->keep_tableaus && !r->have_tabs && p->n_tab) {
       r->dr.tabs = r->A.get<unsigned long long>(p->n_tab);

@@ -1177,6 +1177,7 @@ __global__ void __launch_bounds__(512) clifford_kernel(DevPlan P, DevRes R, Eval
 // groups that exist (entry 0 of the others is 0, which is all a shot of
 // rank-limited coefficients can select there).  The basis is read once into
 // shared memory; every thread of the block must call this (it synchronises).
+template <int NTAB = 3>
 __device__ __forceinline__ void build_tables(uint32_t (*tbl)[256], const SpaceRec& sp, int rank) {
   __shared__ uint32_t s_b[kMaxMeas];
   const int ntab = rank > 16 ? 3 : rank > 8 ? 2 : 1;
@@ -1190,7 +1191,7 @@ __device__ __forceinline__ void build_tables(uint32_t (*tbl)[256], const SpaceRe
       if ((byte >> b) & 1) acc ^= s_b[8 * k + b];
     tbl[k][byte] = acc;
   }
-  if ((int)threadIdx.x < 3 - ntab) tbl[ntab + threadIdx.x][0] = 0u;
+  if ((int)threadIdx.x < NTAB - ntab) tbl[ntab + threadIdx.x][0] = 0u;
 }
 
 // --- K3: Philox4x32-10 counter-based sampling from the affine space -------
@@ -1260,7 +1261,7 @@ __device__ __forceinline__ bool space_is_identity(const SpaceRec& sp, int rank, 
 }
 
 // All shots of a hub variant whose outcome is its coefficient bits, counted
-// in shared memory: byte, 16-bit or 32-bit counters.  The field's place in
+// in shared memory: 4-, 8-, 16- or 32-bit counters.  The field's place in
 // its word, its word's byte address and its increment come from one shift, one
 // mask and one wrapping shift each, with no masked copy of the field.
 template <int CB>
@@ -1270,15 +1271,18 @@ __device__ __forceinline__ void count_field(uint32_t* hist, uint32_t w, int sh, 
     atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(hist) + at), 1u);
   } else {
     const uint32_t f = w >> sh;
-    const uint32_t at = CB == 8 ? f & (cmask & ~3u) : (f << 1) & ((cmask << 1) & ~3u);
+    const uint32_t at = CB == 4   ? (f >> 1) & ((cmask >> 1) & ~3u)
+                        : CB == 8 ? f & (cmask & ~3u)
+                                  : (f << 1) & ((cmask << 1) & ~3u);
     atomicAdd(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(hist) + at),
-              __funnelshift_l(0u, 1u, CB == 8 ? f << 3 : f << 4));     // 1 << (shift mod 32)
+              __funnelshift_l(0u, 1u, CB == 4 ? f << 2 : CB == 8 ? f << 3 : f << 4));     // 1 << (shift mod 32)
   }
 }
 template <int CB>
 __device__ __forceinline__ void count_outcome(uint32_t* hist, uint32_t y) {
   if (CB == 32) atomicAdd(hist + y, 1u);
   else if (CB == 16) atomicAdd(hist + (y >> 1), 1u << ((y & 1u) << 4));
+  else if (CB == 4) atomicAdd(hist + (y >> 3), 1u << ((y & 7u) << 2));
   else atomicAdd(hist + (y >> 2), 1u << ((y & 3u) << 3));
 }
 template <int CB, int L>
@@ -1545,8 +1549,10 @@ __device__ __forceinline__ void hub_variant_rows(const FragDev& F, int v, int* s
 // transposed store Q^T.  Dense counts are written only when kept for
 // inspection.
 // WIDE: 32-bit counters, where they overflow 16 bits (shots > 65535) and for
-// histograms of at most 2^kWideMeas outcomes, where the halved address and
-// increment arithmetic is worth more than the shared memory.
+// histograms of at most 2^kWideMeas outcomes (8 KB), where the halved address
+// and increment arithmetic is worth more than the shared memory: with the
+// setup changes above, 64 circuits of 10 measured bits x 4096 shots went from
+// 201 to 148 us (6.29 M to 4.36 M warp instructions per 1728 variants).
 constexpr int kWideMeas = 11;
 template <bool WIDE>
 __global__ void __launch_bounds__(512) sample_hub_kernel(DevPlan P, DevRes R, EvalParams E, const int2* items,
@@ -1751,6 +1757,15 @@ __device__ __forceinline__ uint32_t sext_bytes(uint32_t x) {
   return r;
 }
 
+// Byte i of x and of y sign-extended to an int16 pair (SEL: y's sign, y's byte
+// 4 + i, x's sign, x's byte i).
+template <unsigned SEL>
+__device__ __forceinline__ uint32_t sext_pair(uint32_t x, uint32_t y) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(y), "n"(SEL));
+  return r;
+}
+
 template <int ZM, int Q, int V>
 __device__ __forceinline__ unsigned hub8_readout(const uint32_t* __restrict__ h32, int m, int M, const int* s_czD,
                                                  float* __restrict__ QT, int16_t* __restrict__ QH, float inv) {
@@ -1847,17 +1862,14 @@ __device__ __forceinline__ unsigned hub8_readout_any(int zm, const uint32_t* __r
 // carries at most 1 into the next), is counted again with 16-bit counters
 // in two passes, each over the outputs o of one half (top marginal bit),
 // and its operand rows are rewritten.
-template <int NT>    // 256 threads (three CTAs per SM) or 512 (two): registers for each
-__global__ void __launch_bounds__(NT, NT >= 512 ? 2 : 3) sample_hub8_kernel(DevPlan P, DevRes R, EvalParams E,
-                                                                          const int2* items, int keep_counts,
-                                                                          int hist_words) {
+__device__ __forceinline__ void hub8_variant(const DevPlan& P, const DevRes& R, const EvalParams& E, int2 it,
+                                             int keep_counts, int hist_words) {
   extern __shared__ __align__(16) uint32_t h32[];
   __shared__ uint32_t tbl[3][256];
   __shared__ int s_czD[16], s_czS[16], s_nzm[2];
   __shared__ unsigned s_tot;
   __shared__ int s_ident;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int2 it = items[blockIdx.x];
   {   // zero the histogram (the plan's widest, so that nothing waits for the variant's record), 16 bytes per store
     uint4* h4 = reinterpret_cast<uint4*>(h32);
     for (int i = tid; i < hist_words / 4; i += nt) h4[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -1965,6 +1977,144 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 2 : 3) sample_hub8_kernel(DevP
   }
 }
 
+// LIST: the variants listed in `items[0 .. R.work[2])` by sample_hub4_kernel,
+// taken in turn by the CTAs of one wave; else one variant per CTA.
+template <int NT, bool LIST>    // 256 threads (three CTAs per SM) or 512 (two): registers for each
+__global__ void __launch_bounds__(NT, NT >= 512 ? 2 : 3) sample_hub8_kernel(DevPlan P, DevRes R, EvalParams E,
+                                                                          const int2* items, int keep_counts,
+                                                                          int hist_words) {
+  if (!LIST) {
+    hub8_variant(P, R, E, items[blockIdx.x], keep_counts, hist_words);
+    return;
+  }
+  for (int i = blockIdx.x, n = (int)R.work[2]; i < n; i += gridDim.x) {
+    hub8_variant(P, R, E, items[i], keep_counts, hist_words);
+    __syncthreads();                    // the variant is read out
+  }
+}
+
+// --- the hub sampler with 4-bit counters -----------------------------------
+// For sparse histograms (at most about four shots per outcome): 2^16 counters
+// take 32 KB, so six CTAs share an SM instead of three, and the zeroing, the
+// readout's loads and the CTAs' fixed latencies (records, barriers, the first
+// generator call) overlap more shots.  A word holds eight outputs; its even and
+// odd counters are two words of byte lanes (sums of 16 counters below 16 fit a
+// byte), combined as in hub8_readout.  A variant whose space is too small for
+// its shots, a counter that wrapped (the total is then short) or an output
+// whose bins sum beyond 127 goes on the list that sample_hub8_kernel works off
+// afterwards (items_list, counted in R.work[2]).  20736 variants x 16384 shots,
+// |A| = 16: 303 us against 352 us with byte counters; x 4096 shots, |A| = 13: 120
+// against 198 us (there the fixed latencies of the larger CTAs weigh most).
+template <int ZM, int Q>
+__device__ __forceinline__ unsigned hub4_readout(const uint32_t* __restrict__ h32, int m, int M, const int* s_czD,
+                                                 int16_t* __restrict__ QH, unsigned& over) {
+  constexpr int NR = 1 << popc4(ZM), NB = 1 << Q;
+  unsigned tot = 0;
+  for (int q = threadIdx.x; q < (M >> 3); q += blockDim.x) {
+    const int o = 8 * q;
+    uint32_t ev[NB], od[NB], se = 0u, so = 0u;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) ev[b] = h32[((uint32_t)o | ((uint32_t)b << m)) >> 3];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      od[b] = (ev[b] >> 4) & 0x0f0f0f0fu;
+      ev[b] &= 0x0f0f0f0fu;
+      se += ev[b];
+      so += od[b];
+    }
+    over |= (se | so) & 0x80808080u;
+    tot = __dp4a(so, 0x01010101u, __dp4a(se, 0x01010101u, tot));
+    uint32_t Fe[NR], Fo[NR];
+    hub8_rows<ZM, Q>(ev, Fe);
+    hub8_rows<ZM, Q>(od, Fo);
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const uint32_t x = (Fe[i] + 0x80808080u) ^ 0x80808080u, y = (Fo[i] + 0x80808080u) ^ 0x80808080u;
+      *reinterpret_cast<uint4*>(QH + (long long)s_czD[i] * M + o) =
+          make_uint4(sext_pair<0xc480>(x, y), sext_pair<0xd591>(x, y), sext_pair<0xe6a2>(x, y), sext_pair<0xf7b3>(x, y));
+    }
+  }
+  return tot;
+}
+template <int Q>
+__device__ __forceinline__ unsigned hub4_readout_any(int zm, const uint32_t* __restrict__ h32, int m, int M,
+                                                     const int* s_czD, int16_t* __restrict__ QH, unsigned& over) {
+  switch (zm & ((1 << Q) - 1)) {
+#define CCS_HUB4_CASE(z) \
+  case z: return hub4_readout<(z) & ((1 << Q) - 1), Q>(h32, m, M, s_czD, QH, over);
+    CCS_HUB4_CASE(0) CCS_HUB4_CASE(1) CCS_HUB4_CASE(2) CCS_HUB4_CASE(3)
+    CCS_HUB4_CASE(4) CCS_HUB4_CASE(5) CCS_HUB4_CASE(6) CCS_HUB4_CASE(7)
+    CCS_HUB4_CASE(8) CCS_HUB4_CASE(9) CCS_HUB4_CASE(10) CCS_HUB4_CASE(11)
+    CCS_HUB4_CASE(12) CCS_HUB4_CASE(13) CCS_HUB4_CASE(14) CCS_HUB4_CASE(15)
+#undef CCS_HUB4_CASE
+    default: return 0u;
+  }
+}
+
+constexpr int kHub4Threads = 128;
+__global__ void __launch_bounds__(kHub4Threads, 6) sample_hub4_kernel(DevPlan P, DevRes R, EvalParams E,
+                                                                    const int2* items, int2* items_list,
+                                                                    int keep_counts, int hist_words) {
+  extern __shared__ __align__(16) uint32_t h32[];
+  __shared__ uint32_t tbl[2][256];
+  __shared__ int s_czD[16], s_czS[16], s_nzm[2];
+  __shared__ unsigned s_tot, s_over;
+  __shared__ int s_ident;
+  const int tid = threadIdx.x, nt = kHub4Threads;
+  const int2 it = items[blockIdx.x];
+  {   // zero the histogram while the variant's record is on its way
+    uint4* h4 = reinterpret_cast<uint4*>(h32);
+    for (int i = tid; i < hist_words / 4; i += nt) h4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 4 * (hist_words / 4) + tid; i < hist_words; i += nt) h32[i] = 0u;
+  }
+  if (tid == 0) s_tot = s_over = 0u;
+  const FragDev& F = P.frags[it.x];
+  const int v = it.y, nA = F.nA, m = F.m, M = 1 << m;
+  const SpaceRec& sp = R.spaces[F.space_off + v];
+  const int rank = sp.rank;
+  const uint32_t off = sp.off;
+  if ((unsigned long long)E.shots > (4ull << rank)) {
+    if (tid == 0) items_list[atomicAdd(&R.work[2], 1u)] = it;
+    return;
+  }
+  if ((tid >> 5) == 1) {
+    const bool id = space_is_identity(sp, rank, nA);
+    if (tid == 32) s_ident = id ? 1 : 0;
+  }
+  hub_variant_rows(F, v, s_czD, s_czS, s_nzm);
+  __syncthreads();
+  const bool ident = s_ident != 0;
+  if (!ident) {
+    build_tables<2>(tbl, sp, rank);
+    __syncthreads();
+  }
+  count_shots<4>(h32, ident, rank, tbl, off, E.shots,
+                 make_uint4(0u, (uint32_t)v, (uint32_t)F.findex, (uint32_t)F.problem), E.keys);
+  __syncthreads();
+  if (keep_counts) {
+    uint32_t* g = R.counts + F.counts_off + ((long long)v << nA);
+    for (uint32_t y = tid; y < (1u << nA); y += nt) g[y] = (h32[y >> 3] >> ((y & 7u) << 2)) & 15u;
+  }
+  int16_t* QH = reinterpret_cast<int16_t*>(R.TQ + F.T_off);
+  const int zm = s_nzm[1];
+  unsigned tot = 0, over = 0;
+  switch (F.qout) {
+    case 0: tot = hub4_readout_any<0>(zm, h32, m, M, s_czD, QH, over); break;
+    case 1: tot = hub4_readout_any<1>(zm, h32, m, M, s_czD, QH, over); break;
+    case 2: tot = hub4_readout_any<2>(zm, h32, m, M, s_czD, QH, over); break;
+    case 3: tot = hub4_readout_any<3>(zm, h32, m, M, s_czD, QH, over); break;
+    default: tot = hub4_readout_any<4>(zm, h32, m, M, s_czD, QH, over); break;
+  }
+  tot = __reduce_add_sync(0xffffffffu, tot);
+  over = __reduce_or_sync(0xffffffffu, over);
+  if ((tid & 31) == 0) {
+    atomicAdd(&s_tot, tot);
+    if (over) atomicOr(&s_over, over);
+  }
+  __syncthreads();
+  if (tid == 0 && (s_tot != E.shots || s_over)) items_list[atomicAdd(&R.work[2], 1u)] = it;
+}
+
 // --- stitched mode: a Clifford hub's operand in closed form (Sec. IX) -------
 // A variant's outcomes y = (o, b) (o the marginal bits, b the quantum-output
 // bits) are uniform, probability 2^-r, on off + span(B), B in reduced
@@ -2047,13 +2197,28 @@ cudaError_t launch_hub_exact(const DevPlan& p, const DevRes& r, const int2* item
 }
 
 cudaError_t launch_sample_hub(const DevPlan& p, const DevRes& r, const EvalParams& e, const int2* items, int n_items,
-                              int max_nA, int threads, int keep_counts, bool bytes_ok, cudaStream_t s) {
+                              int max_nA, int threads, int keep_counts, bool bytes_ok, int2* nibble_list,
+                              int sm_count, cudaStream_t s) {
   if (n_items == 0 || e.shots == 0) return cudaSuccess;
+  if (bytes_ok && threads == kHub4Threads && nibble_list) {
+    const int words = std::max(1, (1 << max_nA) / 8), bytes = 1 << max_nA;
+    cudaError_t err =
+        cudaFuncSetAttribute(sample_hub4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * words);
+    if (err != cudaSuccess) return err;
+    sample_hub4_kernel<<<n_items, kHub4Threads, 4 * words, s>>>(p, r, e, items, nibble_list, keep_counts, words);
+    note_launch();
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    auto rest = sample_hub8_kernel<256, true>;
+    if ((err = cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return err;
+    rest<<<std::min(n_items, 3 * sm_count), 256, bytes, s>>>(p, r, e, nibble_list, keep_counts, bytes / 4);
+    note_launch();
+    return cudaGetLastError();
+  }
   if (bytes_ok && e.shots <= 0xffffu && max_nA >= 2 && max_nA <= 16) {   // byte counters, 256 or 512 threads
     const int t8 = threads >= 512 ? 512 : 256;
     const int hist_words = (1 << max_nA) / 4;
     const size_t smem = (size_t)4 * hist_words + (size_t)t8 * (e.shots <= 32767u ? 0 : 33) * 4;
-    auto kern = t8 == 512 ? sample_hub8_kernel<512> : sample_hub8_kernel<256>;
+    auto kern = t8 == 512 ? sample_hub8_kernel<512, false> : sample_hub8_kernel<256, false>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     kern<<<n_items, t8, smem, s>>>(p, r, e, items, keep_counts, hist_words); note_launch();
