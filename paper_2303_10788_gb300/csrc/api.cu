@@ -1390,7 +1390,7 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
     int grid = std::min(dp.n_items_cliff, c->sm_count * per_sm);
     stage_begin(c, ST_CLIFFORD);
     if (e.shared_body) {
-      if ((err = launch_body(dp, r->dr, (int)c->smem_optin, e.screen != 0, s)) != cudaSuccess)
+      if ((err = launch_body(dp, r->dr, (int)c->smem_optin, e.screen != 0, e.proj != 0, c->sm_count, s)) != cudaSuccess)
         return cuda_fail(c, err, "body kernel");
       if (e.screen && (err = launch_screen(dp, r->dr, e, c->sm_count, (int)c->smem_optin, s)) != cudaSuccess)
         return cuda_fail(c, err, "screen kernel");
@@ -1681,6 +1681,7 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
     const bool variant_path = r->variant_path && !opts->keep_tableaus && p->tableau_fits;
     e.shared_body = (opts->per_variant_body || variant_path) ? 0 : 1;
     e.screen = e.shared_body && p->dp.n_cliff_frags > 0 && !e.keep_tableaus;
+    e.proj = p->dp.n_items_cliff > 8 * c->sm_count;      // more variants than one wave of 8-warp CTAs
     if (opts->hub_sampler < 0 || opts->hub_sampler > 3) return fail(c, CCS_ERR_INVALID_ARG, "bad hub sampler");
     e.hub_sampler = opts->hub_sampler;
     if (opts->hub_sampler == 1) {

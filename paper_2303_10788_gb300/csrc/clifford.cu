@@ -229,108 +229,208 @@ __device__ void prep_rows_from_body(const CliffordOp* s_prep, const int* s_qin, 
 
 }  // namespace
 
-namespace {
-// Deep, narrow circuits (moments of a few ops: a chain) are bound by the
-// latency of each op, not by tableau traffic, so their ops are applied
-// cooperatively: eight lanes per op, lane (h, j) producing output column j
-// (X_a, Z_a, X_b, Z_b) on 32-bit half h of the word and a quarter of the
-// op's sign-flip terms (terms 4j .. 4j+3 of its algebraic normal form, whose
-// factors in v2, v3 are fixed by j), reduced over the four lanes of the half
-// by shuffles: the arithmetic of apply_op_g, split over lanes.  Every lane of
-// the block must call it.
-__device__ __forceinline__ void apply_moment_coop(const CliffordOp* ops, int c0, int n_ops, uint32_t* t32, int zb,
-                                                  uint64_t& rd) {
-  const int lane = threadIdx.x & 31;
-  for (int t0 = (int)threadIdx.x - lane; t0 < 8 * n_ops; t0 += (int)blockDim.x) {
-    const int t = t0 + lane;
-    const bool act = t < 8 * n_ops;
-    const int h = (t >> 2) & 1, j = t & 3;
-    uint32_t u = 0u, r = 0u, v0 = 0u, v1 = 0u, v2 = 0u, v3 = 0u;
-    int col = 0;
-    if (act) {
-      const CliffordOp op = ops[c0 + (t >> 3)];
-      v0 = t32[2 * op.qa + h];
-      v1 = t32[2 * (zb + op.qa) + h];
-      v2 = t32[2 * op.qb + h];
-      v3 = t32[2 * (zb + op.qb) + h];
-      const unsigned M = op.M >> (4 * j), A = (op.anf & ~1u) >> (4 * j);   // ANF term 0 is not used
-      u = (v0 & bm32(M, 0)) ^ (v1 & bm32(M, 1)) ^ (v2 & bm32(M, 2)) ^ (v3 & bm32(M, 3));
-      const uint32_t hi = ((j & 1) ? v2 : ~0u) & ((j & 2) ? v3 : ~0u);
-      r = hi & (bm32(A, 0) ^ (v0 & bm32(A, 1)) ^ (v1 & bm32(A, 2)) ^ ((v0 & v1) & bm32(A, 3)));
-      col = j == 0 ? op.qa : j == 1 ? zb + op.qa : j == 2 ? op.qb : zb + op.qb;
-    }
-    r ^= __shfl_xor_sync(0xffffffffu, r, 1);
-    r ^= __shfl_xor_sync(0xffffffffu, r, 2);
-    __syncwarp();                            // every lane has read its inputs
-    if (act) {
-      t32[2 * col + h] = u;
-      if (j == 0) rd ^= (uint64_t)r << (32 * h);
-    }
-  }
-}
-}  // namespace
-
 // --- shared body: one CTA per (Clifford fragment, 64-row word) -------------
 // Rows evolve independently under conjugation, so each word of every column
 // is an independent problem: the CTA keeps one word per column in shared
-// memory and applies the whole op stream to it, moment by moment.
-template <bool COOP>   // COOP: eight lanes per op (moments of at most 32 ops)
-__global__ void __launch_bounds__(256) body_kernel(DevPlan P, DevRes R, int smem_words) {
+// memory and applies the whole op stream to it, moment by moment.  A moment is
+// a short dependent chain (read four columns, combine, write, barrier) and the
+// body a long one of moments, so what bounds the kernel is a moment's latency
+// and, for wide moments, its instruction issue.  Four lanes share an op, lane j
+// producing output column j (X_a, Z_a, X_b, Z_b) and the sign-flip terms
+// 4 j .. 4 j + 3 of the op's algebraic normal form (their factors in v2, v3
+// are fixed by j); the sign words are summed per lane and reduced once at the
+// end.  The next moment's op is decoded while this moment's loads are in
+// flight, its word fetched a moment earlier still.  Moments of at most 16 ops
+// run in a single warp with no block barrier.  A deep narrow body (301 wires,
+// 307 moments) took 790 cycles a moment with eight lanes per op, a shuffle
+// reduction and a barrier each; BODY_TIMES.
+namespace {
+struct OpLane {          // one lane's part of an op
+  int a0, a1, a2, a3, out;               // column indices
+  uint32_t m0, m1, m2, m3;               // its row of the 4 x 4 matrix, as masks
+  uint32_t q0, q1, q2, q3;               // its sign-flip terms
+  bool act;
+};
+// All ones where the top bit of byte SEL & 7 of x is set (prmt's sign-replicating
+// selectors): four masks from one shifted word.
+__device__ __forceinline__ uint32_t sign_mask(uint32_t x, uint32_t sel) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "r"(sel));
+  return r;
+}
+__device__ __forceinline__ void decode_op(uint2 w, bool act, int j, int zb, OpLane& d) {
+  const int qa = (int)(w.x & 0xffffu), qb = (int)(w.x >> 16);
+  // bits 4 j + k of M and of the sign form: byte j / 2 of the word's halves, bit 4 (j & 1) + k
+  const uint32_t t = (w.y & ~(1u << 16)) << (4 - 4 * (j & 1));             // ANF term 0 is not used
+  const uint32_t sm = 0x8888u + 0x1111u * (uint32_t)(j >> 1), sa = sm + 0x2222u;
+  d.act = act;
+  d.a0 = qa;
+  d.a1 = zb + qa;
+  d.a2 = qb;
+  d.a3 = zb + qb;
+  d.out = ((j & 2) ? qb : qa) + ((j & 1) ? zb : 0);
+  d.m0 = sign_mask(t << 3, sm); d.m1 = sign_mask(t << 2, sm); d.m2 = sign_mask(t << 1, sm); d.m3 = sign_mask(t, sm);
+  d.q0 = sign_mask(t << 3, sa); d.q1 = sign_mask(t << 2, sa); d.q2 = sign_mask(t << 1, sa); d.q3 = sign_mask(t, sa);
+}
+// s2 / s3: all ones where the lane's terms do not contain v2 / v3.
+__device__ __forceinline__ void op_half(const OpLane& d, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, uint32_t s2,
+                                        uint32_t s3, uint32_t& u, uint32_t& r) {
+  u = (v0 & d.m0) ^ (v1 & d.m1) ^ (v2 & d.m2) ^ (v3 & d.m3);
+  r ^= (v2 | s2) & (v3 | s3) & (d.q0 ^ (v0 & d.q1) ^ (v1 & d.q2) ^ (v0 & v1 & d.q3));
+}
+
+// A whole op by one thread: its 31 masks from the word's eight shifts.
+__device__ __forceinline__ void apply_whole(uint2 w, uint2* tab, int zb, uint2& rd) {
+  uint32_t m[16], a[16];
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    const uint32_t t = w.y << s;
+    m[7 - s] = sign_mask(t, 0x8888u);
+    m[15 - s] = sign_mask(t, 0x9999u);
+    a[7 - s] = sign_mask(t, 0xaaaau);
+    a[15 - s] = sign_mask(t, 0xbbbbu);
+  }
+  const int qa = (int)(w.x & 0xffffu), qb = (int)(w.x >> 16);
+  const uint2 V0 = tab[qa], V1 = tab[zb + qa], V2 = tab[qb], V3 = tab[zb + qb];
+  uint2 U[4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t v0 = h ? V0.y : V0.x, v1 = h ? V1.y : V1.x, v2 = h ? V2.y : V2.x, v3 = h ? V3.y : V3.x;
+    const uint32_t v01 = v0 & v1;
+    // the sign form as (1, v2, v3, v2 v3) times polynomials in v0, v1
+    const uint32_t p0 = (v0 & a[1]) ^ (v1 & a[2]) ^ (v01 & a[3]);
+    const uint32_t p2 = a[4] ^ (v0 & a[5]) ^ (v1 & a[6]) ^ (v01 & a[7]);
+    const uint32_t p3 = a[8] ^ (v0 & a[9]) ^ (v1 & a[10]) ^ (v01 & a[11]);
+    const uint32_t p23 = a[12] ^ (v0 & a[13]) ^ (v1 & a[14]) ^ (v01 & a[15]);
+    const uint32_t r = p0 ^ (v2 & p2) ^ (v3 & (p3 ^ (v2 & p23)));
+    if (h) rd.y ^= r;
+    else rd.x ^= r;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t u = (v0 & m[4 * i]) ^ (v1 & m[4 * i + 1]) ^ (v2 & m[4 * i + 2]) ^ (v3 & m[4 * i + 3]);
+      if (h) U[i].y = u;
+      else U[i].x = u;
+    }
+  }
+  tab[qa] = U[0];
+  tab[zb + qa] = U[1];
+  tab[qb] = U[2];
+  tab[zb + qb] = U[3];
+}
+}  // namespace
+
+// MODE 0: one warp, four lanes per op; 1: up to 32 warps, four lanes per op; 2: a
+// thread per op (half the instructions, for plans with many bodies).
+template <int MODE>
+__global__ void __launch_bounds__(MODE == 0 ? 32 : MODE == 1 ? 1024 : 256) body_kernel(DevPlan P, DevRes R, int smem_words) {
+  constexpr bool ONE_WARP = MODE == 0;
+  constexpr int PER = MODE == 2 ? 1 : 4;              // lanes of an op
   extern __shared__ __align__(16) unsigned long long smem_u64[];
-  uint64_t* tab = reinterpret_cast<uint64_t*>(smem_u64);
+  uint2* tab = reinterpret_cast<uint2*>(smem_u64);      // (low, high) halves of a column's word
   const int2 it = P.items_body[blockIdx.x];
   const FragDev& F = P.frags[it.x];
-  const int n = F.n, W = F.W, Wh = F.Wh, zb = n + 1, rcol = 2 * (n + 1), ncol = 2 * n + 3;
-  const int w = it.y, tid = threadIdx.x, nt = blockDim.x;
+  const int n = F.n, W = F.W, Wh = F.Wh, zb = n + 1, rcol = 2 * (n + 1), ncol = 2 * n + 3, n_mom = F.n_moments;
+  const int w = it.y, tid = threadIdx.x;
+  // warps a narrower fragment has no ops for (n / 2 ops a moment) leave
+  const int nt = ONE_WARP ? 32 : min((int)blockDim.x, 32 * max(1, (PER * n / 2 + 31) / 32));
+  if (!ONE_WARP && tid >= nt) return;
+  auto sync = [&]() {
+    if (ONE_WARP) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+  };
   // the op stream and moment offsets follow the column words when they fit
-  const int n_ops = P.moments[F.mom_off + F.n_moments];
-  const bool staged = ncol + n_ops + (F.n_moments + 2) / 2 + 1 <= smem_words;
-  CliffordOp* ops_s = reinterpret_cast<CliffordOp*>(tab + ncol);
+  const int* gmom = P.moments + F.mom_off;
+  const int n_ops = gmom[n_mom];
+  const bool staged = ncol + n_ops + (n_mom + 2) / 2 + 1 <= smem_words;
+  const uint2* gops = reinterpret_cast<const uint2*>(P.cops + F.ops_off);
+  uint2* ops_s = tab + ncol;
   int* mom_s = reinterpret_cast<int*>(tab + ncol + n_ops);
   if (staged) {
-    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(P.cops + F.ops_off);
-    for (int i = tid; i < n_ops; i += nt) reinterpret_cast<unsigned long long*>(ops_s)[i] = src[i];
-    for (int i = tid; i <= F.n_moments; i += nt) mom_s[i] = P.moments[F.mom_off + i];
+#pragma unroll 8
+    for (int i = tid; i < n_ops; i += nt) ops_s[i] = gops[i];
+#pragma unroll 4
+    for (int i = tid; i <= n_mom; i += nt) mom_s[i] = gmom[i];
   }
-  for (int c = tid; c < ncol; c += nt) tab[c] = 0ull;
-  __syncthreads();
   {   // identity: destabilizer i = X_i (words [0, Wh)), stabilizer i = Z_i
-    const int half = w < Wh ? 0 : 1, i0 = 64 * (w - half * Wh);
-    for (int i = i0 + tid; i < min(n, i0 + 64); i += nt) tab[half ? zb + i : i] = 1ull << (i & 63);
-  }
-  __syncthreads();
-  const CliffordOp* ops = staged ? ops_s : P.cops + F.ops_off;
-  const int* mom = staged ? mom_s : P.moments + F.mom_off;
-  const int wk[1] = {0};
-  uint64_t rd[1] = {0ull};
-  if (COOP) {
-    uint32_t* t32 = reinterpret_cast<uint32_t*>(tab);
-    for (int mm = 0; mm < F.n_moments; ++mm) {
-      apply_moment_coop(ops, mom[mm], mom[mm + 1] - mom[mm], t32, zb, rd[0]);
-      __syncthreads();
+    const int half = w < Wh ? 0 : 1, c0 = (half ? zb : 0) + 64 * (w - half * Wh), cn = (half ? zb : 0) + n;
+    for (int c = tid; c < ncol; c += nt) {
+      const int b = c - c0;
+      const bool one = b >= 0 && b < 64 && c < cn;
+      tab[c] = make_uint2(one && b < 32 ? 1u << b : 0u, one && b >= 32 ? 1u << (b - 32) : 0u);
     }
-  } else if (F.n_moments > 0) {
-    // each thread's first op of the next moment is fetched while this
-    // moment's op is applied (the op stream does not depend on the tableau)
-    int b0 = mom[0], b1 = mom[1];
-    CliffordOp nxt{};
-    if (b0 + tid < b1) nxt = ops[b0 + tid];
-    for (int mm = 0; mm < F.n_moments; ++mm) {
-      const int c0 = b0, c1 = b1;
-      const CliffordOp cur = nxt;
-      if (mm + 1 < F.n_moments) {
-        b0 = c1;
-        b1 = mom[mm + 2];
-        if (b0 + tid < b1) nxt = ops[b0 + tid];
+  }
+  sync();
+  const int j = tid % PER, k0 = tid / PER, slots = nt / PER;
+  const uint32_t s2 = (j & 1) ? 0u : ~0u, s3 = (j & 2) ? 0u : ~0u;
+  auto fetch = [&](int o, int end) -> uint2 {
+    if (o >= end) return make_uint2(0u, 0u);
+    return staged ? ops_s[o] : gops[o];
+  };
+  auto bound = [&](int mm) -> int { return mm > n_mom ? n_ops : staged ? mom_s[mm] : gmom[mm]; };
+  uint2 rd = make_uint2(0u, 0u);
+  auto apply = [&](const OpLane& d) {
+    uint2 v0, v1, v2, v3, u;
+    if (d.act) { v0 = tab[d.a0]; v1 = tab[d.a1]; v2 = tab[d.a2]; v3 = tab[d.a3]; }
+    __syncwarp();                              // an op's four lanes have read its columns
+    if (d.act) {
+      op_half(d, v0.x, v1.x, v2.x, v3.x, s2, s3, u.x, rd.x);
+      op_half(d, v0.y, v1.y, v2.y, v3.y, s2, s3, u.y, rd.y);
+      tab[d.out] = u;
+    }
+  };
+  if (MODE == 2) {
+    int b0 = bound(0), b1 = bound(1);
+    uint2 raw = fetch(b0 + k0, b1);            // the next moment's op word is fetched while this one's is applied
+    for (int mm = 0; mm < n_mom; ++mm) {
+      const int b2 = bound(mm + 2);
+      const uint2 now = raw;
+      raw = fetch(b1 + k0, b2);
+      if (b0 + k0 < b1) apply_whole(now, tab, zb, rd);
+      for (int o = b0 + k0 + slots; o < b1; o += slots) apply_whole(fetch(o, b1), tab, zb, rd);
+      b0 = b1;
+      b1 = b2;
+      sync();
+    }
+  } else if (n_mom > 0) {
+    int b0 = bound(0), b1 = bound(1), b2 = bound(2);
+    OpLane cur;
+    decode_op(fetch(b0 + k0, b1), b0 + k0 < b1, j, zb, cur);
+    uint2 raw = fetch(b1 + k0, b2);            // of the next moment
+    for (int mm = 0; mm < n_mom; ++mm) {
+      uint2 v0, v1, v2, v3, u;
+      if (cur.act) { v0 = tab[cur.a0]; v1 = tab[cur.a1]; v2 = tab[cur.a2]; v3 = tab[cur.a3]; }
+      OpLane nxt;                              // decoded while the loads are in flight
+      decode_op(raw, b1 + k0 < b2, j, zb, nxt);
+      const int b3 = bound(mm + 3);
+      raw = fetch(b2 + k0, b3);
+      __syncwarp();                            // an op's four lanes have read its columns
+      if (cur.act) {
+        op_half(cur, v0.x, v1.x, v2.x, v3.x, s2, s3, u.x, rd.x);
+        op_half(cur, v0.y, v1.y, v2.y, v3.y, s2, s3, u.y, rd.y);
+        tab[cur.out] = u;
       }
-      if (c0 + tid < c1) apply_op_g<1>(cur, tab, 1, zb, wk, rd);
-      for (int o = c0 + tid + nt; o < c1; o += nt) apply_op_g<1>(ops[o], tab, 1, zb, wk, rd);
-      __syncthreads();
+      for (int o = b0 + slots; o < b1; o += slots) {    // further ops of a wide moment
+        OpLane d;
+        decode_op(fetch(o + k0, b1), o + k0 < b1, j, zb, d);
+        apply(d);
+      }
+      cur = nxt;
+      b0 = b1;
+      b1 = b2;
+      b2 = b3;
+      sync();
     }
   }
-  atomicXor(reinterpret_cast<unsigned long long*>(&tab[rcol]), (unsigned long long)rd[0]);
-  __syncthreads();
-  unsigned long long* dst = R.body + F.body_off;
+  for (int o = 16; o; o >>= 1) {
+    rd.x ^= __shfl_xor_sync(0xffffffffu, rd.x, o);
+    rd.y ^= __shfl_xor_sync(0xffffffffu, rd.y, o);
+  }
+  if ((tid & 31) == 0) {
+    atomicXor(&tab[rcol].x, rd.x);
+    atomicXor(&tab[rcol].y, rd.y);
+  }
+  sync();
+  uint2* dst = reinterpret_cast<uint2*>(R.body + F.body_off);
   for (int c = tid; c < ncol; c += nt) dst[(size_t)c * W + w] = tab[c];
 }
 
@@ -363,7 +463,14 @@ __device__ __forceinline__ unsigned long long warp_xor64(unsigned long long x) {
 }
 
 // One record, by one CTA: the anticommutation bits (acc, by warp 0), then
-// the ordered row product with its phase, threads over the body's columns.
+// the phase of the ordered row product, threads over the body's columns.  Per
+// column, with rows as i^(x z) X^x Z^z up to sign, the product of the selected
+// rows in order is
+//   i^(sum_a x_a z_a) (-1)^(sum_{a<b} z_a x_b) X^cx Z^cz,
+// X^cx Z^cz = i^(-cx cz) times the Pauli (cx, cz): bit-sliced two-bit counters
+// of x & z, one prefix parity (of z) per word, and parities of XORs (counting
+// the four-valued exponent of every single-qubit product took two prefix
+// parities and two popcounts per word, 25 k cycles a record at 500 wires).
 // The body stays in global memory: a column's W words share one or two
 // 128-byte lines, so after the first touch they come from L1.
 __device__ void z_image(const DevPlan& P, const DevRes& R, const FragDev& F, int k, unsigned long long* s_sel,
@@ -377,15 +484,15 @@ __device__ void z_image(const DevPlan& P, const DevRes& R, const FragDev& F, int
   if (tid < 32) {
     unsigned long long acc = 0ull;      // lane w < W: anticommutation bits of the rows in word w
     if (k < F.nz) {
-      // Z_S: the x-columns of the string's wires, XORed (lanes over wires)
+      // Z_S: the x-columns of the string's wires, XORed
       const int q0 = P.zoffs[F.zw_off + k], q1 = P.zoffs[F.zw_off + k + 1];
-      for (int t0 = q0; t0 < q1; t0 += 32) {
-        const int wq = t0 + lane < q1 ? P.wires[t0 + lane] : -1;
-        if (wq >= 0) atomicXor(&s_ez[wq >> 6], 1ull << (wq & 63));
-        for (int w = 0; w < W; ++w) {
-          const unsigned long long x = warp_xor64(wq >= 0 ? tab[(size_t)wq * W + w] : 0ull);
-          if (lane == w) acc ^= x;
-        }
+      for (int t = q0 + lane; t < q1; t += 32) {
+        const int wq = P.wires[t];
+        atomicXor(&s_ez[wq >> 6], 1ull << (wq & 63));
+      }
+      if (lane < W) {
+#pragma unroll 4
+        for (int t = q0; t < q1; ++t) acc ^= tab[(size_t)P.wires[t] * W + lane];
       }
     } else {
       int wq;
@@ -416,23 +523,25 @@ __device__ void z_image(const DevPlan& P, const DevRes& R, const FragDev& F, int
   int e = 0;
   unsigned bad = 0;
   for (int j = tid; j < n; j += nt) {
-    unsigned cx = 0, cz = 0;
-    const unsigned long long* xc = tab + (size_t)j * W;
-    const unsigned long long* zc = tab + (size_t)(zb + j) * W;
-    for (int w = 0; w < W; ++w) {
-      const unsigned long long sw = s_sel[w];
-      const unsigned long long x = xc[w] & sw;
-      const unsigned long long z = zc[w] & sw;
-      const unsigned long long px = prefix_xor_excl(x) ^ (cx ? ~0ull : 0ull);
-      const unsigned long long pz = prefix_xor_excl(z) ^ (cz ? ~0ull : 0ull);
-      const unsigned long long X1 = px & ~pz, Y1 = px & pz, Z1 = ~px & pz;
-      const unsigned long long X2 = x & ~z, Y2 = x & z, Z2 = ~x & z;
-      const unsigned long long plus = (X1 & Y2) | (Y1 & Z2) | (Z1 & X2);
-      const unsigned long long minus = (X1 & Z2) | (Y1 & X2) | (Z1 & Y2);
-      e += __popcll(plus) - __popcll(minus);
-      cx ^= __popcll(x) & 1;
-      cz ^= __popcll(z) & 1;
+    // (W is even and every column starts on 16 bytes)
+    const ulonglong2* xc = reinterpret_cast<const ulonglong2*>(tab + (size_t)j * W);
+    const ulonglong2* zc = reinterpret_cast<const ulonglong2*>(tab + (size_t)(zb + j) * W);
+    unsigned long long y0 = 0ull, y1 = 0ull, xx = 0ull, sw = 0ull, carry = 0ull;
+    auto word = [&](unsigned long long x, unsigned long long z) {
+      const unsigned long long y = x & z, pz = prefix_xor_excl(z) ^ carry;
+      y1 ^= y0 & y;
+      y0 ^= y;
+      xx ^= x;
+      sw ^= x & pz;
+      carry = (unsigned long long)((long long)(pz ^ z) >> 63);      // all ones: odd so far
+    };
+    for (int w = 0; w < W; w += 2) {
+      const ulonglong2 x = xc[w >> 1], z = zc[w >> 1];
+      word(x.x & s_sel[w], z.x & s_sel[w]);
+      word(x.y & s_sel[w + 1], z.y & s_sel[w + 1]);
     }
+    const unsigned cx = __popcll(xx) & 1, cz = (unsigned)carry & 1u;
+    e += __popcll(y0) + 2 * __popcll(y1) + 2 * (__popcll(sw) & 1) - (int)(cx & cz);
     // the product must be Q itself up to phase
     if (cx != (unsigned)((s_ex[j >> 6] >> (j & 63)) & 1ull) || cz != (unsigned)((s_ez[j >> 6] >> (j & 63)) & 1ull))
       bad = 1;
@@ -575,6 +684,62 @@ __device__ __forceinline__ void absorb64(unsigned long long row, unsigned long l
 }
 }  // namespace
 
+namespace {
+// Echelon basis of the shared rows from their columns (one warp, lane j the
+// rows' bit j as NW words, ne <= 32): for each p in turn a row with bit p set is
+// the pivot row, its bits (one per lane) by ballot, and every column in which
+// it has a one takes column p added: the row operations of all rows at once,
+// about 70 cycles a pivot where 32 rows per warp, merged over eight warps, took
+// 13 to 24 k cycles in all.  eb[p] = the vector with lowest set bit p.
+template <int NW>
+__device__ __forceinline__ unsigned echelon_columns(unsigned long long (&cw)[NW], int ne, unsigned long long* eb) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  unsigned have = 0u;
+  for (int p = 0; p < ne; ++p) {
+    unsigned long long pw[NW];
+    int wr = -1;
+#pragma unroll
+    for (int w = NW - 1; w >= 0; --w) {
+      pw[w] = __shfl_sync(FULL, cw[w], p);
+      if (pw[w]) wr = w;
+    }
+    if (wr < 0) continue;
+    unsigned long long pv = 0ull, own = 0ull;
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+      if (w == wr) { pv = pw[w]; own = cw[w]; }
+    const bool bit = (own & (pv & (0ull - pv))) != 0ull;
+    const unsigned prow = __ballot_sync(FULL, bit);
+    if (bit) {
+#pragma unroll
+      for (int w = 0; w < NW; ++w) cw[w] ^= pw[w];
+    }
+    if (lane == 0) eb[p] = prow;
+    have |= 1u << p;
+  }
+  __syncwarp();
+  return have;
+}
+// The same from the body: column j's stabilizer words without the input rows.
+template <int NW>
+__device__ __forceinline__ unsigned echelon_body(const unsigned long long* body, const FragDev& F, const int* s_col,
+                                                 const int* s_in, int ne, unsigned long long* eb) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long cw[NW];
+#pragma unroll
+  for (int w = 0; w < NW; ++w)
+    cw[w] = lane < ne && w < F.Wh ? body[(size_t)s_col[lane] * F.W + F.Wh + w] : 0ull;
+  for (int k = 0; k < F.qin; ++k) {
+    const int q = s_in[k];
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+      if (w == (q >> 6)) cw[w] &= ~(1ull << (q & 63));
+  }
+  return echelon_columns<NW>(cw, ne, eb);
+}
+}  // namespace
+
 // --- shared-row basis, Z images and offset table ----------------------------
 // CTAs [0, n_cliff_frags): one per Clifford fragment.  Every variant keeps
 // the body's stabilizer rows outside its quantum inputs; only the input rows
@@ -590,12 +755,15 @@ __device__ __forceinline__ void absorb64(unsigned long long row, unsigned long l
 // r = m + 3 o + d: output o in basis d) gets its phase, its (a, b) bits on
 // the quantum inputs, and the parities popc(b_k & a_r) mod 2 for every
 // record k, so that the phase of any product of records needs no vectors.
+constexpr int kMaxRecords = 64;    // measurement records of a fragment: m + 3 qout (m + qout <= 24, qout <= 12)
 __global__ void __launch_bounds__(256) body_basis_kernel(DevPlan P, DevRes R) {
   __shared__ unsigned long long s_eb[8][64];
   __shared__ unsigned long long s_eh[8];
   __shared__ int s_col[64];
   __shared__ int s_in[kMaxCuts];
-  __shared__ unsigned long long s_cw[64][kMaxWh];   // stabilizer halves of the extended columns
+  // measurement records while the table is built; stabilizer halves of the extended columns
+  __shared__ unsigned long long s_buf[kMaxRecords * (2 * kMaxWh + 1)];
+  unsigned long long (*s_cw)[kMaxWh] = reinterpret_cast<unsigned long long (*)[kMaxWh]>(s_buf);
   __shared__ unsigned long long s_zs[4 * kMaxWh];   // record scratch: sel (2 Wh), expected x, expected z
   __shared__ int s_e;
   __shared__ unsigned s_bad, s_last;
@@ -618,27 +786,29 @@ __global__ void __launch_bounds__(256) body_basis_kernel(DevPlan P, DevRes R) {
     if (tid < 64) s_ct[tid] = 0ull;
     if (tid < F.qin) s_in[tid] = P.wires[F.qin_off + tid];
     __syncthreads();
-    const unsigned long long* img = R.zimg + F.zimg_off;
-    auto recp = [&](int r) { return img + (size_t)(r < m ? zm + r : F.nz + (r - m)) * st; };
+    // the records (wires first, then the outputs' bases), staged once
+    for (int i = tid; i < nrec * st; i += nt) {
+      const int r = i / st;
+      s_buf[i] = __ldcg(R.zimg + F.zimg_off + (size_t)(r < m ? zm + r : F.nz + (r - m)) * st + (i - r * st));
+    }
+    __syncthreads();
     for (int pr = tid; pr < nrec * nrec; pr += nt) {
       const int l = pr / nrec, k = pr % nrec;       // bit k of ct[l]: popc(b_k & a_l) mod 2
-      const unsigned long long* ak = recp(k);
-      const unsigned long long* al = recp(l);
-      int c = 0;
-      for (int w = 0; w < Wh; ++w) c += __popcll(__ldcg(ak + Wh + w) & __ldcg(al + w));
-      if (c & 1) atomicOr(&s_ct[l], 1ull << k);
+      unsigned long long c = 0ull;
+      for (int w = 0; w < Wh; ++w) c ^= s_buf[k * st + Wh + w] & s_buf[l * st + w];
+      if (__popcll(c) & 1) atomicOr(&s_ct[l], 1ull << k);
     }
     __syncthreads();
     unsigned long long* out = R.rowbasis + F.rb_off;
     for (int r = tid; r < 64; r += nt) {
       unsigned long long info = 0ull;
       if (r < nrec) {
-        const unsigned long long* ar = recp(r);
-        info = __ldcg(ar + 2 * Wh) & 3ull;
+        const unsigned long long* ar = s_buf + r * st;
+        info = ar[2 * Wh] & 3ull;
         for (int i = 0; i < F.qin; ++i) {
           const int q = s_in[i];
-          info |= ((__ldcg(ar + (q >> 6)) >> (q & 63)) & 1ull) << (2 + i);
-          info |= ((__ldcg(ar + Wh + (q >> 6)) >> (q & 63)) & 1ull) << (16 + i);
+          info |= ((ar[q >> 6] >> (q & 63)) & 1ull) << (2 + i);
+          info |= ((ar[Wh + (q >> 6)] >> (q & 63)) & 1ull) << (16 + i);
         }
       }
       out[65 + r] = r < nrec ? s_ct[r] : 0ull;
@@ -656,6 +826,35 @@ __global__ void __launch_bounds__(256) body_basis_kernel(DevPlan P, DevRes R) {
   }
   __syncthreads();
   const unsigned long long* body = R.body + F.body_off;
+  if (ne <= 32) {       // warp 0: the basis; the other warps: the inputs' rows
+    if (warp == 0) {
+      const unsigned hv = Wh <= 1   ? echelon_body<1>(body, F, s_col, s_in, ne, s_eb[0])
+                          : Wh <= 2 ? echelon_body<2>(body, F, s_col, s_in, ne, s_eb[0])
+                          : Wh <= 4 ? echelon_body<4>(body, F, s_col, s_in, ne, s_eb[0])
+                          : Wh <= 8 ? echelon_body<8>(body, F, s_col, s_in, ne, s_eb[0])
+                                    : echelon_body<kMaxWh>(body, F, s_col, s_in, ne, s_eb[0]);
+      unsigned long long* out = R.rowbasis + F.rb_off;
+      out[lane] = ((hv >> lane) & 1u) ? s_eb[0][lane] : 0ull;
+      out[lane + 32] = 0ull;
+      if (lane == 0) out[64] = hv;
+      return;
+    }
+    for (int i = warp - 1; i < F.qin; i += nwarps - 1) {      // a warp per input, a column per lane
+      const int q = s_in[i];
+      unsigned long long dw = 0ull, sw = 0ull;
+      if (lane < ne) {
+        const unsigned long long* col = body + (size_t)s_col[lane] * W;
+        dw = col[q >> 6] >> (q & 63);
+        sw = col[Wh + (q >> 6)] >> (q & 63);
+      }
+      const unsigned qd = __ballot_sync(0xffffffffu, dw & 1ull), qs = __ballot_sync(0xffffffffu, sw & 1ull);
+      if (lane == 0) {
+        R.rowbasis[F.rb_off + kRbInputRows + i] = qd;
+        R.rowbasis[F.rb_off + kRbInputRows + kMaxCuts + i] = qs;
+      }
+    }
+    return;
+  }
   for (int t = tid; t < ne * Wh; t += nt) s_cw[t / Wh][t % Wh] = body[(size_t)s_col[t / Wh] * W + Wh + t % Wh];
   // each quantum input's destabilizer and stabilizer rows as extended vectors
   for (int t = tid; t < F.qin * ne; t += nt) {
@@ -706,7 +905,9 @@ __global__ void __launch_bounds__(256) body_basis_kernel(DevPlan P, DevRes R) {
 
 // The shared rows' basis projected through one output basis combination of
 // one fragment (one warp per (fragment, combination); the screen reads the
-// result instead of projecting per variant).
+// result instead of projecting per variant: launched where the variants are
+// more than one wave of the screen's warps, a launch costing about as much as
+// a projection).
 __global__ void __launch_bounds__(256) proj_kernel(DevPlan P, DevRes R) {
   const int lane = threadIdx.x & 31;
   const int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -720,8 +921,9 @@ __global__ void __launch_bounds__(256) proj_kernel(DevPlan P, DevRes R) {
   for (int o = 0, t = pc; o < F.qout; ++o, t /= 3) pout |= (unsigned)(t % 3) << (2 * o);
   uint32_t h32 = 0, mine = 0;
   absorb32(((sh >> lane) & 1ull) ? project_ext(rb[lane], nA, F.m, F.qout, pout) : 0u, h32, mine, nA, lane);
-  absorb32(((sh >> (lane + 32)) & 1ull) ? project_ext(rb[lane + 32], nA, F.m, F.qout, pout) : 0u, h32, mine, nA,
-           lane);
+  if (sh >> 32)
+    absorb32(((sh >> (lane + 32)) & 1ull) ? project_ext(rb[lane + 32], nA, F.m, F.qout, pout) : 0u, h32, mine, nA,
+             lane);
   uint32_t* pb = R.pbasis + F.pb_off + 25ll * pc;
   if (lane < 24) pb[lane] = ((h32 >> lane) & 1u) ? mine : 0u;
   if (lane == 0) pb[24] = h32;
@@ -794,7 +996,7 @@ __global__ void __launch_bounds__(256) screen_kernel(DevPlan P, DevRes R, EvalPa
     uint32_t have = 0, mine = 0;
     auto absorb = [&](uint32_t row) { absorb32(row, have, mine, nA, lane); };
     const unsigned long long* rb = R.rowbasis + F.rb_off;
-    if (F.pb_off >= 0) {   // the shared rows' basis for this output basis combination
+    if (F.pb_off >= 0 && E.proj) {   // the shared rows' basis for this output basis combination
       int pc = v;
       for (int i = 0; i < F.qin; ++i) pc >>= 2;
       const uint32_t* pb = R.pbasis + F.pb_off + 25ll * pc;
@@ -803,7 +1005,7 @@ __global__ void __launch_bounds__(256) screen_kernel(DevPlan P, DevRes R, EvalPa
     } else {
       const unsigned long long sh = rb[64];
       absorb(((sh >> lane) & 1ull) ? project(rb[lane]) : 0u);
-      absorb(((sh >> (lane + 32)) & 1ull) ? project(rb[lane + 32]) : 0u);
+      if (sh >> 32) absorb(((sh >> (lane + 32)) & 1ull) ? project(rb[lane + 32]) : 0u);
     }
     {   // new stabilizer rows of the quantum inputs (bits only): the image of
         // C Z C^+ is D, S or their product, from the fragment's input rows
@@ -2258,16 +2460,17 @@ cudaError_t launch_clifford(const DevPlan& p, const DevRes& r, const EvalParams&
   }
 }
 
-cudaError_t launch_body(const DevPlan& p, const DevRes& r, int smem_optin, bool basis, cudaStream_t s) {
+cudaError_t launch_body(const DevPlan& p, const DevRes& r, int smem_optin, bool basis, bool proj, int sm_count,
+                        cudaStream_t s) {
   if (p.n_items_body == 0) return cudaSuccess;
   const int words = std::max(p.max_body_cols, std::min(p.max_body_stage_words, smem_optin / 8));
-  // moments of at most 32 ops (deep, narrow circuits): eight lanes per op,
-  // a warp per 4 ops of the widest moment; otherwise one thread per op of the
-  // widest moment (whole warps, 32..256): fewer idle warps at each barrier
-  const bool coop = p.max_moment_ops <= 32;
-  const int threads = coop ? std::max(32, (8 * p.max_moment_ops + 31) / 32 * 32)
-                           : std::min(256, std::max(32, (p.max_moment_ops + 31) / 32 * 32));
-  auto kern = coop ? body_kernel<true> : body_kernel<false>;
+  // moments of at most 16 ops: one warp (two ops in turn at most, no block
+  // barrier).  Wider ones: with few bodies four lanes per op of the widest
+  // moment, up to 1024 threads; with more than two CTAs per SM, where
+  // instruction issue is what counts, a thread per op
+  const int mode = p.max_moment_ops <= 16 ? 0 : p.n_items_body <= 2 * sm_count ? 1 : 2;
+  const int threads = mode == 0 ? 32 : std::min(mode == 1 ? 1024 : 256, ((mode == 1 ? 4 : 1) * p.max_moment_ops + 31) / 32 * 32);
+  auto kern = mode == 0 ? body_kernel<0> : mode == 1 ? body_kernel<1> : body_kernel<2>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, words * 8);
   if (err != cudaSuccess) return err;
   kern<<<p.n_items_body, threads, (size_t)words * 8, s>>>(p, r, words); note_launch();
@@ -2276,7 +2479,7 @@ cudaError_t launch_body(const DevPlan& p, const DevRes& r, int smem_optin, bool 
   if (err != cudaSuccess || p.n_cliff_frags == 0) return err;
   // fragments with no measurement record get no table: nothing reads it
   body_basis_kernel<<<p.n_cliff_frags + p.n_items_zimg, 256, 0, s>>>(p, r); note_launch();
-  if ((err = cudaGetLastError()) != cudaSuccess || p.n_items_proj == 0) return err;
+  if ((err = cudaGetLastError()) != cudaSuccess || p.n_items_proj == 0 || !proj) return err;
   proj_kernel<<<(p.n_items_proj + 7) / 8, 256, 0, s>>>(p, r); note_launch();
   return cudaGetLastError();
 }

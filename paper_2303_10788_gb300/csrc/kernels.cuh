@@ -187,6 +187,7 @@ struct EvalParams {
   int keep_tableaus;
   int shared_body;            // 1: variants start from their fragment's body tableau
   int screen;                 // 1: the screen finishes every Clifford variant (no tableau kernel)
+  int proj;                   // 1: the screen reads the projected shared-row bases
   int hub_sampler;            // host only: the caller's hub sampler choice (0 automatic)
   double inv_shots;
 };
@@ -218,8 +219,9 @@ long long launch_count();
 // Body tableau of every Clifford fragment (identity evolved by the gate
 // sequence, no preparations or basis changes), one CTA per 64-row word.
 // With basis set, a second launch writes the shared-row bases and the Z
-// images the screen needs.
-cudaError_t launch_body(const DevPlan& p, const DevRes& r, int smem_optin, bool basis, cudaStream_t s);
+// images the screen needs, with proj a third one the projected bases.
+cudaError_t launch_body(const DevPlan& p, const DevRes& r, int smem_optin, bool basis, bool proj, int sm_count,
+                        cudaStream_t s);
 // Screen of every Clifford variant from its fragment's shared-row basis and
 // Z images: outcome space (rank, reduced basis, offset) and Z-string values,
 // without a tableau per variant.  Used unless tableaus are kept; then the
