@@ -383,7 +383,8 @@ struct ccs_plan_s {
   int cliff_smem_words = 0, max_nc_n = 1;
   int nc_basis_chunk = 1;           // basis combinations per statevector item
   int body_smem_words = 0;          // variant kernel started from a shared body (no op staging)
-  FoldSet fold_cliff{}, fold_nc{}, fold_hubs{}, fold_hubs_nc{}, fold_others{};
+  FoldSet fold_cliff{}, fold_nc{}, fold_hubs{}, fold_hubs_nc{}, fold_others{};   // fold_others: Clifford leaves,
+  FoldSet fold_others_nc{};                                                      // and statevector leaves
   int2* d_items_hub = nullptr;      // Clifford hub variants (fused sampler)
   int2* d_items_plain = nullptr;    // other Clifford variants (sampler -> counts)
   int n_items_hub = 0, n_items_plain = 0, max_hub_nA = 0;
@@ -395,6 +396,7 @@ struct ccs_plan_s {
   long long n_qrows = 0;            // operand-row flags of the Clifford hubs
   bool stitch_ok = true;            // every Clifford hub has at most 4 quantum outputs
   bool tableau_fits = true;         // every Clifford fragment's whole tableau fits in shared memory
+  bool z_warp = true;               // every problem's Z-strings fit a warp each
   bool all_star = true;             // no problem is summed over its whole cut index for every output
   std::vector<GStep> gsteps;        // tree contractions (problems that are no stars)
   std::vector<FoldSet> tree_levels;
@@ -896,7 +898,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
           if (d.nz > 0)
             for (int v = 0; v < d.nv; v += zblock_variants(d.nz)) zblocks.push_back(make_int2((int)fi, v));
         }
-        max_body_stage = std::max(max_body_stage, 2 * d.n + 3 + (int)f.cops.size() + (d.n_moments + 2) / 2 + 1);
+        max_body_stage = std::max(max_body_stage, 2 * d.n + 3 + (int)f.cops.size() + (d.n_moments + 5) / 2 + 1);
         for (int mm = 0; mm < f.n_moments(); ++mm)
           max_moment_ops = std::max(max_moment_ops, f.moment_start[mm + 1] - f.moment_start[mm]);
         for (int w = 0; w < d.W; ++w) items_b.push_back(make_int2((int)fi, w));
@@ -1039,8 +1041,8 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     // fold sets: T of non-hub Clifford fragments (main stream) and non-hub
     // statevector fragments (side branch); T^S of every fragment; then the
     // contraction operands Q (hubs) and T' (the others)
-    std::vector<int> fidx_c, fidx_nc, fidx_h, fidx_hn, fidx_o;
-    std::vector<long long> tp_c{0}, tp_nc{0}, tp_h{0}, tp_hn{0}, tp_o{0};
+    std::vector<int> fidx_c, fidx_nc, fidx_h, fidx_hn, fidx_o, fidx_on;
+    std::vector<long long> tp_c{0}, tp_nc{0}, tp_h{0}, tp_hn{0}, tp_o{0}, tp_on{0};
     for (int fi = 0; fi < (int)plan->fdev.size(); ++fi) {
       const FragDev& f = plan->fdev[fi];
       const long long t = (1ll << f.m) * (1ll << (2 * f.n_slots));
@@ -1049,8 +1051,10 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       else { fidx_nc.push_back(fi); tp_nc.push_back(tp_nc.back() + tf); }
       if (f.role == 1) { fidx_h.push_back(fi); tp_h.push_back(tp_h.back() + t); }
       if (f.role == 1 && !f.clifford) { fidx_hn.push_back(fi); tp_hn.push_back(tp_hn.back() + t); }
-      if (f.role == 2) { fidx_o.push_back(fi); tp_o.push_back(tp_o.back() + t); }
+      if (f.role == 2 && f.clifford) { fidx_o.push_back(fi); tp_o.push_back(tp_o.back() + t); }
+      if (f.role == 2 && !f.clifford) { fidx_on.push_back(fi); tp_on.push_back(tp_on.back() + t); }
     }
+    std::vector<long long> direct_per_m;       // floats per hub output of a star contracted leaf by leaf
     std::vector<int> tree_level, tree_small;   // launch level of every step (-1: in the small problems' CTA)
     for (auto& P : plan->problems) {
       ProblemDev d{};
@@ -1064,6 +1068,11 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       d.zexp_off = plan->n_zexp;
       plan->n_marg += 1ll << d.n_marg;
       plan->n_zexp += d.nz;
+      if (d.nz > 0) {
+        long long entries = 0;
+        for (int l = 0; l < d.n_frags; ++l) entries += 1ll << (2 * plan->fdev[f0 + l].n_slots);
+        if (entries > 128 || d.k > 3) plan->z_warp = false;
+      }
       plan->out_prefix.push_back(plan->n_marg);
       plan->z_prefix.push_back(plan->n_zexp);
       if (P.hub < 0) {          // not a star: fragment tensors contracted pair by pair
@@ -1139,9 +1148,8 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
           d.r_off = plan->r_total;
           d.part_off = plan->part_total;
           d.blk_off = plan->gemm_blocks;
-          for (int t = 0; t < d.mtiles; ++t) plan->direct_items.push_back(make_int2((int)plan->pdev.size(), t));
-          plan->direct_stage_floats =
-              std::max(plan->direct_stage_floats, std::max(tm * per_m, tm + (long long)d.N));
+          direct_per_m.resize(plan->pdev.size() + 1, 0);
+          direct_per_m.back() = per_m;
         }
         if (!d.direct) {
           const long long base = (long long)d.mtiles * d.ntiles;
@@ -1203,6 +1211,28 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       plan->pdev.push_back(d);
     }
 
+    // Stars contracted leaf by leaf: slices small enough for two CTAs per SM over
+    // the whole plan, but of at least 16 hub outputs (a 32-byte sector of an int16
+    // operand row).  The largest slice that fits shared memory left one
+    // 100-qubit circuit with four CTAs (24 us; 32 CTAs: 8 us).
+    {
+      long long outputs = 0;
+      for (auto& d : plan->pdev)
+        if (d.direct) outputs += d.M;
+      long long goal = 16;
+      while (2 * goal * 2 * std::max(c->sm_count, 148) <= outputs) goal *= 2;
+      for (size_t pi = 0; pi < plan->pdev.size(); ++pi) {
+        ProblemDev& d = plan->pdev[pi];
+        if (!d.direct) continue;
+        const long long per_m = direct_per_m[pi], tm = std::min<long long>(d.TM, goal);
+        d.TM = (int)tm;
+        d.mtiles = (int)(d.M / tm);
+        for (int t = 0; t < d.mtiles; ++t) plan->direct_items.push_back(make_int2((int)pi, t));
+        plan->direct_stage_floats =
+            std::max(plan->direct_stage_floats, std::max(tm * per_m, tm + (long long)d.N));
+      }
+    }
+
     // the tree contractions' launches: one per level over all problems, the last steps together at the end
     std::vector<std::vector<int>> tree_sets;
     for (size_t i = 0; i < plan->gsteps.size(); ++i)
@@ -1232,14 +1262,15 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     for (int s = 0; s < 4; ++s) { prep[s] = prep_op(s); prep_matrix(s, &prepm[8 * s]); }
     for (int b = 0; b < 3; ++b) { basis[b] = basis_op(b); basis_matrix(b, &basism[8 * b]); }
 
-    int *d_fidx_c, *d_fidx_nc, *d_fidx_h, *d_fidx_hn, *d_fidx_o;
-    long long *d_tp_c, *d_tp_nc, *d_tp_h, *d_tp_hn, *d_tp_o;
+    int *d_fidx_c, *d_fidx_nc, *d_fidx_h, *d_fidx_hn, *d_fidx_o, *d_fidx_on;
+    long long *d_tp_c, *d_tp_nc, *d_tp_h, *d_tp_hn, *d_tp_o, *d_tp_on;
     if (!c->host_only) {
       Staging st;
       st.add(fidx_c, &d_fidx_c); st.add(fidx_nc, &d_fidx_nc); st.add(tp_c, &d_tp_c);
       st.add(tp_nc, &d_tp_nc); st.add(fidx_h, &d_fidx_h); st.add(fidx_o, &d_fidx_o);
       st.add(tp_h, &d_tp_h); st.add(tp_o, &d_tp_o);
       st.add(fidx_hn, &d_fidx_hn); st.add(tp_hn, &d_tp_hn);
+      st.add(fidx_on, &d_fidx_on); st.add(tp_on, &d_tp_on);
       st.add(items_hub, &plan->d_items_hub); st.add(items_plain, &plan->d_items_plain);
       bool okf = st.commit(c, plan->A);
       if (!okf) { return fail(c, CCS_ERR_OOM, "plan upload failed"); }
@@ -1248,6 +1279,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       plan->fold_hubs = FoldSet{d_fidx_h, d_tp_h, (int)fidx_h.size(), tp_h.back()};
       plan->fold_hubs_nc = FoldSet{d_fidx_hn, d_tp_hn, (int)fidx_hn.size(), tp_hn.back()};
       plan->fold_others = FoldSet{d_fidx_o, d_tp_o, (int)fidx_o.size(), tp_o.back()};
+      plan->fold_others_nc = FoldSet{d_fidx_on, d_tp_on, (int)fidx_on.size(), tp_on.back()};
     }
     if (c->host_only) {
       plan->dp.n_items_cliff = (int)items_c.size();
@@ -1381,6 +1413,9 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
       return cuda_fail(c, err, "statevector kernel");
     stage_end(c, ST_STATEVEC);
     if ((err = launch_fold(dp, r->dr, e, p->fold_nc, s2)) != cudaSuccess) return cuda_fail(c, err, "fold kernel");
+    // the statevector leaves' contraction operands too, beside the Clifford branch
+    if ((err = launch_operands(dp, r->dr, e, FoldSet{nullptr, nullptr, 0, 0}, p->fold_others_nc, s2)) != cudaSuccess)
+      return cuda_fail(c, err, "operand kernels");
   }
   if (dp.n_items_cliff) {
     const int threads = r->cliff_threads;
@@ -1774,7 +1809,7 @@ int ccs_recombine(ccs_ctx c, ccs_plan p, ccs_res r, const ccs_recomb_opts* opts,
     cudaSetDevice(c->device);
     const bool stitched = r->ep.mode == CCS_STITCH;
     const bool tc = !(opts && opts->no_tensor_cores) && !stitched;   // stitched rows skip zeros on CUDA cores
-    RecombSizes rz{p->r_total, p->part_total, p->gemm_blocks, p->n_marg, p->n_zexp,
+    RecombSizes rz{p->r_total, p->part_total, p->gemm_blocks, p->n_marg, p->n_zexp, p->z_warp ? 1 : 0,
                    p->d_direct_items, (int)p->direct_items.size(), (int)p->direct_stage_floats, p->chain,
                    p->d_r_prefix, p->d_blk_prefix, p->d_out_prefix, p->d_z_prefix, p->max_tile_smem,
                    p->pdev.data(), (int)p->pdev.size(), r->rt_scratch, tc ? 1 : 0, stitched ? 1 : 0, KRange{0, -1},
@@ -2190,7 +2225,7 @@ extern "C" int ccs_recombine_noalloc(ccs_ctx c, ccs_plan p, ccs_res r, int preci
       }
       scratch = g_noalloc_addr[c->device];
     }
-    RecombSizes rz{p->r_total, p->part_total, p->gemm_blocks, p->n_marg, p->n_zexp,
+    RecombSizes rz{p->r_total, p->part_total, p->gemm_blocks, p->n_marg, p->n_zexp, p->z_warp ? 1 : 0,
                    p->d_direct_items, (int)p->direct_items.size(), (int)p->direct_stage_floats, p->chain,
                    p->d_r_prefix, p->d_blk_prefix, p->d_out_prefix, p->d_z_prefix, p->max_tile_smem,
                    p->pdev.data(), (int)p->pdev.size(), nullptr, 0, r->ep.mode == CCS_STITCH ? 1 : 0,

@@ -243,13 +243,20 @@ __device__ void prep_rows_from_body(const CliffordOp* s_prep, const int* s_qin, 
 // flight, its word fetched a moment earlier still.  Moments of at most 16 ops
 // run in a single warp with no block barrier.  A deep narrow body (301 wires,
 // 307 moments) took 790 cycles a moment with eight lanes per op, a shuffle
-// reduction and a barrier each; BODY_TIMES.
+// reduction and a barrier each: 117 us for 64 such bodies,
+// 43 us so; 86 wires in 20 moments: 15 and 7.7 us.
 namespace {
+// An op as the kernel stages it: x = the byte offsets of columns X_a (low half)
+// and X_b, y = M | sign form << 16 without the form's constant term.  Lanes
+// without an op take the idle one, on the all-zero dummy columns with all masks
+// zero, so that nothing branches.
+__device__ __forceinline__ uint2 stage_op(uint2 w) {
+  return make_uint2((w.x & 0xffffu) * 8u | ((w.x >> 16) * 8u) << 16, w.y & ~(1u << 16));
+}
 struct OpLane {          // one lane's part of an op
-  int a0, a1, a2, a3, out;               // column indices
+  uint32_t xa, xb, out;                  // byte offsets of X_a, X_b and of its output column
   uint32_t m0, m1, m2, m3;               // its row of the 4 x 4 matrix, as masks
   uint32_t q0, q1, q2, q3;               // its sign-flip terms
-  bool act;
 };
 // All ones where the top bit of byte SEL & 7 of x is set (prmt's sign-replicating
 // selectors): four masks from one shifted word.
@@ -258,19 +265,18 @@ __device__ __forceinline__ uint32_t sign_mask(uint32_t x, uint32_t sel) {
   asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "r"(sel));
   return r;
 }
-__device__ __forceinline__ void decode_op(uint2 w, bool act, int j, int zb, OpLane& d) {
-  const int qa = (int)(w.x & 0xffffu), qb = (int)(w.x >> 16);
+// sh, sm, sa: the lane's shift and byte selectors; zo: the byte offset from an X
+// to its Z column where lane j writes one, else 0.
+__device__ __forceinline__ OpLane decode_op(uint2 w, int j, uint32_t sh, uint32_t sm, uint32_t sa, uint32_t zo) {
+  OpLane d;
+  d.xa = w.x & 0xffffu;
+  d.xb = w.x >> 16;
+  d.out = ((j & 2) ? d.xb : d.xa) + zo;
   // bits 4 j + k of M and of the sign form: byte j / 2 of the word's halves, bit 4 (j & 1) + k
-  const uint32_t t = (w.y & ~(1u << 16)) << (4 - 4 * (j & 1));             // ANF term 0 is not used
-  const uint32_t sm = 0x8888u + 0x1111u * (uint32_t)(j >> 1), sa = sm + 0x2222u;
-  d.act = act;
-  d.a0 = qa;
-  d.a1 = zb + qa;
-  d.a2 = qb;
-  d.a3 = zb + qb;
-  d.out = ((j & 2) ? qb : qa) + ((j & 1) ? zb : 0);
+  const uint32_t t = w.y << sh;
   d.m0 = sign_mask(t << 3, sm); d.m1 = sign_mask(t << 2, sm); d.m2 = sign_mask(t << 1, sm); d.m3 = sign_mask(t, sm);
   d.q0 = sign_mask(t << 3, sa); d.q1 = sign_mask(t << 2, sa); d.q2 = sign_mask(t << 1, sa); d.q3 = sign_mask(t, sa);
+  return d;
 }
 // s2 / s3: all ones where the lane's terms do not contain v2 / v3.
 __device__ __forceinline__ void op_half(const OpLane& d, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, uint32_t s2,
@@ -280,7 +286,7 @@ __device__ __forceinline__ void op_half(const OpLane& d, uint32_t v0, uint32_t v
 }
 
 // A whole op by one thread: its 31 masks from the word's eight shifts.
-__device__ __forceinline__ void apply_whole(uint2 w, uint2* tab, int zb, uint2& rd) {
+__device__ __forceinline__ void apply_whole(uint2 w, char* tab, uint32_t zb8, uint2& rd) {
   uint32_t m[16], a[16];
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
@@ -290,8 +296,10 @@ __device__ __forceinline__ void apply_whole(uint2 w, uint2* tab, int zb, uint2& 
     a[7 - s] = sign_mask(t, 0xaaaau);
     a[15 - s] = sign_mask(t, 0xbbbbu);
   }
-  const int qa = (int)(w.x & 0xffffu), qb = (int)(w.x >> 16);
-  const uint2 V0 = tab[qa], V1 = tab[zb + qa], V2 = tab[qb], V3 = tab[zb + qb];
+  uint2 *pa = reinterpret_cast<uint2*>(tab + (w.x & 0xffffu)), *pb = reinterpret_cast<uint2*>(tab + (w.x >> 16));
+  uint2 *za = reinterpret_cast<uint2*>(reinterpret_cast<char*>(pa) + zb8);
+  uint2 *zz = reinterpret_cast<uint2*>(reinterpret_cast<char*>(pb) + zb8);
+  const uint2 V0 = *pa, V1 = *za, V2 = *pb, V3 = *zz;
   uint2 U[4];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -312,10 +320,73 @@ __device__ __forceinline__ void apply_whole(uint2 w, uint2* tab, int zb, uint2& 
       else U[i].x = u;
     }
   }
-  tab[qa] = U[0];
-  tab[zb + qa] = U[1];
-  tab[qb] = U[2];
-  tab[zb + qb] = U[3];
+  *pa = U[0];
+  *za = U[1];
+  *pb = U[2];
+  *zz = U[3];
+}
+
+// The op stream of one body applied to its word of every column (the sign words
+// summed into rd).  STAGED: ops and moment offsets (three sentinels behind them)
+// in shared memory, else both stay in global memory.
+template <int MODE, bool STAGED, class Sync>
+__device__ __forceinline__ void run_body(char* tab, int n, int nt, int n_mom, int n_ops, const uint2* ops, const int* mom,
+                                         uint2& rd, Sync sync) {
+  constexpr int PER = MODE == 2 ? 1 : 4;              // lanes of an op
+  const int tid = threadIdx.x, j = tid % PER, k0 = tid / PER, slots = nt / PER;
+  const uint32_t zb8 = 8u * (uint32_t)(n + 1);
+  const uint2 idle = make_uint2(8u * (uint32_t)n * 0x10001u, 0u);
+  auto fetch = [&](int o, int end) -> uint2 {
+    uint2 w = idle;
+    if (o < end) w = STAGED ? ops[o] : stage_op(ops[o]);
+    return w;
+  };
+  auto bound = [&](int mm) -> int { return STAGED ? mom[mm] : mm > n_mom ? n_ops : mom[mm]; };
+  int b0 = bound(0), b1 = bound(1), b2 = bound(2);
+  if (MODE == 2) {
+    uint2 raw = fetch(b0 + k0, b1);            // the next moment's op is fetched while this one's is applied
+    for (int mm = 0; mm < n_mom; ++mm) {
+      const uint2 now = raw;
+      raw = fetch(b1 + k0, b2);
+      if (b0 + k0 < b1) apply_whole(now, tab, zb8, rd);
+      for (int o = b0 + k0 + slots; o < b1; o += slots) apply_whole(fetch(o, b1), tab, zb8, rd);
+      b0 = b1;
+      b1 = b2;
+      b2 = bound(mm + 3);
+      sync();
+    }
+    return;
+  }
+  const uint32_t s2 = (j & 1) ? 0u : ~0u, s3 = (j & 2) ? 0u : ~0u, zo = (j & 1) ? zb8 : 0u;
+  const uint32_t sh = 4u - 4u * (uint32_t)(j & 1), sm = 0x8888u + 0x1111u * (uint32_t)(j >> 1), sa = sm + 0x2222u;
+  auto at = [&](uint32_t off) -> uint2& { return *reinterpret_cast<uint2*>(tab + off); };
+  char* ztab = tab + zb8;
+  auto zat = [&](uint32_t off) -> uint2& { return *reinterpret_cast<uint2*>(ztab + off); };
+  OpLane cur = decode_op(fetch(b0 + k0, b1), j, sh, sm, sa, zo);
+  uint2 raw = fetch(b1 + k0, b2);              // of the next moment
+  for (int mm = 0; mm < n_mom; ++mm) {
+    uint2 v0 = at(cur.xa), v1 = zat(cur.xa), v2 = at(cur.xb), v3 = zat(cur.xb), u;
+    const OpLane nxt = decode_op(raw, j, sh, sm, sa, zo);        // while the loads are in flight
+    const int b3 = bound(mm + 3);
+    raw = fetch(b2 + k0, b3);
+    __syncwarp();                              // an op's four lanes have read its columns
+    op_half(cur, v0.x, v1.x, v2.x, v3.x, s2, s3, u.x, rd.x);
+    op_half(cur, v0.y, v1.y, v2.y, v3.y, s2, s3, u.y, rd.y);
+    at(cur.out) = u;
+    for (int o = b0 + slots; o < b1; o += slots) {    // further ops of a wide moment
+      const OpLane d = decode_op(fetch(o + k0, b1), j, sh, sm, sa, zo);
+      v0 = at(d.xa); v1 = zat(d.xa); v2 = at(d.xb); v3 = zat(d.xb);
+      __syncwarp();
+      op_half(d, v0.x, v1.x, v2.x, v3.x, s2, s3, u.x, rd.x);
+      op_half(d, v0.y, v1.y, v2.y, v3.y, s2, s3, u.y, rd.y);
+      at(d.out) = u;
+    }
+    cur = nxt;
+    b0 = b1;
+    b1 = b2;
+    b2 = b3;
+    sync();
+  }
 }
 }  // namespace
 
@@ -341,15 +412,15 @@ __global__ void __launch_bounds__(MODE == 0 ? 32 : MODE == 1 ? 1024 : 256) body_
   // the op stream and moment offsets follow the column words when they fit
   const int* gmom = P.moments + F.mom_off;
   const int n_ops = gmom[n_mom];
-  const bool staged = ncol + n_ops + (n_mom + 2) / 2 + 1 <= smem_words;
+  const bool staged = ncol + n_ops + (n_mom + 5) / 2 + 1 <= smem_words;
   const uint2* gops = reinterpret_cast<const uint2*>(P.cops + F.ops_off);
   uint2* ops_s = tab + ncol;
   int* mom_s = reinterpret_cast<int*>(tab + ncol + n_ops);
   if (staged) {
 #pragma unroll 8
-    for (int i = tid; i < n_ops; i += nt) ops_s[i] = gops[i];
+    for (int i = tid; i < n_ops; i += nt) ops_s[i] = stage_op(gops[i]);
 #pragma unroll 4
-    for (int i = tid; i <= n_mom; i += nt) mom_s[i] = gmom[i];
+    for (int i = tid; i < n_mom + 4; i += nt) mom_s[i] = i <= n_mom ? gmom[i] : n_ops;
   }
   {   // identity: destabilizer i = X_i (words [0, Wh)), stabilizer i = Z_i
     const int half = w < Wh ? 0 : 1, c0 = (half ? zb : 0) + 64 * (w - half * Wh), cn = (half ? zb : 0) + n;
@@ -360,67 +431,9 @@ __global__ void __launch_bounds__(MODE == 0 ? 32 : MODE == 1 ? 1024 : 256) body_
     }
   }
   sync();
-  const int j = tid % PER, k0 = tid / PER, slots = nt / PER;
-  const uint32_t s2 = (j & 1) ? 0u : ~0u, s3 = (j & 2) ? 0u : ~0u;
-  auto fetch = [&](int o, int end) -> uint2 {
-    if (o >= end) return make_uint2(0u, 0u);
-    return staged ? ops_s[o] : gops[o];
-  };
-  auto bound = [&](int mm) -> int { return mm > n_mom ? n_ops : staged ? mom_s[mm] : gmom[mm]; };
   uint2 rd = make_uint2(0u, 0u);
-  auto apply = [&](const OpLane& d) {
-    uint2 v0, v1, v2, v3, u;
-    if (d.act) { v0 = tab[d.a0]; v1 = tab[d.a1]; v2 = tab[d.a2]; v3 = tab[d.a3]; }
-    __syncwarp();                              // an op's four lanes have read its columns
-    if (d.act) {
-      op_half(d, v0.x, v1.x, v2.x, v3.x, s2, s3, u.x, rd.x);
-      op_half(d, v0.y, v1.y, v2.y, v3.y, s2, s3, u.y, rd.y);
-      tab[d.out] = u;
-    }
-  };
-  if (MODE == 2) {
-    int b0 = bound(0), b1 = bound(1);
-    uint2 raw = fetch(b0 + k0, b1);            // the next moment's op word is fetched while this one's is applied
-    for (int mm = 0; mm < n_mom; ++mm) {
-      const int b2 = bound(mm + 2);
-      const uint2 now = raw;
-      raw = fetch(b1 + k0, b2);
-      if (b0 + k0 < b1) apply_whole(now, tab, zb, rd);
-      for (int o = b0 + k0 + slots; o < b1; o += slots) apply_whole(fetch(o, b1), tab, zb, rd);
-      b0 = b1;
-      b1 = b2;
-      sync();
-    }
-  } else if (n_mom > 0) {
-    int b0 = bound(0), b1 = bound(1), b2 = bound(2);
-    OpLane cur;
-    decode_op(fetch(b0 + k0, b1), b0 + k0 < b1, j, zb, cur);
-    uint2 raw = fetch(b1 + k0, b2);            // of the next moment
-    for (int mm = 0; mm < n_mom; ++mm) {
-      uint2 v0, v1, v2, v3, u;
-      if (cur.act) { v0 = tab[cur.a0]; v1 = tab[cur.a1]; v2 = tab[cur.a2]; v3 = tab[cur.a3]; }
-      OpLane nxt;                              // decoded while the loads are in flight
-      decode_op(raw, b1 + k0 < b2, j, zb, nxt);
-      const int b3 = bound(mm + 3);
-      raw = fetch(b2 + k0, b3);
-      __syncwarp();                            // an op's four lanes have read its columns
-      if (cur.act) {
-        op_half(cur, v0.x, v1.x, v2.x, v3.x, s2, s3, u.x, rd.x);
-        op_half(cur, v0.y, v1.y, v2.y, v3.y, s2, s3, u.y, rd.y);
-        tab[cur.out] = u;
-      }
-      for (int o = b0 + slots; o < b1; o += slots) {    // further ops of a wide moment
-        OpLane d;
-        decode_op(fetch(o + k0, b1), o + k0 < b1, j, zb, d);
-        apply(d);
-      }
-      cur = nxt;
-      b0 = b1;
-      b1 = b2;
-      b2 = b3;
-      sync();
-    }
-  }
+  if (staged) run_body<MODE, true>(reinterpret_cast<char*>(tab), n, nt, n_mom, n_ops, ops_s, mom_s, rd, sync);
+  else run_body<MODE, false>(reinterpret_cast<char*>(tab), n, nt, n_mom, n_ops, gops, gmom, rd, sync);
   for (int o = 16; o; o >>= 1) {
     rd.x ^= __shfl_xor_sync(0xffffffffu, rd.x, o);
     rd.y ^= __shfl_xor_sync(0xffffffffu, rd.y, o);
@@ -756,7 +769,7 @@ __device__ __forceinline__ unsigned echelon_body(const unsigned long long* body,
 // the quantum inputs, and the parities popc(b_k & a_r) mod 2 for every
 // record k, so that the phase of any product of records needs no vectors.
 constexpr int kMaxRecords = 64;    // measurement records of a fragment: m + 3 qout (m + qout <= 24, qout <= 12)
-__global__ void __launch_bounds__(256) body_basis_kernel(DevPlan P, DevRes R) {
+__global__ void __launch_bounds__(256, 4) body_basis_kernel(DevPlan P, DevRes R) {
   __shared__ unsigned long long s_eb[8][64];
   __shared__ unsigned long long s_eh[8];
   __shared__ int s_col[64];
@@ -1007,24 +1020,29 @@ __global__ void __launch_bounds__(256) screen_kernel(DevPlan P, DevRes R, EvalPa
       absorb(((sh >> lane) & 1ull) ? project(rb[lane]) : 0u);
       if (sh >> 32) absorb(((sh >> (lane + 32)) & 1ull) ? project(rb[lane + 32]) : 0u);
     }
-    {   // new stabilizer rows of the quantum inputs (bits only): the image of
-        // C Z C^+ is D, S or their product, from the fragment's input rows
-      uint32_t row = 0;
-      if (lane < F.qin) {
-        const unsigned s = (pin >> (2 * lane)) & 3u;
-        const int sc = s < 2 ? 2 : s == 2 ? 1 : 3;   // image of Z under the preparation: 1 X, 2 Z, 3 Y
-        const unsigned long long e = ((sc & 1) ? rb[kRbInputRows + lane] : 0ull) ^
-                                     ((sc & 2) ? rb[kRbInputRows + kMaxCuts + lane] : 0ull);
-        row = project(e);
+    // full rank already: the whole space whatever the inputs prepare (reduced
+    // basis = unit vectors); most variants of scrambling circuits end here
+    uint32_t vec = lane < nA ? 1u << lane : 0u;
+    if (have != (nA >= 32 ? ~0u : (1u << nA) - 1u)) {
+      {   // new stabilizer rows of the quantum inputs (bits only): the image of
+          // C Z C^+ is D, S or their product, from the fragment's input rows
+        uint32_t row = 0;
+        if (lane < F.qin) {
+          const unsigned s = (pin >> (2 * lane)) & 3u;
+          const int sc = s < 2 ? 2 : s == 2 ? 1 : 3;   // image of Z under the preparation: 1 X, 2 Z, 3 Y
+          const unsigned long long e = ((sc & 1) ? rb[kRbInputRows + lane] : 0ull) ^
+                                       ((sc & 2) ? rb[kRbInputRows + kMaxCuts + lane] : 0ull);
+          row = project(e);
+        }
+        absorb(row);
       }
-      absorb(row);
-    }
-    // reduced form in pivot order; non-pivot bits' relations by ballot
-    uint32_t vec = ((have >> lane) & 1u) ? mine : 0u;
-    for (int q = nA - 1; q > 0; --q) {
-      if (!((have >> q) & 1u)) continue;
-      const uint32_t bq = __shfl_sync(FULLW, vec, q);
-      if (lane < q && ((vec >> q) & 1u)) vec ^= bq;
+      // reduced form in pivot order; non-pivot bits' relations by ballot
+      vec = ((have >> lane) & 1u) ? mine : 0u;
+      for (int q = nA - 1; q > 0; --q) {
+        if (!((have >> q) & 1u)) continue;
+        const uint32_t bq = __shfl_sync(FULLW, vec, q);
+        if (lane < q && ((vec >> q) & 1u)) vec ^= bq;
+      }
     }
     const int rank = __popc(have);
     uint32_t off = 0;

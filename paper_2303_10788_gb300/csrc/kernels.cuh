@@ -305,6 +305,7 @@ struct KRange {
 
 struct RecombSizes {
   long long r_total, part_total, gemm_blocks, out_total, z_total;
+  int z_warp;                    // 1: every problem with Z-strings is small enough for a warp per string
   const int2* direct_items;      // (problem, hub-output slice) contracted leaf by leaf, one CTA each
   int n_direct;
   int direct_stage_floats;       // floats of each of the two intermediate buffers

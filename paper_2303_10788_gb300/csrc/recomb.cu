@@ -69,6 +69,30 @@ __device__ __forceinline__ void for_each_prep(const FragDev& F, const PauliSplit
   }
 }
 
+// The same tuples for at most two inputs as nine fixed slots (input 0 fastest, in
+// for_each_prep's order): coef 0 marks an absent one.  The slots' loads do not
+// wait for one another, and the coefficients are signed powers of two, so that
+// coef times a value is exact in FP32.
+__device__ __forceinline__ void prep_slots(const FragDev& F, const PauliSplit& ps, int (&vin)[9], float (&coef)[9]) {
+#pragma unroll
+  for (int t = 0; t < 9; ++t) { vin[t] = 0; coef[t] = 1.f; }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int P = i < F.qin ? ps.pin[i] : -1;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const int c = i == 0 ? t % 3 : t / 3;
+      int s = 0;
+      float w;
+      if (P < 0) w = c == 0 ? 1.f : 0.f;                       // no such input
+      else if (P == 0 || P == 3) { s = c; w = c == 2 ? 0.f : (P == 3 && c == 1) ? -1.f : 1.f; }
+      else { s = c == 0 ? P + 1 : c - 1; w = c == 0 ? 2.f : -1.f; }
+      vin[t] += s << (2 * i);
+      coef[t] *= w;
+    }
+  }
+}
+
 __device__ __forceinline__ float to_bf16f(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 // sum += p with the low part the rounding loses kept in comp (Neumaier)
 __device__ __forceinline__ void neumaier(float& sum, float& comp, float p) {
@@ -101,7 +125,35 @@ __global__ void fold_kernel(DevPlan P, DevRes R, EvalParams E, const int* fidx, 
     const bool use_counts = F.clifford && E.mode == CCS_SAMPLED;
     const int m = F.m, nA = F.nA;
     double acc = 0.0;
-    for_each_prep(F, ps, [&](int vin, double coef) {
+    if (F.qin <= 2 && F.qout <= 1 && (!use_counts || E.shots < (1u << 24))) {     // every load in flight at once, added in the same order
+      int vin[9];
+      float coef[9], val[9][2];
+      prep_slots(F, ps, vin, coef);
+      const bool two = F.qout == 1, flip = two && ps.pout[0] != 0;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        const long long y = ((vin[t] + (long long)vstride * vout) << nA) | o;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          val[t][b] = 0.f;
+          if (coef[t] != 0.f && (b == 0 || two)) {
+            const long long yb = y | ((long long)b << m);
+            if (use_counts) val[t][b] = (float)R.counts[F.counts_off + yb];      // exact below 2^24 shots
+            else val[t][b] = R.dist[F.dist_off + yb];
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        if (coef[t] == 0.f) continue;
+        const double c0 = use_counts ? (double)coef[t] * ((double)val[t][0] * E.inv_shots) : (double)(coef[t] * val[t][0]);
+        acc += c0;
+        if (two) {
+          const double c1 = use_counts ? (double)coef[t] * ((double)val[t][1] * E.inv_shots) : (double)(coef[t] * val[t][1]);
+          acc += flip ? -c1 : c1;
+        }
+      }
+    } else for_each_prep(F, ps, [&](int vin, double coef) {
       const long long v = vin + (long long)vstride * vout;
       for (int b = 0; b < (1 << F.qout); ++b) {
         int neg = 0;
@@ -995,7 +1047,7 @@ __device__ __forceinline__ long long spread(long long v, int nd, const uint8_t* 
 // the per-element loops below do no dependent global loads.
 constexpr int kMaxProblemFrags = kMaxProblemFragments;   // checked when the plan is built
 constexpr int kLeafStage = 2048;   // floats of a leaf table staged in shared memory
-static_assert(2 * kZTree <= kLeafStage, "the Z-string tensors of a tree share the leaf table's space");
+static_assert(2 * kZTree <= kLeafStage && 16 * 128 <= kLeafStage, "the Z-string tensors of a tree share the leaf table's space");
 struct ProblemShared {
   int nf, hub, k;
   int m[kMaxProblemFrags], ns[kMaxProblemFrags];
@@ -1004,16 +1056,17 @@ struct ProblemShared {
   long long T_off[kMaxProblemFrags];
 };
 
+// A warp per fragment, a lane per array entry (at least as many warps as fragments).
 __device__ void load_problem(const DevPlan& P, const ProblemDev& Pb, ProblemShared& S) {
-  const int t = threadIdx.x;
-  if (t == 0) { S.nf = Pb.n_frags; S.hub = Pb.hub; S.k = Pb.k; }
-  if (t < Pb.n_frags) {
-    const FragDev& L = P.frags[Pb.frag0 + t];
-    S.m[t] = L.m;
-    S.ns[t] = L.n_slots;
-    S.T_off[t] = L.T_off;
-    for (int i = 0; i < L.n_slots; ++i) S.slot_cut[t][i] = L.slot_cut[i];
-    for (int j = 0; j < L.m; ++j) S.marg_pos[t][j] = L.marg_pos[j];
+  const int l = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) { S.nf = Pb.n_frags; S.hub = Pb.hub; S.k = Pb.k; }
+  for (int f = l; f < Pb.n_frags; f += blockDim.x >> 5) {
+    const FragDev& L = P.frags[Pb.frag0 + f];
+    if (lane < kMaxCuts) S.slot_cut[f][lane] = L.slot_cut[lane];
+    if (lane < kMaxMarginal) S.marg_pos[f][lane] = L.marg_pos[lane];
+    if (lane == 24) S.m[f] = L.m;
+    if (lane == 25) S.ns[f] = L.n_slots;
+    if (lane == 26) S.T_off[f] = L.T_off;
   }
 }
 
@@ -1041,6 +1094,20 @@ __device__ float fold_z_value(const DevRes& R, const FragDev& F, int zi, int Pi)
   int vstride = 1;
   for (int i = 0; i < F.qin; ++i) vstride *= 4;
   double acc = 0.0;
+  if (F.qin <= 2) {      // every load in flight at once, added in the same order
+    int vin[9];
+    float coef[9], val[9];
+    prep_slots(F, ps, vin, coef);
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+      val[t] = coef[t] != 0.f
+                   ? R.zval[F.zval_off + ((vin[t] + (long long)vstride * vout) * F.nz + zi) * (1 << F.qout) + u]
+                   : 0.f;
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+      if (coef[t] != 0.f) acc += (double)(coef[t] * val[t]);
+    return (float)acc;
+  }
   for_each_prep(F, ps, [&](int vin, double coef) {
     const long long v = vin + (long long)vstride * vout;
     acc += coef * (double)R.zval[F.zval_off + (v * F.nz + zi) * (1 << F.qout) + u];
@@ -1106,13 +1173,50 @@ __device__ __noinline__ void z_string_block(const DevPlan& P, const DevRes& R, c
     }
     part += (double)t;
   }
-  red[threadIdx.x] = part;
+  for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
   __syncthreads();
-  for (int s = blockDim.x / 2; s; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    double v = (int)threadIdx.x < (int)(blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) zexp_out[Pb.zexp_off + zi] = ldexp(v, -S.k);
   }
-  if (threadIdx.x == 0) zexp_out[Pb.zexp_off + zi] = ldexp(red[0], -S.k);
+}
+
+// The same by one warp per string, for problems whose fragments have at most
+// kZWarp string entries in all (k <= 3): sixteen strings a CTA and no barrier.
+// (A CTA per string spent 20 k cycles in barriers and one chain of loads;
+// 512 strings of 64 circuits: Z_TIMES.)
+constexpr int kZWarp = 128;
+__device__ __noinline__ void z_string_warp(const DevPlan& P, const DevRes& R, const long long* prefix, int np, long long g,
+                                           float* s_tz, double* zexp_out, KRange kr) {
+  const int lane = threadIdx.x & 31, pi = find_seg(prefix, np, g);
+  const ProblemDev& Pb = P.problems[pi];
+  const int zi = (int)(g - prefix[pi]), nf = Pb.n_frags;
+  int tot = 0;
+  for (int l = 0; l < nf; ++l) tot += 1 << (2 * P.frags[Pb.frag0 + l].n_slots);
+  for (int i = lane; i < tot; i += 32) {
+    int l = 0, o = 0;
+    for (int d; i >= o + (d = 1 << (2 * P.frags[Pb.frag0 + l].n_slots)); ++l) o += d;
+    s_tz[i] = fold_z_value(R, P.frags[Pb.frag0 + l], zi, i - o);
+  }
+  __syncwarp();
+  const long long K = 1ll << (2 * Pb.k);
+  double part = 0.0;
+  for (long long Pp = kr.lo_of(K) + lane; Pp < kr.hi_of(K); Pp += 32) {
+    float t = 1.f;
+    int o = 0;
+    for (int l = 0; l < nf; ++l) {
+      const FragDev& L = P.frags[Pb.frag0 + l];
+      int pl = 0;
+      for (int j = 0; j < L.n_slots; ++j) pl |= (int)((Pp >> (2 * L.slot_cut[j])) & 3) << (2 * j);
+      t *= s_tz[o + pl];
+      o += 1 << (2 * L.n_slots);
+    }
+    part += (double)t;
+  }
+  for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if (lane == 0) zexp_out[Pb.zexp_off + zi] = ldexp(part, -Pb.k);
 }
 
 // Contraction of a star leaf by leaf (the tensor-network order of Sec.
@@ -1141,7 +1245,7 @@ __device__ __forceinline__ float hub_elem(const int16_t* A, float sc, long long 
 // (every operand load used twice), four rows in flight.
 template <class T> constexpr int first_vec() { return sizeof(T) == 2 ? 4 : 2; }   // hub outputs per thread
 constexpr int kFirstX = 2;      // leaf outputs per thread (1 or 2)
-constexpr int kFirstRows = 4;   // operand rows in flight per thread (divides 4^slots)
+constexpr int kFirstRows = 8;   // operand rows in flight per thread
 template <int VW, int NX, class T, class Expand>
 __device__ __forceinline__ void first_leaf_global(const T* __restrict__ At, float sc, int bf16, long long Mfull,
                                                   int lm, int lG, int ml, int lrest, long long klo, long long khi,
@@ -1160,24 +1264,25 @@ __device__ __forceinline__ void first_leaf_global(const T* __restrict__ At, floa
 #pragma unroll
     for (int v = 0; v < VW; ++v) { s0[v] = c0[v] = 0.f; if (NX == 2) s1[v] = c1[v] = 0.f; }
     const T* base = At + mv * VW;
-    for (int g0 = 0; g0 < G; g0 += kFirstRows) {      // G = 4^slots >= 4 (a leaf without cuts is staged)
+    for (int g0 = 0; g0 < G; g0 += kFirstRows) {      // G = 4^slots: 4, or a multiple of 8
       using Raw = typename RawVec<T, VW>::type;
       Raw a[kFirstRows];
 #pragma unroll
       for (int u = 0; u < kFirstRows; ++u) {
         const int g = g0 + u;
         int kg;
-        if (kg_tab) kg = kg_tab[g];
+        if (kg_tab) kg = g < G ? kg_tab[g] : 0;
         else {
           kg = 0;
           for (int i = 0; i < S.ns[l]; ++i) kg |= ((g >> (2 * i)) & 3) << (2 * S.slot_cut[l][i]);
         }
         const long long kk = (long long)(kr | kg);
-        a[u] = (kk >= klo && kk < khi) ? __ldg(reinterpret_cast<const Raw*>(base + kk * Mfull)) : Raw{};
+        a[u] = (g < G && kk >= klo && kk < khi) ? __ldg(reinterpret_cast<const Raw*>(base + kk * Mfull)) : Raw{};
       }
 #pragma unroll
       for (int u = 0; u < kFirstRows; ++u) {
         const int g = g0 + u;
+        if (g >= G) break;                              // G = 4: half a batch
         float t0 = tv[x0 * G + g], t1 = nx == 2 ? tv[(x0 + 1) * G + g] : 0.f;
         if (bf16 && !tv_rounded) { t0 = to_bf16f(t0); t1 = to_bf16f(t1); }
 #pragma unroll
@@ -1209,17 +1314,24 @@ __device__ __forceinline__ void contract_item(const DevPlan& P, const DevRes& R,
   __syncthreads();
   float* X = s_buf;
   float* Y = s_buf + stage_floats;
+  // cut positions of the digits in leaf order (four bits each, the first leaf's
+  // lowest), and each leaf's first digit
+  unsigned long long digits = 0ull;
+  {
+    int nd = 0;
+    for (int l = 0; l < S.nf; ++l) {
+      if (l == S.hub) continue;
+      for (int i = 0; i < S.ns[l]; ++i) digits |= (unsigned long long)S.slot_cut[l][i] << (4 * nd++);
+    }
+  }
   // compact cut index (groups in leaf order, the first leaf's lowest) ->
   // cut index, for the digits of leaves from `from` on
   auto expand = [&](int kc, int from) -> int {
-    int k = 0, rem = kc;
-    for (int l = from; l < S.nf; ++l) {
-      if (l == S.hub) continue;
-      for (int i = 0; i < S.ns[l]; ++i) {
-        k |= (rem & 3) << (2 * S.slot_cut[l][i]);
-        rem >>= 2;
-      }
-    }
+    unsigned long long ps = digits;
+    for (int l = 0; l < from; ++l)
+      if (l != S.hub) ps >>= 4 * S.ns[l];
+    int k = 0;
+    for (int rem = kc; rem; rem >>= 2, ps >>= 4) k |= (rem & 3) << (2 * (int)(ps & 15ull));
     return k;
   };
   int first = 0;
@@ -1332,13 +1444,21 @@ __device__ __forceinline__ void contract_item(const DevPlan& P, const DevRes& R,
 
 __global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, int precision,
                                                       const int2* direct_items, int n_direct, int stage_floats,
-                                                      const long long* z_prefix, int np, long long z_total,
+                                                      const long long* z_prefix, int np, long long z_total, int z_warp,
                                                       double* marg_out, double* zexp_out, KRange krg) {
   extern __shared__ __align__(16) float s_buf[];   // two buffers of stage_floats
   __shared__ double red[512];
   __shared__ ProblemShared S;
   __shared__ __align__(8) float s_T[kLeafStage];
-  for (long long b = blockIdx.x; b < n_direct + z_total; b += gridDim.x) {
+  const long long z_blocks = z_warp ? (z_total + 15) / 16 : z_total;
+  for (long long b = blockIdx.x; b < n_direct + z_blocks; b += gridDim.x) {
+    if (b >= n_direct && z_warp) {
+      const int w = threadIdx.x >> 5;
+      const long long g = (b - n_direct) * 16 + w;
+      if (g < z_total) z_string_warp(P, R, z_prefix, np, g, s_T + w * kZWarp, zexp_out, krg);
+      __syncthreads();
+      continue;
+    }
     if (b >= n_direct) {
       z_string_block(P, R, z_prefix, np, b - n_direct, S, red, s_T, kLeafStage, zexp_out, krg);
       __syncthreads();
@@ -1567,7 +1687,7 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
     note_launch();
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  const long long blocks = z.n_direct + z.z_total;
+  const long long blocks = z.n_direct + (z.z_warp ? (z.z_total + 15) / 16 : z.z_total);
   if (blocks > 0) {
     const size_t smem = (size_t)z.direct_stage_floats * 2 * 4;
     if (smem > 48 * 1024) {
@@ -1576,7 +1696,7 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
     }
     contract_kernel<<<(unsigned)(blocks < 65535ll * 16 ? blocks : 65535ll * 16), 512, smem, s>>>(
         p, r, precision, z.direct_items, z.n_direct, z.direct_stage_floats, z.z_prefix, p.n_problems, z.z_total,
-        marg_out, zexp_out, z.krange);
+        z.z_warp, marg_out, zexp_out, z.krange);
     note_launch();
     err = cudaGetLastError();
   }
