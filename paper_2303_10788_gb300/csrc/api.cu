@@ -1407,7 +1407,8 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
   }
   if (dp.n_items_nc) {
     int grid = std::min(dp.n_items_nc, c->sm_count * 4);
-    int threads = std::min(512, std::max(32, 1 << p->max_nc_n));   // one output amplitude per thread
+    // one group of four amplitudes per thread, or an amplitude in small states
+    int threads = p->max_nc_n <= 8 ? std::max(32, 1 << p->max_nc_n) : std::min(512, (1 << p->max_nc_n) / 4);
     stage_begin(c, ST_STATEVEC);
     if ((err = launch_statevector(dp, r->dr, p->max_nc_n, threads, grid, s2)) != cudaSuccess)
       return cuda_fail(c, err, "statevector kernel");
