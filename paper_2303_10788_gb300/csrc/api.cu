@@ -1211,16 +1211,24 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       plan->pdev.push_back(d);
     }
 
-    // Stars contracted leaf by leaf: slices small enough for two CTAs per SM over
-    // the whole plan, but of at least 16 hub outputs (a 32-byte sector of an int16
-    // operand row).  The largest slice that fits shared memory left one
-    // 100-qubit circuit with four CTAs (24 us; 32 CTAs: 8 us).
+    // Z-strings by warps once there are more of them than SMs: below that a CTA each
+    // has the shorter chain (contraction kernel with a CTA and with a warp per string:
+    // 16 strings 8.9 and 9.9 us, 128 9.5 and 10.1, 160 10.0 both, 256 15.5 and 10.4,
+    // 512 17.7 and 10.4 us).
+    if (plan->n_zexp <= std::max(c->sm_count, 148)) plan->z_warp = false;
+
+    // Stars contracted leaf by leaf: the largest slices that fit shared memory, cut
+    // (to 16 hub outputs at least, a 32-byte sector of an int16 operand row) until
+    // the plan has about 64 CTAs.  Every CTA builds its leaves' operands again, so
+    // smaller slices only pay while most of the chip idles (kernel times: one
+    // 100-qubit circuit 18.7 us with the largest slices, 10.4 us with 64 CTAs;
+    // 32 circuits 26 us so, 46 us with two CTAs per SM; 64 wide hubs 10.5 and 20 us).
     {
       long long outputs = 0;
       for (auto& d : plan->pdev)
         if (d.direct) outputs += d.M;
       long long goal = 16;
-      while (2 * goal * 2 * std::max(c->sm_count, 148) <= outputs) goal *= 2;
+      while (2 * goal * 64 <= outputs) goal *= 2;
       for (size_t pi = 0; pi < plan->pdev.size(); ++pi) {
         ProblemDev& d = plan->pdev[pi];
         if (!d.direct) continue;
