@@ -739,14 +739,30 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     plan->A.ctx = c;
     std::string err;
     // Per problem, on host threads: parse, cut search (if asked), fragment
-    // and compile.  Results are joined in problem order, so the plan does not
-    // depend on the thread count.
+    // and compile, in one go unless the learned choice comes in between.
+    // Results are joined in problem order, so the plan does not depend on the
+    // thread count.  The gate lists go where they were made (kept until
+    // then, freeing the plan of 16 circuits took 79 us on one thread).
     const int np = n_problems;
     std::vector<Problem> pr(np);
     std::vector<std::vector<Frag>> pf(np);
     std::vector<std::vector<CutCandidate>> pc(np);
-    std::vector<int> prc(np, CCS_OK);
+    std::vector<int> prc(np, CCS_OK), frc(np, CCS_OK);
     std::vector<std::string> perr(np);
+    auto fragment = [&](int pi) {
+      frc[pi] = fragment_problem(pr[pi], pi, pf[pi], perr[pi]);
+      if (frc[pi] != CCS_OK) return;
+      for (auto& f : pf[pi]) {
+        if (f.clifford) compile_clifford(f);
+        else compile_nc(f);
+        decltype(f.gates)().swap(f.gates);
+        decltype(f.gparam)().swap(f.gparam);
+      }
+      decltype(pr[pi].gates)().swap(pr[pi].gates);
+      decltype(pr[pi].gparam)().swap(pr[pi].gparam);
+    };
+    // the learned choice runs the scorer on the GPU: one problem at a time
+    const bool learned = o.use_learned && c->cut_model && !c->host_only;
     parallel_for(np, [&](int pi) {
       const ccs_problem& q = probs[pi];
       Problem& P = pr[pi];
@@ -770,11 +786,11 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
         if (prc[pi] != CCS_OK) return;
         P.cuts = pc[pi].front().cuts;
       }
+      if (!learned) fragment(pi);
     });
     for (int pi = 0; pi < np; ++pi)
       if (prc[pi] != CCS_OK) { return fail(c, prc[pi], perr[pi]); }
-    // the learned choice runs the scorer on the GPU: one problem at a time
-    if (o.use_learned && c->cut_model && !c->host_only)
+    if (learned) {
       for (int pi = 0; pi < np; ++pi)
         if (pc[pi].size() > 1) {
           int pick = 0;
@@ -782,16 +798,10 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
           if (rc != CCS_OK) { return rc; }
           pr[pi].cuts = pc[pi][pick].cuts;
         }
-    parallel_for(np, [&](int pi) {
-      prc[pi] = fragment_problem(pr[pi], pi, pf[pi], perr[pi]);
-      if (prc[pi] != CCS_OK) return;
-      for (auto& f : pf[pi]) {
-        if (f.clifford) compile_clifford(f);
-        else compile_nc(f);
-      }
-    });
+      parallel_for(np, fragment);
+    }
     for (int pi = 0; pi < np; ++pi)
-      if (prc[pi] != CCS_OK) { return fail(c, prc[pi], "problem " + std::to_string(pi) + ": " + perr[pi]); }
+      if (frc[pi] != CCS_OK) { return fail(c, frc[pi], "problem " + std::to_string(pi) + ": " + perr[pi]); }
     for (int pi = 0; pi < np; ++pi) {
       const int base = (int)plan->frags.size();      // fragment ids become plan-global
       for (auto& id : pr[pi].frag_ids) id += base;
@@ -809,23 +819,22 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     int img_words_max = 0, body_words_max = 0;
     int max_body_stage = 0, max_moment_ops = 1;
     int max_body_cols = 0;
-    std::vector<long long> cost_c, cost_nc;
+    // a fragment's items (variants, or preparations) are consecutive and cost the same
+    struct Run { int frag, first, count; long long cost; };
+    std::vector<Run> runs_c, runs_nc;
     {   // sizes first: every array below is filled without reallocation
-      size_t n_cops = 0, n_nops = 0, n_mom = 0, n_var = 0, n_wire = 0;
+      size_t n_cops = 0, n_nops = 0, n_mom = 0, n_wire = 0;
       for (const Frag& f : plan->frags) {
         n_cops += f.cops.size();
         n_nops += f.nops.size();
         n_mom += f.moment_start.size();
         n_wire += 2 * f.qout_wire.size() + f.marg_wire.size() + f.qin_wire.size();
         for (auto& zw : f.zwires) n_wire += zw.size();
-        if (f.clifford) n_var += f.n_variants();
       }
       cops.reserve(n_cops);
       nops.reserve(n_nops);
       moments.reserve(n_mom);
       wires.reserve(n_wire);
-      items_c.reserve(n_var);
-      cost_c.reserve(n_var);
       plan->fdev.reserve(plan->frags.size());
     }
     for (size_t fi = 0; fi < plan->frags.size(); ++fi) {
@@ -908,10 +917,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
         plan->cliff_smem_words =
             std::max(plan->cliff_smem_words, (size_t)staged * 8 <= c->smem_optin ? staged : words);
         plan->body_smem_words = std::max(plan->body_smem_words, words);
-        for (int v = 0; v < d.nv; ++v) {
-          items_c.push_back(make_int2((int)fi, v));
-          cost_c.push_back((long long)d.W * (d.n_moments + 4) * std::max(1, d.n / 16) + d.nz * 4 + d.nA * d.n);
-        }
+        runs_c.push_back({(int)fi, 0, d.nv, (long long)d.W * (d.n_moments + 4) * std::max(1, d.n / 16) + d.nz * 4 + d.nA * d.n});
       } else {
         d.space_off = d.counts_off = d.tab_off = d.body_off = d.rb_off = d.zimg_off = d.pb_off = -1;
         plan->max_nc_n = std::max(plan->max_nc_n, d.n);
@@ -933,28 +939,18 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     }
     // a per-variant tableau (kept tableaus, per-variant bodies) must fit in
     // shared memory; the shared-body path has no such limit (checked at evaluation)
-    plan->tableau_fits = (size_t)plan->cliff_smem_words * 8 <= c->smem_optin || items_c.empty();
-    // Items costliest first, ties in insertion order.  A fragment's items are
-    // consecutive and cost the same, so the runs of equal cost are sorted
-    // stably instead of the items (the same order, far fewer comparisons).
-    auto sort_items = [](std::vector<int2>& it, std::vector<long long>& cost) {
-      std::vector<std::pair<size_t, size_t>> runs;
-      for (size_t i = 0; i < it.size();) {
-        size_t j = i + 1;
-        while (j < it.size() && cost[j] == cost[i]) ++j;
-        runs.push_back({i, j});
-        i = j;
-      }
-      std::stable_sort(runs.begin(), runs.end(),
-                       [&](const std::pair<size_t, size_t>& a, const std::pair<size_t, size_t>& b) {
-                         return cost[a.first] > cost[b.first];
-                       });
-      std::vector<int2> out;
-      out.reserve(it.size());
-      for (auto& r : runs) out.insert(out.end(), it.begin() + r.first, it.begin() + r.second);
-      it.swap(out);
+    plan->tableau_fits = (size_t)plan->cliff_smem_words * 8 <= c->smem_optin || runs_c.empty();
+    // Items costliest first, ties in insertion order: the runs are sorted, then spread out.
+    auto spread = [](std::vector<Run>& runs, std::vector<int2>& it) {
+      std::stable_sort(runs.begin(), runs.end(), [](const Run& a, const Run& b) { return a.cost > b.cost; });
+      size_t n = 0;
+      for (auto& r : runs) n += r.count;
+      it.resize(n);
+      int2* o = it.data();
+      for (auto& r : runs)
+        for (int i = 0; i < r.count; ++i) *o++ = make_int2(r.frag, r.first + i);
     };
-    sort_items(items_c, cost_c);
+    spread(runs_c, items_c);
     // Non-Clifford items: with enough variants to fill the GPU, one item per
     // preparation combination (the gates run once, every basis combination of
     // the outputs is applied to a copy of the state); otherwise one per variant
@@ -969,13 +965,10 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
         const int n_prep = 1 << (2 * d.qin), n_basis = d.nv / n_prep;
         const long long nops = plan->frags[fi].nops.size();
         for (int b0 = 0; b0 < n_basis; b0 += std::min(chunk, n_basis))
-          for (int pc = 0; pc < n_prep; ++pc) {
-            items_nc.push_back(make_int2(fi, pc + n_prep * b0));
-            cost_nc.push_back((1ll << d.n) * (nops + 4 + 8ll * std::min(chunk, n_basis - b0)));
-          }
+          runs_nc.push_back({fi, n_prep * b0, n_prep, (1ll << d.n) * (nops + 4 + 8ll * std::min(chunk, n_basis - b0))});
       }
     }
-    sort_items(items_nc, cost_nc);
+    spread(runs_nc, items_nc);
 
     int f0 = 0;
     plan->t_prefix.push_back(0);
@@ -1025,16 +1018,19 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
         if (f.clifford && f.role == 1) { f.counts_off = off; off += (long long)f.nv << f.nA; }
     }
     std::vector<int2> items_hub, items_plain;
-    for (auto& it : items_c) {
-      const FragDev& f = plan->fdev[it.x];
-      if (f.role == 1) {
-        items_hub.push_back(it);
+    {
+      std::vector<Run> hubs, plain;
+      for (auto& r : runs_c) {
+        const FragDev& f = plan->fdev[r.frag];
+        if (f.role != 1) { plain.push_back(r); continue; }
+        hubs.push_back(r);
         plan->max_hub_nA = std::max(plan->max_hub_nA, f.nA);
         plan->min_hub_nA = std::min(plan->min_hub_nA, f.nA);
         plan->min_hub_m = std::min(plan->min_hub_m, f.m);
         if (f.m < 2 || f.qout > 4 || f.nA > 16) plan->hub_bytes_ok = false;
       }
-      else items_plain.push_back(it);
+      spread(hubs, items_hub);
+      spread(plain, items_plain);
     }
     plan->n_items_hub = (int)items_hub.size();
     plan->n_items_plain = (int)items_plain.size();
