@@ -449,6 +449,24 @@ __device__ __forceinline__ float4 hub4_stream(const int16_t* p) {
                      (float)(short)((unsigned)w.y >> 16));
 }
 
+// A thread's 4 x NN partial sums, consecutive in memory (16-byte aligned where
+// NN is a multiple of four): as 16-byte stores.  Single words at that stride
+// write every 32-byte sector eight times over.
+template <int NN, class F>
+__device__ __forceinline__ void store_part(float* dst, F&& at) {
+  if constexpr (NN % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < 4 * NN; i += 4)
+      *reinterpret_cast<float4*>(dst + i) = make_float4(at(i / NN, i % NN), at(i / NN, i % NN + 1),
+                                                        at(i / NN, i % NN + 2), at(i / NN, i % NN + 3));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NN; ++j) dst[i * NN + j] = at(i, j);
+  }
+}
+
 template <int NN>
 __device__ __forceinline__ void stream_fma(float (&acc)[4][NN], float4 a, const float* rrow, int bf16) {
   if (bf16) { a.x = to_bf16f(a.x); a.y = to_bf16f(a.y); a.z = to_bf16f(a.z); a.w = to_bf16f(a.w); }
@@ -521,11 +539,7 @@ __global__ void __launch_bounds__(256, 2) gemm_stream_kernel(const T* __restrict
         stream_fma<NN>(acc, hub4_stream(ap + (long long)r * M), Rs + r * NN, bf16);
   }
   if (!act) return;
-  float* dst = part + ((long long)split * M + m) * NN;    // 4 x NN contiguous floats
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < NN; ++j) dst[i * NN + j] = acc[i][j] * sc;
+  store_part<NN>(part + ((long long)split * M + m) * NN, [&](int i, int j) { return acc[i][j] * sc; });
 }
 
 // The same split-K product for dense operands with the loads moved off the
@@ -642,11 +656,7 @@ __global__ void __launch_bounds__(288, 2) gemm_stream_bulk_kernel(const T* __res
   const int m = m0 + 4 * (int)threadIdx.x;
   if (m >= M) return;
   const bool good = !*abort_flag;
-  float* dst = part + ((long long)split * M + m) * NN;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < NN; ++j) dst[i * NN + j] = good ? acc[i][j] * sc : 0.f;
+  store_part<NN>(part + ((long long)split * M + m) * NN, [&](int i, int j) { return good ? acc[i][j] * sc : 0.f; });
 }
 
 // --- the first leaf contracted while streaming --------------------------
@@ -822,11 +832,7 @@ __global__ void __launch_bounds__(288, 2) gemm_fact_bulk_kernel(const T* __restr
   const int m = m0 + 4 * (int)threadIdx.x;
   if (m >= M) return;
   const bool good = !*abort_flag;
-  float* dst = part + ((long long)split * M + m) * N;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < N; ++j) dst[i * N + j] = good ? acc[i][j] * sc : 0.f;
+  store_part<N>(part + ((long long)split * M + m) * N, [&](int i, int j) { return good ? acc[i][j] * sc : 0.f; });
 }
 
 template <int N1, int NR, class T>
