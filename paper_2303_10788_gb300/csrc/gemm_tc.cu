@@ -13,6 +13,14 @@
 // registers while the other accumulator fills, then write the FP32 partial
 // tile.  Split-K partials are summed in FP64 by the common reduction kernel.
 //
+// A sampled hub's operand holds 16-bit count sums, hub output fastest.  It is
+// read as it is (box of 64 cut indices x 64 outputs, twice), converted to bf16
+// in place by eight more warps -- an element is two bytes before and after, so
+// neither the place nor the swizzle changes -- and multiplied as an MN-major A
+// tile.  A transposing conversion pass through memory before the GEMM read and
+// wrote the operand once more: 67 MB of counts (K = 65536, M = 512, N = 16) took
+// 42 us there and 25 us here, now 23 us in all.
+//
 // Every wait on an mbarrier is bounded by a clock budget; on expiry the
 // kernel records an error bit in the status word, stops issuing, waits
 // (bounded) for its own copies in flight, frees its tensor memory and
@@ -64,6 +72,24 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// The same for an MN-major tile: 128-byte rows of 64 outputs, one per cut index;
+// 8-row groups 1024 bytes apart, the next 64 outputs 64 rows further.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(const void* tile) {
+  const uint64_t a = s_addr(tile);
+  uint64_t d = (a & 0x3FFFFull) >> 4;       // start address
+  d |= (uint64_t)(kBK * 128 >> 4) << 16;    // stride between blocks of 64 outputs
+  d |= (uint64_t)(1024 >> 4) << 32;         // stride between 8-row groups
+  d |= 1ull << 46;                          // descriptor version
+  d |= 2ull << 61;                          // 128-byte swizzle
+  return d;
+}
+
+// Two 16-bit count sums times the scale, as bf16.
+__device__ __forceinline__ uint32_t counts_bf16(int w, float scale) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn((float)(short)(w & 0xffff) * scale, (float)(w >> 16) * scale);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 // Shared-memory matrix descriptor: K-major tile of 128-byte rows with the
 // 128-byte swizzle; 8-row groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_sw128(const void* tile) {
@@ -110,9 +136,13 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(bar)) : "memory");
 }
 
-__global__ void __launch_bounds__(192, 1)
+constexpr int kConvWarps = 8;   // a tile's 1024 16-byte pieces: four per lane
+
+template <bool COUNTS>
+__global__ void __launch_bounds__(192 + (COUNTS ? 32 * kConvWarps : 0), 1)
     gemm_bf16_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M,
-                        int N, int k_tiles, int tiles_per_split, int mtiles, float* partials, unsigned* status) {
+                        int N, int k_tiles, int tiles_per_split, int mtiles, float scale, float* partials,
+                        unsigned* status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int a_bytes = kBM * kBK * 2, b_bytes = N * kBK * 2;
@@ -122,7 +152,8 @@ __global__ void __launch_bounds__(192, 1)
   uint64_t* empty = full + kStages;
   uint64_t* acc_full = empty + kStages;      // [2]: accumulator b complete
   uint64_t* acc_empty = acc_full + 2;        // [2]: accumulator b drained
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* conv = acc_empty + 2;            // a stage's counts converted
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(conv + kStages);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = blockIdx.x % mtiles, split = blockIdx.x / mtiles;
@@ -136,6 +167,7 @@ __global__ void __launch_bounds__(192, 1)
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
+      mbar_init(&conv[s], kConvWarps);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
@@ -155,9 +187,10 @@ __global__ void __launch_bounds__(192, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  // instruction descriptor: f32 accumulate, bf16 A and B, both K-major, M = 128, N
+  // instruction descriptor: f32 accumulate, bf16 A and B, K-major (counts: A MN-major), M = 128, N
   const uint32_t idesc =
-      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+      (COUNTS ? 1u << 15 : 0u) | (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
+      ((uint32_t)(kBM >> 4) << 24);
   int issued = 0;   // TMA stages issued by the producer
   if (warp == 0) {
     if (lane == 0) {
@@ -169,7 +202,12 @@ __global__ void __launch_bounds__(192, 1)
         }
         if (*abort_flag) break;
         mbar_expect_tx(&full[s], (uint32_t)(a_bytes + b_bytes));
-        tma_load_2d(A_s + s * a_bytes, &tmA, &full[s], (kt0 + i) * kBK, mt * kBM);
+        if constexpr (COUNTS) {
+          for (int h = 0; h < kBM / 64; ++h)
+            tma_load_2d(A_s + s * a_bytes + h * kBK * 128, &tmA, &full[s], mt * kBM + h * 64, (kt0 + i) * kBK);
+        } else {
+          tma_load_2d(A_s + s * a_bytes, &tmA, &full[s], (kt0 + i) * kBK, mt * kBM);
+        }
         tma_load_2d(B_s + s * b_bytes, &tmB, &full[s], (kt0 + i) * kBK, 0);
         issued = i + 1;
       }
@@ -187,21 +225,48 @@ __global__ void __launch_bounds__(192, 1)
         const int i1 = min(nk, (g + 1) * kGroup);
         for (int i = g * kGroup; i < i1; ++i) {
           const int s = i % kStages;
-          if (!mbar_wait(&full[s], (i / kStages) & 1) || *abort_flag) {
+          if (!mbar_wait(&full[s], (i / kStages) & 1) ||
+              (COUNTS && !mbar_wait(&conv[s], (i / kStages) & 1)) || *abort_flag) {
             atomicOr(status, 4u);
             *abort_flag = 1;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint64_t ad = smem_desc_sw128(A_s + s * a_bytes), bd = smem_desc_sw128(B_s + s * b_bytes);
+          const uint64_t ad = COUNTS ? smem_desc_mn_sw128(A_s + s * a_bytes) : smem_desc_sw128(A_s + s * a_bytes);
+          const uint64_t bd = smem_desc_sw128(B_s + s * b_bytes);
+          constexpr int a_step = COUNTS ? 16 * 128 >> 4 : 2;   // 16 rows of 128 bytes
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk)   // 16 bf16 = 32 bytes = 2 descriptor units per step
-            mma_bf16(tmem + (uint32_t)(b * N), ad + 2 * kk, bd + 2 * kk, idesc,
+            mma_bf16(tmem + (uint32_t)(b * N), ad + a_step * kk, bd + 2 * kk, idesc,
                      (i > g * kGroup || kk > 0) ? 1u : 0u);
           mma_commit(&empty[s]);
         }
         mma_commit(&acc_full[b]);   // arrives when this group's MMAs have completed
       }
+    }
+  } else if (COUNTS && warp >= 6) {
+    // conversion warps
+    const int t = (int)threadIdx.x - 192;
+    for (int i = 0; i < nk; ++i) {
+      const int s = i % kStages;
+      bool ok = !*abort_flag && mbar_wait(&full[s], (i / kStages) & 1);
+      ok = __all_sync(0xffffffffu, ok) != 0;
+      if (!ok) {
+        if (lane == 0) { atomicOr(status, 4u); *abort_flag = 1; }
+        break;
+      }
+      int4* tile = reinterpret_cast<int4*>(A_s + s * a_bytes);
+      constexpr int kPer = kBM * kBK * 2 / 16 / (32 * kConvWarps);
+      int4 v[kPer];
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) v[j] = tile[t + 32 * kConvWarps * j];
+#pragma unroll
+      for (int j = 0; j < kPer; ++j)
+        tile[t + 32 * kConvWarps * j] = make_int4((int)counts_bf16(v[j].x, scale), (int)counts_bf16(v[j].y, scale),
+                                                  (int)counts_bf16(v[j].z, scale), (int)counts_bf16(v[j].w, scale));
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads them next
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&conv[s]);
     }
   } else {
     // drain warps: TMEM lanes 32*(warp % 4) .. +31 = tile rows
@@ -241,8 +306,10 @@ __global__ void __launch_bounds__(192, 1)
       float* dst = partials + ((long long)split * M + m) * N;
       const bool good = !*abort_flag;
 #pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (j < N) dst[j] = good ? sum[j] : 0.f;
+      for (int j = 0; j < 32; j += 4)        // N is 16 or 32, the partials 16-byte aligned
+        if (j < N)
+          *reinterpret_cast<float4*>(dst + j) =
+              good ? make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
   __syncwarp();
@@ -255,6 +322,12 @@ __global__ void __launch_bounds__(192, 1)
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
 }
+
+bool gemm_tc_supported(int M, int N, long long K) {
+  return (N == 16 || N == 32) && K % kBK == 0 && K >= 1024 && M >= 1;
+}
+
+size_t gemm_tc_smem(int N) { return (size_t)kStages * (kBM * kBK * 2 + N * kBK * 2) + 1024 + 256; }
 
 namespace {
 
@@ -276,40 +349,53 @@ EncodeTiled encode_fn() {
   return fn;
 }
 
-bool make_map(CUtensorMap* map, const void* base, long long inner, long long rows, int box_rows) {
+bool make_map(CUtensorMap* map, CUtensorMapDataType type, const void* base, long long inner, long long rows,
+              int box_rows) {
   EncodeTiled enc = encode_fn();
   if (!enc) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)inner * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
+  const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};     // 128 bytes: the swizzle's width
   const cuuint32_t estr[2] = {1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+  return enc(map, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-}  // namespace
-
-bool gemm_tc_supported(int M, int N, long long K) {
-  return (N == 16 || N == 32) && K % kBK == 0 && K >= 1024 && M >= 1;
-}
-
-size_t gemm_tc_smem(int N) { return (size_t)kStages * (kBM * kBK * 2 + N * kBK * 2) + 1024 + 256; }
-
-cudaError_t launch_gemm_tc(const void* A, const void* Bt, int M, int N, long long K, int splits, float* partials,
-                           unsigned* status, cudaStream_t s) {
-  if (!gemm_tc_supported(M, N, K)) return cudaErrorInvalidValue;
-  if ((reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(Bt) & 15)) return cudaErrorMisalignedAddress;
+template <bool COUNTS>
+cudaError_t launch(const void* A, float scale, const void* Bt, int M, int N, long long K, int splits, float* partials,
+                   unsigned* status, cudaStream_t s) {
+  if (!gemm_tc_supported(M, N, K) || (COUNTS && M % kBM)) return cudaErrorInvalidValue;
+  if ((reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(Bt) & 15) ||
+      (reinterpret_cast<uintptr_t>(partials) & 15))
+    return cudaErrorMisalignedAddress;
   CUtensorMap ta, tb;
-  if (!make_map(&ta, A, K, M, kBM) || !make_map(&tb, Bt, K, N, N)) return cudaErrorInvalidValue;
+  const bool ok = COUNTS ? make_map(&ta, CU_TENSOR_MAP_DATA_TYPE_UINT16, A, M, K, kBK)
+                         : make_map(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, K, M, kBM);
+  if (!ok || !make_map(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Bt, K, N, N)) return cudaErrorInvalidValue;
   const int k_tiles = (int)(K / kBK);
   const int per = (k_tiles + splits - 1) / splits;
   const int mtiles = (M + kBM - 1) / kBM;
   const size_t smem = gemm_tc_smem(N);
-  cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e =
+      cudaFuncSetAttribute(gemm_bf16_tc_kernel<COUNTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  gemm_bf16_tc_kernel<<<mtiles * splits, 192, smem, s>>>(ta, tb, M, N, k_tiles, per, mtiles, partials, status); note_launch();
+  gemm_bf16_tc_kernel<COUNTS><<<mtiles * splits, 192 + (COUNTS ? 32 * kConvWarps : 0), smem, s>>>(
+      ta, tb, M, N, k_tiles, per, mtiles, scale, partials, status);
+  note_launch();
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_gemm_tc(const void* A, const void* Bt, int M, int N, long long K, int splits, float* partials,
+                           unsigned* status, cudaStream_t s) {
+  return launch<false>(A, 1.f, Bt, M, N, K, splits, partials, status, s);
+}
+
+cudaError_t launch_gemm_tc_counts(const int16_t* At, float scale, const void* Bt, int M, int N, long long K, int splits,
+                                  float* partials, unsigned* status, cudaStream_t s) {
+  return launch<true>(At, scale, Bt, M, N, K, splits, partials, status, s);
 }
 
 }  // namespace ccs

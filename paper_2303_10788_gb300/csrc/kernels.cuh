@@ -351,5 +351,9 @@ int featurize(const Problem& p, const std::vector<ccs_cut>& cuts, std::vector<fl
 bool gemm_tc_supported(int M, int N, long long K);
 cudaError_t launch_gemm_tc(const void* A, const void* Bt, int M, int N, long long K, int splits, float* partials,
                            unsigned* status, cudaStream_t s);
+// The same of a sampled hub's operand as it lies (K rows of M 16-bit count sums,
+// times scale); M a multiple of 128.
+cudaError_t launch_gemm_tc_counts(const int16_t* At, float scale, const void* Bt, int M, int N, long long K, int splits,
+                                  float* partials, unsigned* status, cudaStream_t s);
 
 }  // namespace ccs

@@ -1656,14 +1656,18 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
       for (int i = 0; i < z.n_problems; ++i) {
         const ProblemDev& Pb = z.host_problems[i];
         if (!Pb.tc) continue;
-        {
+        const HubView hub = hub_host_view(r, Pb);
+        if (hub.h && Pb.M % 128 == 0) {          // count sums: converted inside the GEMM
+          err = launch_gemm_tc_counts(hub.h, hub.scale, z.rt_scratch + Pb.rt_off, Pb.M, Pb.N, Pb.K, Pb.splits,
+                                      scratch + Pb.part_off, r.status, s);
+        } else {
           const long long tiles = ((Pb.K + 63) / 64) * ((Pb.M + 63) / 64);
           hub_bf16_kernel<<<(unsigned)(tiles < 152 * 32 ? tiles : 152 * 32), 256, 0, s>>>(
-              hub_host_view(r, Pb), reinterpret_cast<__nv_bfloat16*>(r.TQh) + Pb.hub_T_off, Pb.M, Pb.K); note_launch();
+              hub, reinterpret_cast<__nv_bfloat16*>(r.TQh) + Pb.hub_T_off, Pb.M, Pb.K); note_launch();
           if ((err = cudaGetLastError()) != cudaSuccess) return err;
+          err = launch_gemm_tc(r.TQh + Pb.hub_T_off, z.rt_scratch + Pb.rt_off, Pb.M, Pb.N, Pb.K, Pb.splits,
+                               scratch + Pb.part_off, r.status, s);
         }
-        err = launch_gemm_tc(r.TQh + Pb.hub_T_off, z.rt_scratch + Pb.rt_off, Pb.M, Pb.N, Pb.K, Pb.splits,
-                             scratch + Pb.part_off, r.status, s);
         if (err != cudaSuccess) return err;
       }
     }
