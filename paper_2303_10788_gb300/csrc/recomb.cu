@@ -297,34 +297,89 @@ static __host__ __device__ bool fact_path(const ProblemDev& Pb, int precision, i
   return Pb.stream && Pb.fact && !Pb.direct && precision == CCS_FP32 && !stitched && full_range;
 }
 
-__global__ void build_r_kernel(DevPlan P, DevRes R, int precision, const long long* prefix, int np,
-                               long long total, float* scratch, uint16_t* rt_scratch, int stitched, int full_range) {
-  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
-       g += (long long)gridDim.x * blockDim.x) {
-    const int pi = find_seg(prefix, np, g);
-    const ProblemDev& Pb = P.problems[pi];
-    const long long loc = g - prefix[pi];
-    const long long Pp = loc / Pb.N;
-    const long long ol = loc - Pp * Pb.N;
-    // a streamed stitched hub reads no R row of a zero operand row; a problem
-    // on the first-leaf path builds its own smaller table instead of R
-    if (stitched && Pb.stream && Pb.hub_qrow_off >= 0 && !R.qnz[Pb.hub_qrow_off + Pp]) continue;
-    if (fact_path(Pb, precision, stitched, full_range != 0) && !(rt_scratch && Pb.tc)) continue;
-    float v = 1.f;
-    int off = 0;
-    for (int l = 0; l < Pb.n_frags; ++l) {
-      if (l == Pb.hub) continue;
-      const FragDev& L = P.frags[Pb.frag0 + l];
-      const int x = (int)((ol >> off) & ((1ll << L.m) - 1));
-      off += L.m;
-      int pl = 0;
-      for (int i = 0; i < L.n_slots; ++i) pl |= (int)((Pp >> (2 * L.slot_cut[i])) & 3) << (2 * i);
-      v *= R.TQ[L.T_off + ((long long)x << (2 * L.n_slots)) + pl];
+// Fragment descriptors of one problem, read once into shared memory so that
+// the per-element loops below do no dependent global loads.
+constexpr int kMaxProblemFrags = kMaxProblemFragments;   // checked when the plan is built
+constexpr int kLeafStage = 2048;   // floats of a leaf table staged in shared memory
+static_assert(2 * kZTree <= kLeafStage && 16 * 128 <= kLeafStage, "the Z-string tensors of a tree share the leaf table's space");
+struct ProblemShared {
+  int nf, hub, k;
+  int m[kMaxProblemFrags], ns[kMaxProblemFrags];
+  int slot_cut[kMaxProblemFrags][kMaxCuts];
+  int marg_pos[kMaxProblemFrags][kMaxMarginal];
+  long long T_off[kMaxProblemFrags];
+};
+
+// A warp per fragment, a lane per array entry (at least as many warps as fragments).
+__device__ void load_problem(const DevPlan& P, const ProblemDev& Pb, ProblemShared& S) {
+  const int l = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) { S.nf = Pb.n_frags; S.hub = Pb.hub; S.k = Pb.k; }
+  for (int f = l; f < Pb.n_frags; f += blockDim.x >> 5) {
+    const FragDev& L = P.frags[Pb.frag0 + f];
+    if (lane < kMaxCuts) S.slot_cut[f][lane] = L.slot_cut[lane];
+    if (lane < kMaxMarginal) S.marg_pos[f][lane] = L.marg_pos[lane];
+    if (lane == 24) S.m[f] = L.m;
+    if (lane == 25) S.ns[f] = L.n_slots;
+    if (lane == 26) S.T_off[f] = L.T_off;
+  }
+}
+
+// Slot digits of fragment l in cut index Pp.
+__device__ __forceinline__ int frag_digits(const ProblemShared& S, int l, long long Pp) {
+  int pl = 0;
+  for (int i = 0; i < S.ns[l]; ++i) pl |= (int)((Pp >> (2 * S.slot_cut[l][i])) & 3) << (2 * i);
+  return pl;
+}
+
+// A CTA takes 1024 consecutive elements, and reads the descriptors of its
+// problem once (an element spans one dependent chain of descriptor loads
+// otherwise).  A tensor-core problem gets only R'^T, written along K
+// (K = 65536, N = 16: 18.2 us an element at a time along N, 13.4 us so).
+constexpr int kRPerThread = 4;
+__global__ void __launch_bounds__(256) build_r_kernel(DevPlan P, DevRes R, int precision, const long long* prefix,
+                                                      int np, long long total, float* scratch, uint16_t* rt_scratch,
+                                                      int stitched, int full_range) {
+  __shared__ ProblemShared S;
+  const long long span = 256ll * kRPerThread;
+  for (long long base = blockIdx.x * span; base < total; base += gridDim.x * span) {
+    const long long end = min(total, base + span);
+    for (long long g0 = base; g0 < end;) {              // the problems this stretch crosses
+      const int pi = find_seg(prefix, np, g0);
+      const long long first = prefix[pi], g1 = min(end, prefix[pi + 1]);
+      const ProblemDev& Pb = P.problems[pi];
+      const bool tc = precision == CCS_BF16 && Pb.tc && rt_scratch;
+      // a problem on the first-leaf path builds its own smaller table instead of R
+      const bool skip = fact_path(Pb, precision, stitched, full_range != 0) && !(rt_scratch && Pb.tc);
+      __syncthreads();
+      if (!skip) load_problem(P, Pb, S);
+      __syncthreads();
+      if (!skip) {
+#pragma unroll
+        for (int u = 0; u < kRPerThread; ++u) {
+          const long long g = g0 + threadIdx.x + 256ll * u, loc = g - first;
+          if (g >= g1) continue;
+          const int sh = tc ? 2 * S.k : __ffs(Pb.N) - 1;      // K and N are powers of two
+          const long long hi = loc >> sh, lo = loc - (hi << sh);
+          const long long Pp = tc ? lo : hi, ol = tc ? hi : lo;
+          // a streamed stitched hub reads no R row of a zero operand row
+          if (stitched && Pb.stream && Pb.hub_qrow_off >= 0 && !R.qnz[Pb.hub_qrow_off + Pp]) continue;
+          float v = 1.f;
+          int off = 0;
+          for (int l = 0; l < S.nf; ++l) {
+            if (l == S.hub) continue;
+            const int x = (int)((ol >> off) & ((1ll << S.m[l]) - 1));
+            off += S.m[l];
+            v *= R.TQ[S.T_off[l] + ((long long)x << (2 * S.ns[l])) + frag_digits(S, l, Pp)];
+          }
+          if (tc) {      // R'^T for the tensor-core GEMM
+            reinterpret_cast<__nv_bfloat16*>(rt_scratch)[Pb.rt_off + loc] = __float2bfloat16_rn(to_bf16f(v));
+          } else {
+            scratch[Pb.r_off + loc] = precision == CCS_BF16 ? to_bf16f(v) : v;
+          }
+        }
+      }
+      g0 = g1;
     }
-    if (precision == CCS_BF16) v = to_bf16f(v);
-    scratch[Pb.r_off + loc] = v;
-    if (precision == CCS_BF16 && Pb.tc && rt_scratch)   // R'^T for the tensor-core GEMM
-      reinterpret_cast<__nv_bfloat16*>(rt_scratch)[Pb.rt_off + ol * Pb.K + Pp] = __float2bfloat16_rn(v);
   }
 }
 
@@ -991,13 +1046,19 @@ __global__ void __launch_bounds__(256) reduce_scatter_kernel(DevPlan P, const lo
                                                              long long total, const float* scratch, double* marg_out,
                                                              int use_tc) {
   __shared__ double red[8][32];
+  __shared__ ProblemShared S;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (long long base = blockIdx.x * 32ll; base < total; base += gridDim.x * 32ll) {
     const long long g = base + lane;
     float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
     int pi = -1;
+    // the descriptors arrive beside the partials, when the 32 outputs are one
+    // problem's (65536 outputs of 76 splits: 17.1 us read afterwards, 15.1 us so)
+    const int p0 = find_seg(prefix, np, base);
+    const bool staged = min(total, base + 32) <= prefix[p0 + 1];
+    if (staged) load_problem(P, P.problems[p0], S);
     if (g < total) {
-      pi = find_seg(prefix, np, g);
+      pi = staged ? p0 : find_seg(prefix, np, g);
       const ProblemDev& Pb = P.problems[pi];
       if (Pb.direct || Pb.general) pi = -1;   // written by the leaf-by-leaf or the general contraction
       else {
@@ -1027,14 +1088,23 @@ __global__ void __launch_bounds__(256) reduce_scatter_kernel(DevPlan P, const lo
       const long long loc = g - prefix[pi];
       const long long m = loc / Pb.N, n = loc - m * Pb.N;
       long long o = 0;
-      const FragDev& Hb = P.frags[Pb.frag0 + Pb.hub];
-      for (int j = 0; j < Hb.m; ++j) o |= ((m >> j) & 1) << Hb.marg_pos[j];
       int off = 0;
-      for (int l = 0; l < Pb.n_frags; ++l) {
-        if (l == Pb.hub) continue;
-        const FragDev& L = P.frags[Pb.frag0 + l];
-        for (int j = 0; j < L.m; ++j) o |= ((n >> (off + j)) & 1) << L.marg_pos[j];
-        off += L.m;
+      if (staged) {
+        for (int j = 0; j < S.m[S.hub]; ++j) o |= ((m >> j) & 1) << S.marg_pos[S.hub][j];
+        for (int l = 0; l < S.nf; ++l) {
+          if (l == S.hub) continue;
+          for (int j = 0; j < S.m[l]; ++j) o |= ((n >> (off + j)) & 1) << S.marg_pos[l][j];
+          off += S.m[l];
+        }
+      } else {
+        const FragDev& Hb = P.frags[Pb.frag0 + Pb.hub];
+        for (int j = 0; j < Hb.m; ++j) o |= ((m >> j) & 1) << Hb.marg_pos[j];
+        for (int l = 0; l < Pb.n_frags; ++l) {
+          if (l == Pb.hub) continue;
+          const FragDev& L = P.frags[Pb.frag0 + l];
+          for (int j = 0; j < L.m; ++j) o |= ((n >> (off + j)) & 1) << L.marg_pos[j];
+          off += L.m;
+        }
       }
       marg_out[Pb.marg_off + o] = ldexp(acc, -Pb.k);
     }
@@ -1047,40 +1117,6 @@ __device__ __forceinline__ long long spread(long long v, int nd, const uint8_t* 
   long long p = 0;
   for (int j = 0; j < nd; ++j) p |= ((v >> (2 * j)) & 3ll) << (2 * pos[j]);
   return p;
-}
-
-// Fragment descriptors of one problem, read once into shared memory so that
-// the per-element loops below do no dependent global loads.
-constexpr int kMaxProblemFrags = kMaxProblemFragments;   // checked when the plan is built
-constexpr int kLeafStage = 2048;   // floats of a leaf table staged in shared memory
-static_assert(2 * kZTree <= kLeafStage && 16 * 128 <= kLeafStage, "the Z-string tensors of a tree share the leaf table's space");
-struct ProblemShared {
-  int nf, hub, k;
-  int m[kMaxProblemFrags], ns[kMaxProblemFrags];
-  int slot_cut[kMaxProblemFrags][kMaxCuts];
-  int marg_pos[kMaxProblemFrags][kMaxMarginal];
-  long long T_off[kMaxProblemFrags];
-};
-
-// A warp per fragment, a lane per array entry (at least as many warps as fragments).
-__device__ void load_problem(const DevPlan& P, const ProblemDev& Pb, ProblemShared& S) {
-  const int l = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) { S.nf = Pb.n_frags; S.hub = Pb.hub; S.k = Pb.k; }
-  for (int f = l; f < Pb.n_frags; f += blockDim.x >> 5) {
-    const FragDev& L = P.frags[Pb.frag0 + f];
-    if (lane < kMaxCuts) S.slot_cut[f][lane] = L.slot_cut[lane];
-    if (lane < kMaxMarginal) S.marg_pos[f][lane] = L.marg_pos[lane];
-    if (lane == 24) S.m[f] = L.m;
-    if (lane == 25) S.ns[f] = L.n_slots;
-    if (lane == 26) S.T_off[f] = L.T_off;
-  }
-}
-
-// Slot digits of fragment l in cut index Pp.
-__device__ __forceinline__ int frag_digits(const ProblemShared& S, int l, long long Pp) {
-  int pl = 0;
-  for (int i = 0; i < S.ns[l]; ++i) pl |= (int)((Pp >> (2 * S.slot_cut[l][i])) & 3) << (2 * i);
-  return pl;
 }
 
 // T_f^S(zi, P) folded from the variants' Z-string values the way T_f is
@@ -1625,7 +1661,7 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
       need_gemm = need_gemm || (!tc && !Pb.stream);
     }
     if (z.r_total > 0 && need_r) {
-      build_r_kernel<<<grid(z.r_total, 256), 256, 0, s>>>(p, r, precision, z.r_prefix, p.n_problems, z.r_total,
+      build_r_kernel<<<grid(z.r_total, 256 * kRPerThread), 256, 0, s>>>(p, r, precision, z.r_prefix, p.n_problems, z.r_total,
                                                           scratch, use_tc ? z.rt_scratch : nullptr, z.stitched,
                                                           z.krange.full() ? 1 : 0);
       note_launch();
