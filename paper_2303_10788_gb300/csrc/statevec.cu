@@ -13,7 +13,7 @@
 // four times.  A fragment is a chain of such steps, bound by their latency;
 // in a batch the instructions per step decide how much of the chip is taken
 // from the Clifford branch beside it (64 circuits: 194 us beside it before,
-// 77 us so; one 100-qubit circuit: 32 us before, 29.7 us so).  Amplitudes are stored at swz(i), so that
+// 72 us so; one 100-qubit circuit: 32 us before, 24.8 us so).  Amplitudes are stored at swz(i), so that
 // the groups of a half warp fall on distinct 8-byte banks for nearly every pair
 // of wires.
 // Outputs per variant: the exact marginal on A_f and the Z-string values, both
@@ -101,8 +101,8 @@ __device__ __forceinline__ int digit_out(int v, int qin, int i) {
 }  // namespace
 
 // States of at most this many wires take four lanes per group (kernel times, one
-// lane and four: 25 ops on 6 wires 20.4 and 13.2 us, 31 on 7 23.5 and 12.5 us,
-// 37 on 8 20.0 and 14.2 us); at 9 wires the two are equal (71 ops: 29.9 us).
+// lane and four: 13 ops on 4 wires 9.9 and 8.9 us, 25 on 6 13.2 and 9.3 us, 31 on
+// 7 14.7 and 9.8 us, 37 on 8 14.9 and 12.1 us); at 9 wires the two were equal.
 constexpr int kSmallState = 8;
 constexpr int kOpStage = 128;   // fused ops staged in shared memory at a time
 constexpr int kZChunk = 256;    // Z-string masks built per pass
@@ -131,6 +131,25 @@ __global__ void __launch_bounds__(512) statevector_kernel(DevPlan P, DevRes R, i
     const int pc = it.y % n_prep, b0 = it.y / n_prep, b1 = min(n_basis, b0 + P.nc_basis_chunk);
     const unsigned N = 1u << n;
     const int op0 = P.moments[F.mom_off], op1 = P.moments[F.mom_off + F.n_moments];
+    // a chunk of ops on its way to shared memory: the matrices as asynchronous
+    // copies of 8 bytes (all in flight at once; plain loads in a loop: 29.9 us
+    // for a 100-qubit circuit's kernel, 24.8 us so; with nothing cached the
+    // stage 41.8 and 31.8 us), the wires as places
+    auto stage = [&](int c0, int cnt) {
+      static_assert(sizeof(NCOp) == 17 * 8, "two wires, then the matrix");
+      const NCOp* src = P.nops + F.ops_off + c0;
+      for (int i = tid; i < cnt * 16; i += blockDim.x) {
+        const int o = i >> 4, w = 2 * (i & 15);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(mat_s + 32 * o + w)),
+                     "l"(src[o].m + w)
+                     : "memory");
+      }
+      for (int o = tid; o < cnt; o += blockDim.x) {
+        const int2 ab = *reinterpret_cast<const int2*>(src + o);
+        pl_s[o] = op_place(ab.x, ab.y);
+      }
+    };
+    stage(op0, min(kOpStage, op1 - op0));      // beside the loads of the preparation and the masks
     {   // the prepared product state: amplitude i is the product of its inputs' entries
       unsigned inb = 0;
       for (int o = 0; o < qin; ++o) inb |= 1u << P.wires[F.qin_off + o];
@@ -155,17 +174,10 @@ __global__ void __launch_bounds__(512) statevector_kernel(DevPlan P, DevRes R, i
     };
     const bool z_once = nz <= kZChunk;     // one chunk: its masks before the ops, beside the other loads
     if (z_once) z_masks(0, nz);
-    __syncthreads();
     for (int c0 = op0; c0 < op1; c0 += kOpStage) {
       const int cnt = min(kOpStage, op1 - c0);
-      const float* src = reinterpret_cast<const float*>(P.nops + F.ops_off + c0);
-      static_assert(sizeof(NCOp) == 34 * 4, "two wires, then the matrix");
-      for (int i = tid; i < cnt * 34; i += blockDim.x) {
-        const int o = i / 34, w = i - 34 * o;
-        const float v = src[i];
-        if (w >= 2) mat_s[32 * o + w - 2] = v;
-        else if (w == 0) pl_s[o] = op_place(__float_as_int(v), __float_as_int(src[i + 1]));
-      }
+      if (c0 != op0) stage(c0, cnt);
+      asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
       // the next op's places and matrix are prepared while this op's amplitudes
       // are on their way
@@ -236,6 +248,7 @@ __global__ void __launch_bounds__(512) statevector_kernel(DevPlan P, DevRes R, i
         }
       }
     }
+    if (op0 == op1) __syncthreads();
     // U |prep> stays in psi; each basis combination changes a copy, its last
     // output on the way to the probabilities
     unsigned amask = 0;
