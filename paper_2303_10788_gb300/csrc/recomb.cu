@@ -506,7 +506,8 @@ __device__ __forceinline__ float4 hub4_stream(const int16_t* p) {
 
 // A thread's 4 x NN partial sums, consecutive in memory (16-byte aligned where
 // NN is a multiple of four): as 16-byte stores.  Single words at that stride
-// write every 32-byte sector eight times over.
+// write every 32-byte sector eight times over, all CTAs at the kernel's end (537 MB
+// hub operand, 16 leaf outputs: 116 us so, 99 us with 16-byte stores).
 template <int NN, class F>
 __device__ __forceinline__ void store_part(float* dst, F&& at) {
   if constexpr (NN % 4 == 0) {
