@@ -1474,17 +1474,23 @@ __device__ __forceinline__ uint32_t space_point(const uint32_t (*tbl)[256], uint
 // with every pivot bit clear) has the identity basis and a zero offset, so a
 // shot's outcome is its coefficient bits; checked, not assumed.  One warp, a
 // basis vector per lane (one thread reading them in turn took as long as a
-// hundred shots of the whole CTA).
+// hundred shots of the whole CTA).  CB: the counters' width; count_field takes a
+// counter's place in its word from the low log2(32 / CB) bits of the unmasked
+// field, so a space needs that many bits to count as one (a hub that measures
+// nothing has none: its shots go through the tables, all to outcome 0).
+template <int CB>
 __device__ __forceinline__ bool space_is_identity(const SpaceRec& sp, int rank, int nA) {
+  constexpr int kPlaceBits = CB == 4 ? 3 : CB == 8 ? 2 : CB == 16 ? 1 : 0;
   const int j = (int)threadIdx.x & 31;
   const bool ok = j >= rank || sp.basis[j] == (1u << j);
-  return __all_sync(0xffffffffu, ok) && rank == nA && sp.off == 0u;
+  return __all_sync(0xffffffffu, ok) && rank == nA && rank >= kPlaceBits && sp.off == 0u;
 }
 
 // All shots of a hub variant whose outcome is its coefficient bits, counted
 // in shared memory: 4-, 8-, 16- or 32-bit counters.  The field's place in
 // its word, its word's byte address and its increment come from one shift, one
-// mask and one wrapping shift each, with no masked copy of the field.
+// mask and one wrapping shift each, with no masked copy of the field (hence
+// space_is_identity's least rank).
 template <int CB>
 __device__ __forceinline__ void count_field(uint32_t* hist, uint32_t w, int sh, uint32_t cmask) {
   if (CB == 32) {
@@ -1793,7 +1799,7 @@ __global__ void __launch_bounds__(512) sample_hub_kernel(DevPlan P, DevRes R, Ev
   const int rank = sp.rank;
   const uint32_t off = sp.off;
   if ((threadIdx.x >> 5) == 1) {
-    const bool id = space_is_identity(sp, rank, nA);
+    const bool id = space_is_identity<WIDE ? 32 : 16>(sp, rank, nA);
     if (threadIdx.x == 32) s_ident = id ? 1 : 0;
   }
   if (F.qout <= 4) hub_variant_rows(F, v, s_czD, s_czS, s_nzm);   // warp 0: at most 16 rows
@@ -2103,7 +2109,7 @@ __device__ __forceinline__ void hub8_variant(const DevPlan& P, const DevRes& R, 
   const int rank = sp.rank;
   const uint32_t off = sp.off;
   if ((tid >> 5) == 1) {
-    const bool id = space_is_identity(sp, rank, nA);
+    const bool id = space_is_identity<8>(sp, rank, nA);
     if (tid == 32) s_ident = id ? 1 : 0;
   }
   // the variant's operand rows: one D and sign mask per Z-basis choice
@@ -2299,7 +2305,7 @@ __global__ void __launch_bounds__(kHub4Threads, 6) sample_hub4_kernel(DevPlan P,
     return;
   }
   if ((tid >> 5) == 1) {
-    const bool id = space_is_identity(sp, rank, nA);
+    const bool id = space_is_identity<4>(sp, rank, nA);
     if (tid == 32) s_ident = id ? 1 : 0;
   }
   hub_variant_rows(F, v, s_czD, s_czS, s_nzm);
