@@ -493,11 +493,14 @@ __global__ void __launch_bounds__(256) ml_rebuild_kernel(DevPlan P, DevRes R, co
 }
 
 // --- blocks of 16 to 64 rows: one-sided Jacobi in registers ------------------
-// The columns of G = J / |J|_F + I (so G is positive semidefinite and its
-// singular vectors are J's eigenvectors), are made orthogonal by plane
+// With H = J - (tr J / D) I, the columns of G = H / |H|_F + I (positive
+// definite, as H has no eigenvalue below -sqrt(1 - 1/D) |H|_F; its singular
+// vectors are J's eigenvectors) are made orthogonal by plane
 // rotations from the right (Hestenes 1958; Golub & Van Loan, Sec. 8.6): then
-// v_k = g_k / |g_k|, the eigenvalue is its Rayleigh quotient, and no separate
-// eigenvector matrix is rotated.  A worker of LW lanes keeps two
+// v_k = g_k / |g_k|, the eigenvalue is its Rayleigh quotient with J, and no
+// separate eigenvector matrix is rotated.  The mean is taken out so that the
+// rounding of columns of length one is measured against the eigenvalues'
+// spread, not against the mean of a nearly scalar block.  A worker of LW lanes keeps two
 // groups of four columns in registers, two or four rows a lane as packed FP32
 // pairs: a step rotates four disjoint pairs (their inner products reduced
 // together), a round runs
@@ -672,8 +675,11 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 //   p <- c p - conj(z) q,  q <- z p + c q
 // (t may carry the estimates' rounding, c and z must not: the rotation is
 // unitary for any t).  The lanes of pair i compute its rotation.  A pair below
-// 2^-23 of its norms' product is left alone; one above 2^-16 asks for another
-// sweep (the rotations' error is quadratic in it).
+// 2^-23 of its norms' product is left alone; one above 2^-21 asks for another
+// sweep.  (Between well separated eigenvalues a sweep from 2^-16 on ends below
+// 2^-23, but inside a cluster, whose vectors turn by large angles, it gains a bit
+// or two: stopped at 2^-16, a block of rank one and 63 other eigenvalues within
+// 1e-5 kept off-diagonals of that size, 1.9e-5 of |J|_F in all, 4e-6 so.)
 template <int D, int P0, int Q0, int P1, int Q1, int P2, int Q2, int P3, int Q3>
 __device__ __forceinline__ void jacobi_step(MlCol<MlShape<D>::RH> (&g)[8], float (&nr)[8], bool& more) {
   constexpr int LW = MlShape<D>::LW, RH = MlShape<D>::RH;
@@ -702,7 +708,7 @@ __device__ __forceinline__ void jacobi_step(MlCol<MlShape<D>::RH> (&g)[8], float
   const float be = b1 ? (b2 ? nr[Q3] : nr[Q2]) : (b2 ? nr[Q1] : nr[Q0]);
   const float g2 = fmaf(re, re, im * im), ab = al * be;
   const bool rot = g2 > 1.4210855e-14f * ab;                 // 2^-46
-  more = more || g2 > 2.3283064e-10f * ab;                   // 2^-32
+  more = more || g2 > 2.2737368e-13f * ab;                   // 2^-42
   if (!__any_sync(FULL, rot)) return;
   float c = 1.f, zr = 0.f, zi = 0.f, dn = 0.f;
   if (rot) {
@@ -801,6 +807,10 @@ __global__ void __launch_bounds__(MlShape<D>::NT, MlShape<D>::MINB)
   MlCol<RH> g[8];
   float nr[8];
   const float scale = 1.f / (float)D;
+  float mean = 0.f;                                  // tr J / D
+#pragma unroll 8
+  for (int i = 0; i < D; ++i) mean += X[3 * spread6(i)].x;
+  mean *= scale * scale;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int col = i < 4 ? 4 * wk + i : 4 * (NG - 1 - wk) + i - 4;
@@ -809,7 +819,7 @@ __global__ void __launch_bounds__(MlShape<D>::NT, MlShape<D>::MINB)
       const int r = 2 * (wl + h * LW);
       float4 x = *reinterpret_cast<const float4*>(X + (spread6(r) | (spread6(col) << 1)));
       x = make_float4(x.x * scale, x.y * scale, x.z * scale, x.w * scale);
-      g[i].x[h] = pk(x.x, x.z);
+      g[i].x[h] = pk(col == r ? x.x - mean : x.x, col == r + 1 ? x.z - mean : x.z);
       g[i].y[h] = pk(x.y, x.w);
       if (live) *reinterpret_cast<float4*>(vec + col * D + r) = x;      // J's columns, read again at the end
     }
@@ -825,8 +835,11 @@ __global__ void __launch_bounds__(MlShape<D>::NT, MlShape<D>::MINB)
   float fro = 0.f;
 #pragma unroll 8
   for (int i = 0; i < D; ++i) fro += nx[i];
-  // G = J / |J|_F + I: norms of order one whatever the block's scale
-  const float inv_fro = fro > 0.f ? 1.f / sqrtf(fro) : 0.f;
+  // G = H / |H|_F + I: norms of order one whatever the block's scale.  A block that is
+  // scalar to rounding, |H|_F <= 2^-24 |J|_F (|J|_F^2 = |H|_F^2 + D mean^2), or zero
+  // has the unit vectors
+  const bool scalar = fro <= 3.5527137e-15f * ((float)D * mean * mean);
+  const float inv_fro = scalar ? 0.f : 1.f / sqrtf(fro);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int col = i < 4 ? 4 * wk + i : 4 * (NG - 1 - wk) + i - 4;
@@ -883,7 +896,7 @@ __global__ void __launch_bounds__(MlShape<D>::NT, MlShape<D>::MINB)
     if (!go) break;
   }
   // unit eigenvectors v_k, in any order, and their eigenvalues as Rayleigh
-  // quotients of the block itself: |J|_F (|g_k| - 1) would carry the rounding
+  // quotients of the block itself: |H|_F (|g_k| - 1) would carry the rounding
   // of the rotations of columns of length one and more (three times the error)
   column_norms<D>(g, nr);
   S::sync();                      // the exchange buffer is free
@@ -895,7 +908,7 @@ __global__ void __launch_bounds__(MlShape<D>::NT, MlShape<D>::MINB)
 #pragma unroll
     for (int h = 0; h < RH; ++h) {
       const int r = 2 * (wl + h * LW);
-      if (fro == 0.f) {           // the zero block
+      if (scalar) {
         g[i].x[h] = pk(k == r ? 1.f : 0.f, k == r + 1 ? 1.f : 0.f);
         g[i].y[h] = pk(0.f, 0.f);
       } else {
