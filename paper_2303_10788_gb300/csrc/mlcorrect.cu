@@ -35,6 +35,7 @@
 //     eigenvectors with eigenvalues max(lambda - theta, 0), then T'_f(o, P);
 //     written to T_f, and a hub's operand (by preparation at its inputs) is
 //     rewritten in FP32.
+#include "fsum.hpp"
 #include "kernels.cuh"
 
 namespace ccs {
@@ -319,18 +320,11 @@ __global__ void __launch_bounds__(256, 3) ml_eig_kernel(DevPlan P, DevRes R, con
 }
 
 // One CTA per fragment: theta over its eigenvalue list, which stays in
-// registers up to 16 per thread.  A pass adds the kept values in compensated
-// FP32 (sum and lost low part, together beyond 40 bits) and only the warps'
-// sums in FP64: with FP64 adds and compares per value a pass was bound by the
-// FP64 units (16 fragments of 8192 values: 76 us in all, 25 us so).
+// registers up to 16 per thread.  A pass adds the kept values in three FP32
+// parts (no fewer bits than FP64) and only the warps' sums in FP64: with FP64
+// adds and compares per value a pass was bound by the FP64 units (16 fragments
+// of 8192 values: 76 us, 32 us so; a pair of FP32 parts, of fewer bits, 25 us).
 constexpr int kThetaThreads = 1024, kThetaRegs = 16;
-
-// sum += v, the lost low part kept in comp (Neumaier)
-__device__ __forceinline__ void ml_add(float& sum, float& comp, float v) {
-  const float t = sum + v;
-  comp += fabsf(sum) >= fabsf(v) ? (sum - t) + v : (v - t) + sum;
-  sum = t;
-}
 
 __global__ void __launch_bounds__(kThetaThreads) ml_threshold_kernel(DevPlan P, const MlFrag* __restrict__ fr,
                                                                      const float* __restrict__ scratch,
@@ -358,27 +352,29 @@ __global__ void __launch_bounds__(kThetaThreads) ml_threshold_kernel(DevPlan P, 
   // loop should rounding ever make it oscillate
   for (long long it = 0; it <= n + 1 && it < 4096; ++it) {
     const float cut = __double2float_rd(theta);      // v > theta exactly when v > cut, for a float v
-    float s = 0.f, c = 0.f;
+    Sum3 s;
     int cnt = 0;
     if (in_regs) {
 #pragma unroll
       for (int i = 0; i < kThetaRegs; ++i)
-        if (v[i] > cut) { ml_add(s, c, v[i]); ++cnt; }
+        if (v[i] > cut) { s.add(v[i]); ++cnt; }
     } else {
 #pragma unroll 4
       for (long long i = tid; i < n; i += kThetaThreads) {
         const float x = ev[i];
-        if (x > cut) { ml_add(s, c, x); ++cnt; }
+        if (x > cut) { s.add(x); ++cnt; }
       }
     }
     for (int o = 16; o > 0; o >>= 1) {
-      const float so = __shfl_xor_sync(0xffffffffu, s, o), co = __shfl_xor_sync(0xffffffffu, c, o);
-      ml_add(s, c, so);
-      c += co;
+      Sum3 other;
+      other.s = __shfl_xor_sync(0xffffffffu, s.s, o);
+      other.c = __shfl_xor_sync(0xffffffffu, s.c, o);
+      other.e = __shfl_xor_sync(0xffffffffu, s.e, o);
+      s.add(other);
     }
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) {
-      s_sum[warp] = (double)s + (double)c;
+      s_sum[warp] = s.value();
       s_cnt[warp] = cnt;
     }
     __syncthreads();
