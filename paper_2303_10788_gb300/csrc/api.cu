@@ -427,8 +427,8 @@ struct ccs_res_s {
   int cliff_words = 1;        // words per op per thread in the tableau kernel
   int sample_spc = 4096;
   int hub_threads = 512;      // threads of the fused hub sampler CTA (either counter width)
-  bool hub_bytes = false;     // use the byte-counter hub sampler (64 KB of counters at |A| = 16; at 128
-                              // threads the 4-bit-counter one, while it applies)
+  bool hub_bytes = false;     // use the byte-counter hub sampler (64 KB of counters at |A| = 16)
+  bool hub_nibble = false;    // with hub_bytes: the 4-bit-counter one, while it applies
   int2* nibble_list = nullptr;   // variants the 4-bit counters leave to the byte counters
   bool variant_path = false;  // autotuned: every variant simulates its whole circuit (small plans)
   float* scratch = nullptr;   // recombination: R operand + split-K partials
@@ -1444,7 +1444,8 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
       stage_begin(c, ST_SAMPLE);
       if ((err = launch_sample_hub(dp, r->dr, e, p->d_items_hub, p->n_items_hub, p->max_hub_nA, r->hub_threads,
                                    e.keep_tableaus, p->hub_bytes_ok && r->hub_bytes,
-                                   nibble_ok(p, e.shots) ? r->nibble_list : nullptr, c->sm_count, s)) != cudaSuccess)
+                                   r->hub_nibble && nibble_ok(p, e.shots) ? r->nibble_list : nullptr, c->sm_count,
+                                   s)) != cudaSuccess)
         return cuda_fail(c, err, "hub sample kernel");
       if ((err = launch_sample(dp, r->dr, e, p->d_items_plain, p->n_items_plain, r->sample_spc, 256, s)) !=
           cudaSuccess)
@@ -1480,6 +1481,7 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
 // evaluations each) and keep the fastest; cached per shape bucket (widest
 // Clifford fragment rounded up to 64 wires, Clifford variant count rounded up
 // to a power of two, shots, mode).
+constexpr int kTunedNibble = -128;           // hub sampler of a tuned shape: the 4-bit-counter one
 constexpr int kVariantPathMaxItems = 8192;   // Clifford variants up to which the autotuner also times the per-variant path
 
 static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
@@ -1494,8 +1496,9 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
   if (it != c->tuned.end()) {
     int vp = 0;
     std::tie(r->cliff_threads, r->cliff_words, r->sample_spc, r->hub_threads, vp) = it->second;
-    r->hub_bytes = r->hub_threads < 0;       // cached as minus the threads of the byte-counter kernel
-    r->hub_threads = std::abs(r->hub_threads);
+    r->hub_bytes = r->hub_threads < 0;       // cached as minus the threads of the byte-counter kernel, or kTunedNibble
+    r->hub_nibble = r->hub_threads == kTunedNibble;
+    r->hub_threads = r->hub_nibble ? 256 : std::abs(r->hub_threads);
     r->variant_path = vp != 0;
     if (r->variant_path) { r->ep.shared_body = 0; r->ep.screen = 0; }
     return CCS_OK;
@@ -1519,7 +1522,7 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
   const int threads_c[] = {128, 256, 512};
   const int words_c[] = {1, 2, 4, 8};
   const int spc_c[] = {1024, 2048, 4096, 8192};
-  const int hub_c[] = {128, 512, 256, 512, 128};  // 16-bit counters, byte counters, 4-bit counters
+  const int hub_c[] = {128, 512, 256, 512, 256};  // 16-bit counters, byte counters, 4-bit counters (its rest by bytes)
   const int max_w = 2 * ((max_n + 63) / 64);
   const bool sampled = r->ep.mode == CCS_SAMPLED;
   int rc = CCS_OK;
@@ -1542,17 +1545,19 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
     if ((rc = time_it(&ms)) == CCS_OK && ms < best) { best = ms; bs = spc_c[si]; }
   }
   r->sample_spc = bs;
-  bool bb = r->hub_bytes;
+  bool bb = r->hub_bytes, bn = r->hub_nibble;
   for (int hi = 0; sampled && p->n_items_hub && hi < 5 && rc == CCS_OK; ++hi) {
     const bool bytes = hi >= 2;
     if (bytes && !p->hub_bytes_ok) continue;
     if (hi == 4 && !nibble_ok(p, r->ep.shots)) continue;
     r->hub_bytes = bytes;
+    r->hub_nibble = hi == 4;
     r->hub_threads = hub_c[hi];
-    if ((rc = time_it(&ms)) == CCS_OK && ms < best) { best = ms; bh = hub_c[hi]; bb = bytes; }
+    if ((rc = time_it(&ms)) == CCS_OK && ms < best) { best = ms; bh = hub_c[hi]; bb = bytes; bn = hi == 4; }
   }
   r->hub_threads = bh;
   r->hub_bytes = bb;
+  r->hub_nibble = bn;
   // Small plans whose tableaus fit in shared memory: the per-variant path
   // (every variant simulates its whole circuit in one kernel, no shared-body
   // chain) can be faster than the shared body's chain of short kernels; it
@@ -1587,7 +1592,7 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != CCS_OK) return rc;
-  c->tuned[key] = std::make_tuple(bt, bw, bs, bb ? -bh : bh, r->variant_path ? 1 : 0);
+  c->tuned[key] = std::make_tuple(bt, bw, bs, bn ? kTunedNibble : bb ? -bh : bh, r->variant_path ? 1 : 0);
   return CCS_OK;
 }
 
@@ -1595,7 +1600,8 @@ int ccs_get_tuning(ccs_ctx c, ccs_res r, int* cliff_threads, int* words_per_op, 
                    int* hub_threads, int* variant_path) {
   return abi_guard([&](int code, const char* m) { return fail(c, code, m); }, [&]() -> int {
     if (!c || !r) return fail(c, CCS_ERR_INVALID_ARG, "bad arguments");
-    if (hub_threads) *hub_threads = (r->hub_bytes && r->plan->hub_bytes_ok) ? -r->hub_threads : r->hub_threads;
+    if (hub_threads)
+      *hub_threads = !(r->hub_bytes && r->plan->hub_bytes_ok) ? r->hub_threads : r->hub_nibble ? -128 : -r->hub_threads;
     if (variant_path) *variant_path = r->ep.shared_body ? 0 : 1;
     if (cliff_threads) *cliff_threads = r->cliff_threads;
     if (words_per_op) *words_per_op = r->ep.shared_body ? 1 : r->cliff_words;
@@ -1658,9 +1664,8 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
         // small hub CTAs when a variant has few shots and few outputs (more CTAs per SM);
         // byte counters when the histogram would otherwise fill an SM's shared memory
         r->hub_bytes = p->hub_bytes_ok && p->max_hub_nA >= 13;
-        r->hub_threads = r->hub_bytes && nibble_ok(p, opts->shots) ? 128
-                         : r->hub_bytes                            ? 256
-                         : (p->max_hub_nA <= 12 && opts->shots <= 4096) ? 128 : 512;
+        r->hub_nibble = r->hub_bytes && nibble_ok(p, opts->shots);
+        r->hub_threads = r->hub_bytes ? 256 : (p->max_hub_nA <= 12 && opts->shots <= 4096) ? 128 : 512;
       }
       if (p->rt_total) {
         d.TQh = r->A.get<uint16_t>(p->n_T);
@@ -1730,6 +1735,7 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
     }
     if (opts->hub_sampler >= 2) {
       r->hub_bytes = p->hub_bytes_ok;
+      r->hub_nibble = false;
       r->hub_threads = opts->hub_sampler == 3 ? 512 : 256;
     }
     e.inv_shots = e.shots ? 1.0 / (double)e.shots : 0.0;

@@ -2427,7 +2427,7 @@ cudaError_t launch_sample_hub(const DevPlan& p, const DevRes& r, const EvalParam
                               int max_nA, int threads, int keep_counts, bool bytes_ok, int2* nibble_list,
                               int sm_count, cudaStream_t s) {
   if (n_items == 0 || e.shots == 0) return cudaSuccess;
-  if (bytes_ok && threads == kHub4Threads && nibble_list) {
+  if (bytes_ok && nibble_list) {
     const int words = std::max(1, (1 << max_nA) / 8), bytes = 1 << max_nA;
     cudaError_t err =
         cudaFuncSetAttribute(sample_hub4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * words);

@@ -236,7 +236,7 @@ cudaError_t launch_sample(const DevPlan& p, const DevRes& r, const EvalParams& e
 // hub's contraction operand Q into TQ, and dense counts if keep_counts.
 // bytes_ok: every hub has >= 2 marginal bits, <= 4 quantum outputs and |A| <= 16
 // (the byte-counter kernel applies); nibble_list: room for n_items records when
-// the 4-bit-counter kernel applies too (used at 128 threads), else NULL
+// the 4-bit-counter kernel is to be used, else NULL
 cudaError_t launch_sample_hub(const DevPlan& p, const DevRes& r, const EvalParams& e, const int2* items,
                               int n_items, int max_nA, int threads, int keep_counts, bool bytes_ok, int2* nibble_list,
                               int sm_count, cudaStream_t s);
