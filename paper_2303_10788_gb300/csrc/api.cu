@@ -419,7 +419,7 @@ struct ccs_res_s {
   cudaGraphExec_t graph = nullptr;
   long long graph_launches = 0;   // kernel nodes of the captured graph
   cudaGraphExec_t rgraph = nullptr;   // recombination graph
-  int rgraph_key = -1;
+  long long rgraph_key = -1;
   long long rgraph_launches = 0;
   EvalParams graph_key{};
   int graph_valid = 0;
@@ -1833,7 +1833,8 @@ int ccs_recombine(ccs_ctx c, ccs_plan p, ccs_res r, const ccs_recomb_opts* opts,
     }
     cudaError_t e;
     if (opts && opts->use_graph && !c->profiling && rz.krange.full()) {
-      const int key = prec * 2 + (tc ? 1 : 0) + (stitched ? 4 : 0) + (r->dr.hub_i16 ? 8 : 0);
+      // the scale of 16-bit count sums (1 / shots) is a captured launch argument
+      const long long key = prec * 2 + (tc ? 1 : 0) + (stitched ? 4 : 0) + (r->dr.hub_i16 ? 8 + 16ll * r->ep.shots : 0);
       if (!r->rgraph || r->rgraph_key != key) {
         if (r->rgraph) { cudaGraphExecDestroy(r->rgraph); r->rgraph = nullptr; }
         cudaStream_t s = c->stream;
