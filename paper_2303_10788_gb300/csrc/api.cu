@@ -34,7 +34,7 @@ struct ccs_ctx_s {
   std::string err;
   ccs_mpnn cut_model = nullptr;   // learned cut scorer (not owned)
   // autotuner results: shape bucket -> (Clifford threads per CTA, shots per sampler CTA)
-  std::map<std::tuple<int, int, unsigned, int>, std::tuple<int, int, int, int, int>> tuned;
+  std::map<std::tuple<int, int, unsigned, int, int>, std::tuple<int, int, int, int, int>> tuned;
   // second stream for the statevector branch (forked from / joined into `stream`)
   cudaStream_t side = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
@@ -1480,7 +1480,8 @@ static int enqueue_eval(ccs_ctx c, ccs_plan p, ccs_res r) {
 // candidate on this plan with CUDA events (one warm-up + three timed
 // evaluations each) and keep the fastest; cached per shape bucket (widest
 // Clifford fragment rounded up to 64 wires, Clifford variant count rounded up
-// to a power of two, shots, mode).
+// to a power of two, shots, mode, hubs of 13 measured bits or more, the counters
+// the hubs can use).
 constexpr int kTunedNibble = -128;           // hub sampler of a tuned shape: the 4-bit-counter one
 constexpr int kVariantPathMaxItems = 8192;   // Clifford variants up to which the autotuner also times the per-variant path
 
@@ -1490,8 +1491,10 @@ static int autotune(ccs_ctx c, ccs_plan p, ccs_res r) {
     if (f.clifford) max_n = std::max(max_n, f.n);
   int items = 1;
   while (items < p->dp.n_items_cliff) items <<= 1;
-  const auto key =
-      std::make_tuple((max_n + 63) / 64, items, r->ep.shots, r->ep.mode * 4 + r->ep.shared_body * 2 + r->ep.screen);
+  // (the hubs decide which samplers there are to choose from)
+  const int hubs = (p->max_hub_nA >= 13 ? 4 : 0) + (p->hub_bytes_ok ? 2 : 0) + (nibble_ok(p, r->ep.shots) ? 1 : 0);
+  const auto key = std::make_tuple((max_n + 63) / 64, items, r->ep.shots,
+                                   r->ep.mode * 4 + r->ep.shared_body * 2 + r->ep.screen, hubs);
   auto it = c->tuned.find(key);
   if (it != c->tuned.end()) {
     int vp = 0;
@@ -1600,8 +1603,12 @@ int ccs_get_tuning(ccs_ctx c, ccs_res r, int* cliff_threads, int* words_per_op, 
                    int* hub_threads, int* variant_path) {
   return abi_guard([&](int code, const char* m) { return fail(c, code, m); }, [&]() -> int {
     if (!c || !r) return fail(c, CCS_ERR_INVALID_ARG, "bad arguments");
-    if (hub_threads)
-      *hub_threads = !(r->hub_bytes && r->plan->hub_bytes_ok) ? r->hub_threads : r->hub_nibble ? -128 : -r->hub_threads;
+    if (hub_threads) {   // of the last evaluation: its shots may rule narrow counters out
+      const bool sampled = r->ep.mode == CCS_SAMPLED;
+      const bool bytes = r->hub_bytes && r->plan->hub_bytes_ok && !(sampled && r->ep.shots > 0xffffu);
+      const bool nibble = bytes && r->hub_nibble && !(sampled && !nibble_ok(r->plan, r->ep.shots));
+      *hub_threads = nibble ? -128 : bytes ? -r->hub_threads : r->hub_threads;
+    }
     if (variant_path) *variant_path = r->ep.shared_body ? 0 : 1;
     if (cliff_threads) *cliff_threads = r->cliff_threads;
     if (words_per_op) *words_per_op = r->ep.shared_body ? 1 : r->cliff_words;

@@ -48,6 +48,28 @@ def test_forced_16_bit_counters_take_512_threads(sparse):
     assert evaluate(sparse, shots=4096, hub_sampler=1) == 512
 
 
+@pytest.mark.parametrize("shots,want", [(32767, -128), (32768, -256), (65535, -256), (65536, 256)])
+def test_reported_counters_are_those_of_the_last_evaluation(sparse, shots, want):
+    """13 measured bits: 4-bit counters up to four shots per outcome and 32767
+    shots, byte counters up to 65535."""
+    assert evaluate(sparse, shots=shots) == want
+
+
+def test_tuned_shapes_are_kept_per_kind_of_hub():
+    """Two plans of one shape bucket, the second's hub too narrow for byte and
+    4-bit counters: it is tuned for itself, and reports neither."""
+    ctx = ccs.ccs_create(0)
+    launches = []
+    for m in (11, 1, 1):
+        plan = ccs.ccs_build_fragments(ctx, [star(m)])
+        before = ccs.ccs_launch_count()
+        res = ccs.ccs_eval_variants(ctx, plan, mode=ccs.CCS_SAMPLED, shots=4096, autotune=True)
+        launches.append(ccs.ccs_launch_count() - before)
+    assert ccs.ccs_get_tuning(ctx, res)[3] > 0
+    # the third takes the second's shape from the cache: one evaluation's launches
+    assert launches[1] > 4 * launches[2] > 0
+
+
 def test_narrow_hubs_keep_128_threads():
     ctx = ccs.ccs_create(0)
     plan = ccs.ccs_build_fragments(ctx, [star(8)])
