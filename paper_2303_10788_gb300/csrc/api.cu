@@ -352,6 +352,7 @@ bool upload(ccs_ctx c, Allocs& A, const std::vector<T>& h, T** out) {
 // hold (512 MB; a problem beyond that is summed directly).
 constexpr double kTreeSmallWork = 1 << 16;
 constexpr long long kTreeTmpMax = 1ll << 26;
+constexpr int kTreeLogThreads = 17;   // threads (log2) a step's entries are split up to
 
 struct ccs_plan_s {
   ccs_ctx ctx = nullptr;
@@ -1252,8 +1253,11 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     std::vector<std::vector<long long>> tree_prefix(tree_sets.size(), std::vector<long long>{0});
     for (size_t l = 0; l < tree_sets.size(); ++l)
       for (int i : tree_sets[l]) {
-        const GStep& g = plan->gsteps[i];
-        tree_prefix[l].push_back(tree_prefix[l].back() + (1ll << (g.ma + g.mb + 2 * (g.fa + g.fb))));
+        GStep& g = plan->gsteps[i];
+        const int le = g.ma + g.mb + 2 * (g.fa + g.fb);
+        // at least four terms a lane, a CTA per entry at most, and no more than the chip's threads
+        g.lg = std::max(0, std::min({8, 2 * g.ns - 2, kTreeLogThreads - le}));
+        tree_prefix[l].push_back(tree_prefix[l].back() + ((((1ll << (le + g.lg)) + 255) >> 8) << 8));
       }
     std::vector<int*> d_tree_ids(tree_sets.size());
     std::vector<long long*> d_tree_prefix(tree_sets.size());

@@ -89,6 +89,7 @@ struct GStep {
   int a_tmp, b_tmp;                 // 1: in gtmp
   int ma, mb, fa, fb, ns;           // marginal bits; free and shared cut digits
   int na, nb;                       // digits of A's and of B's index (fa + ns, fb + ns)
+  int lg;                           // 2^lg threads sum an entry of a step launched by level
   int za, zb, zo;                   // offsets of A, B and the result among the Z-string tensors (no marginal bits)
   long long a_off, b_off, out_off;
   uint8_t a_free[kMaxCuts], a_sh[kMaxCuts], b_free[kMaxCuts], b_sh[kMaxCuts];   // digit positions

@@ -1120,6 +1120,27 @@ __device__ __forceinline__ long long spread(long long v, int nd, const uint8_t* 
   return p;
 }
 
+// Lanes (log2) that share an entry's sum over ns cut digits when a CTA of
+// 2^log_threads threads has 2^log_entries entries: at least four terms each.
+__device__ __forceinline__ int tree_lanes(int log_threads, int log_entries, int ns) {
+  return max(0, min(log_threads - log_entries, 2 * ns - 2));
+}
+// The sum over an entry's 2^lg lanes (consecutive threads, lg the same for the
+// whole CTA) in a fixed order, on the entry's first lane.  Above a warp it passes
+// through red, an entry per warp, and every thread of the CTA must call it.
+__device__ __forceinline__ double lanes_sum(double v, int lg, double* red) {
+  for (int o = min(16, (1 << lg) >> 1); o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lg > 5) {
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) red[w] = v;
+    __syncthreads();
+    if ((threadIdx.x & ((1 << lg) - 1)) == 0)
+      for (int i = 1; i < (1 << (lg - 5)); ++i) v += red[w + i];
+    __syncthreads();
+  }
+  return v;
+}
+
 // T_f^S(zi, P) folded from the variants' Z-string values the way T_f is
 // folded from their distributions: the preparation tuples of P's input
 // Paulis (weights mu) at the output bases of P's output Paulis, each taking
@@ -1180,12 +1201,18 @@ __device__ __noinline__ void z_string_block(const DevPlan& P, const DevRes& R, c
     for (int t = 0; t < Pb.g_count; ++t) {
       __syncthreads();
       const GStep& G = P.gsteps[Pb.g_first + t];
-      for (int e = threadIdx.x; e < (1 << (2 * (G.fa + G.fb))); e += blockDim.x) {
-        const int ia = (int)spread(e & ((1 << (2 * G.fa)) - 1), G.fa, G.a_free);
-        const int ib = (int)spread(e >> (2 * G.fa), G.fb, G.b_free);
+      const int le = 2 * (G.fa + G.fb), lg = tree_lanes(9, le, G.ns);      // 512 threads
+      for (int g = threadIdx.x; g < (blockDim.x > (1u << le) ? (int)blockDim.x : 1 << le); g += blockDim.x) {
+        const int e = g >> lg;
         double acc = 0.0;
-        for (int q = 0; q < (1 << (2 * G.ns)); ++q)
-          acc = fma(zt[G.za + (ia | (int)spread(q, G.ns, G.a_sh))], zt[G.zb + (ib | (int)spread(q, G.ns, G.b_sh))], acc);
+        if (e < (1 << le)) {
+          const int ia = (int)spread(e & ((1 << (2 * G.fa)) - 1), G.fa, G.a_free);
+          const int ib = (int)spread(e >> (2 * G.fa), G.fb, G.b_free);
+          for (int q = g & ((1 << lg) - 1); q < (1 << (2 * G.ns)); q += 1 << lg)
+            acc = fma(zt[G.za + (ia | (int)spread(q, G.ns, G.a_sh))], zt[G.zb + (ib | (int)spread(q, G.ns, G.b_sh))], acc);
+        }
+        acc = lanes_sum(acc, lg, red);
+        if (e >= (1 << le) || (g & ((1 << lg) - 1))) continue;
         if (G.last) zexp_out[Pb.zexp_off + zi] = ldexp(acc, -S.k);
         else zt[G.zo + e] = acc;
       }
@@ -1543,10 +1570,14 @@ cudaError_t launch_fold(const DevPlan& p, const DevRes& r, const EvalParams& e, 
 // whole call went from 2.09 to 0.11 ms).  The steps are short sums over few
 // shared digits, so they are bound by launch and load latency; FP64 throughout
 // costs nothing there, and leaves only the tensors' own FP32 rounding.
+// Two fragments with many cuts between them make the sum long and the entries
+// few, so that up to a CTA's threads share an entry (recombination of a pair
+// joined by four cuts beside another pair: 254 us with one thread per entry,
+// 95 us so).
 __device__ __forceinline__ double tree_sum(const GStep& S, const float* __restrict__ T, const double* tmp, bool bf16,
-                                           long long ia, long long ib) {
+                                           long long ia, long long ib, int lane, int lg) {
   double acc = 0.0;
-  for (int s = 0; s < (1 << (2 * S.ns)); ++s) {
+  for (int s = lane; s < (1 << (2 * S.ns)); s += 1 << lg) {
     const long long xa = S.a_off + (ia | spread(s, S.ns, S.a_sh)), xb = S.b_off + (ib | spread(s, S.ns, S.b_sh));
     double a, b;
     if (S.a_tmp) a = tmp[xa];
@@ -1558,43 +1589,56 @@ __device__ __forceinline__ double tree_sum(const GStep& S, const float* __restri
   return acc;
 }
 
-// Entry e of a step: into gtmp, or (the last one) the marginal, e its index.
-__device__ __forceinline__ void tree_entry(const DevPlan& P, const DevRes& R, const GStep& S, bool bf16, long long e,
-                                           double* marg_out) {
-  if (!S.last) {
-    const int fd = 2 * (S.fa + S.fb);
-    const long long pf = e & ((1ll << fd) - 1), o = e >> fd;
-    const long long pa = pf & ((1ll << (2 * S.fa)) - 1), pb = pf >> (2 * S.fa);
-    const long long oa = o & ((1ll << S.ma) - 1), ob = o >> S.ma;
-    R.gtmp[S.out_off + e] = tree_sum(S, R.T, R.gtmp, bf16, (oa << (2 * S.na)) | spread(pa, S.fa, S.a_free),
-                                     (ob << (2 * S.nb)) | spread(pb, S.fb, S.b_free));
-    return;
+// Thread g of a step whose entries take 2^lg lanes each: entry g >> lg, into gtmp
+// or (the last step) the marginal, where the entry is its index.
+__device__ __forceinline__ void tree_entry(const DevPlan& P, const DevRes& R, const GStep& S, bool bf16, long long g,
+                                           int lg, double* red, double* marg_out) {
+  const long long e = g >> lg;
+  const int lane = (int)g & ((1 << lg) - 1), fd = 2 * (S.fa + S.fb);
+  const bool in = e < (1ll << (S.ma + S.mb + fd));
+  double acc = 0.0;
+  if (in) {
+    long long oa = 0, ob = 0, pa = 0, pb = 0;
+    if (S.last) {
+      for (int j = 0; j < S.ma; ++j) oa |= ((e >> S.pos[j]) & 1) << j;
+      for (int j = 0; j < S.mb; ++j) ob |= ((e >> S.pos[S.ma + j]) & 1) << j;
+    } else {
+      const long long pf = e & ((1ll << fd) - 1), o = e >> fd;
+      pa = spread(pf & ((1ll << (2 * S.fa)) - 1), S.fa, S.a_free);
+      pb = spread(pf >> (2 * S.fa), S.fb, S.b_free);
+      oa = o & ((1ll << S.ma) - 1);
+      ob = o >> S.ma;
+    }
+    acc = tree_sum(S, R.T, R.gtmp, bf16, (oa << (2 * S.na)) | pa, (ob << (2 * S.nb)) | pb, lane, lg);
   }
-  long long oa = 0, ob = 0;
-  for (int j = 0; j < S.ma; ++j) oa |= ((e >> S.pos[j]) & 1) << j;
-  for (int j = 0; j < S.mb; ++j) ob |= ((e >> S.pos[S.ma + j]) & 1) << j;
-  const ProblemDev& Pb = P.problems[S.problem];
-  marg_out[Pb.marg_off + e] = ldexp(tree_sum(S, R.T, R.gtmp, bf16, oa << (2 * S.na), ob << (2 * S.nb)), -Pb.k);
+  if (lg) acc = lanes_sum(acc, lg, red);
+  if (!in || lane) return;
+  if (S.last) marg_out[P.problems[S.problem].marg_off + e] = ldexp(acc, -P.problems[S.problem].k);
+  else R.gtmp[S.out_off + e] = acc;
 }
 
-// One launch of independent steps (FoldSet: fidx = step, t_prefix = entries).
+// One launch of independent steps (FoldSet: fidx = step, t_prefix = threads, a
+// multiple of a CTA's for each step).
 __global__ void __launch_bounds__(256) tree_level_kernel(DevPlan P, DevRes R, int precision, FoldSet f,
                                                          double* marg_out) {
-  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < f.total;
-       g += (long long)gridDim.x * blockDim.x) {
-    const int i = find_seg(f.t_prefix, f.nf, g);
-    tree_entry(P, R, P.gsteps[f.fidx[i]], precision == CCS_BF16, g - f.t_prefix[i], marg_out);
+  __shared__ double red[8];
+  for (long long b = blockIdx.x * 256ll; b < f.total; b += gridDim.x * 256ll) {
+    const int i = find_seg(f.t_prefix, f.nf, b);
+    const GStep& S = P.gsteps[f.fidx[i]];
+    tree_entry(P, R, S, precision == CCS_BF16, b + threadIdx.x - f.t_prefix[i], S.lg, red, marg_out);
   }
 }
 
 // Every step but the last of one small problem, by one CTA: the steps follow
 // each other at a block barrier instead of a launch.
 __global__ void __launch_bounds__(512) tree_small_kernel(DevPlan P, DevRes R, int precision, const int* problems) {
+  __shared__ double red[16];
   const ProblemDev& Pb = P.problems[problems[blockIdx.x]];
   for (int i = 0; i + 1 < Pb.g_count; ++i) {
     const GStep& S = P.gsteps[Pb.g_first + i];
-    const long long n = 1ll << (S.ma + S.mb + 2 * (S.fa + S.fb));
-    for (long long e = threadIdx.x; e < n; e += blockDim.x) tree_entry(P, R, S, precision == CCS_BF16, e, nullptr);
+    const int le = S.ma + S.mb + 2 * (S.fa + S.fb), lg = tree_lanes(9, le, S.ns);
+    for (long long b = 0; b < (1ll << (le + lg)); b += 512)
+      tree_entry(P, R, S, precision == CCS_BF16, b + threadIdx.x, lg, red, nullptr);
     __syncthreads();
   }
 }
