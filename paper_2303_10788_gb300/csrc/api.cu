@@ -346,11 +346,13 @@ bool upload(ccs_ctx c, Allocs& A, const std::vector<T>& h, T** out) {
 
 }  // namespace
 
-// Tree contractions: a problem's steps but the last run in one CTA up to this
-// many multiply-adds (512 threads, a few microseconds; a level launched on its
-// own costs about as much), and the doubles of intermediate tensors a plan may
+// Tree contractions: a problem's steps run in one CTA, beside the Z-strings, up to
+// this many multiply-adds (512 threads, a few microseconds) and outputs (an output
+// takes a thread 1.3 us: 2^14 of them 62 us there, 5 us in a launch of their own),
+// or all steps but the last do; and the doubles of intermediate tensors a plan may
 // hold (512 MB; a problem beyond that is summed directly).
 constexpr double kTreeSmallWork = 1 << 16;
+constexpr int kTreeSmallMarg = 11;
 constexpr long long kTreeTmpMax = 1ll << 26;
 constexpr int kTreeLogThreads = 17;   // threads (log2) a step's entries are split up to
 
@@ -401,8 +403,8 @@ struct ccs_plan_s {
   bool all_star = true;             // no problem is summed over its whole cut index for every output
   std::vector<GStep> gsteps;        // tree contractions (problems that are no stars)
   std::vector<FoldSet> tree_levels;
-  int* d_tree_small = nullptr;
-  int n_tree_small = 0;
+  int *d_tree_small = nullptr, *d_tree_whole = nullptr;
+  int n_tree_small = 0, n_tree_whole = 0;
   long long n_gtmp = 0;             // doubles of their intermediate tensors
   ~ccs_plan_s() { A.release(); }
 };
@@ -1052,7 +1054,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       if (f.role == 2 && !f.clifford) { fidx_on.push_back(fi); tp_on.push_back(tp_on.back() + t); }
     }
     std::vector<long long> direct_per_m;       // floats per hub output of a star contracted leaf by leaf
-    std::vector<int> tree_level, tree_small;   // launch level of every step (-1: in the small problems' CTA)
+    std::vector<int> tree_level, tree_small, tree_whole;   // launch level of every step (-1: in the problem's own CTA)
     for (auto& P : plan->problems) {
       ProblemDev d{};
       d.k = (int)P.cuts.size();
@@ -1081,13 +1083,16 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
                       tree_level, plan->n_gtmp, d.g_zlen)) {
           d.g_first = (int)g0;
           d.g_count = (int)(plan->gsteps.size() - g0);
-          // few multiply-adds in all steps but the last: one CTA runs them
-          double work = 0.0;
-          for (size_t i = g0; i + 1 < plan->gsteps.size(); ++i) {
+          // few multiply-adds in all steps, or all but the last: one CTA runs them
+          double work = 0.0, last = 0.0;
+          for (size_t i = g0; i < plan->gsteps.size(); ++i) {
             const GStep& g = plan->gsteps[i];
-            work += std::ldexp(1.0, g.ma + g.mb + 2 * (g.fa + g.fb + g.ns));
+            work += last = std::ldexp(1.0, g.ma + g.mb + 2 * (g.fa + g.fb + g.ns));
           }
-          if (work <= kTreeSmallWork) {
+          if (work <= kTreeSmallWork && d.n_marg <= kTreeSmallMarg) {
+            tree_whole.push_back((int)plan->pdev.size());
+            for (size_t i = g0; i < plan->gsteps.size(); ++i) tree_level[i] = -1;
+          } else if (work - last <= kTreeSmallWork && d.g_count > 1) {
             tree_small.push_back((int)plan->pdev.size());
             for (size_t i = g0; i + 1 < plan->gsteps.size(); ++i) tree_level[i] = -1;
           }
@@ -1245,10 +1250,10 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
         if ((int)tree_sets.size() <= tree_level[i]) tree_sets.resize(tree_level[i] + 1);
         tree_sets[tree_level[i]].push_back((int)i);
       }
-    if (!plan->gsteps.empty()) {
+    if (tree_whole.size() < (size_t)std::count_if(plan->gsteps.begin(), plan->gsteps.end(), [](const GStep& g) { return g.last; })) {
       tree_sets.emplace_back();
       for (size_t i = 0; i < plan->gsteps.size(); ++i)
-        if (plan->gsteps[i].last) tree_sets.back().push_back((int)i);
+        if (plan->gsteps[i].last && tree_level[i] >= 0) tree_sets.back().push_back((int)i);
     }
     std::vector<std::vector<long long>> tree_prefix(tree_sets.size(), std::vector<long long>{0});
     for (size_t l = 0; l < tree_sets.size(); ++l)
@@ -1309,7 +1314,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     st.add(plan->blk_prefix, &plan->d_blk_prefix); st.add(plan->direct_items, &plan->d_direct_items);
     GStep* dgs = nullptr;
     if (!plan->gsteps.empty()) {
-      st.add(plan->gsteps, &dgs); st.add(tree_small, &plan->d_tree_small);
+      st.add(plan->gsteps, &dgs); st.add(tree_small, &plan->d_tree_small); st.add(tree_whole, &plan->d_tree_whole);
       for (size_t l = 0; l < tree_sets.size(); ++l) {
         st.add(tree_sets[l], &d_tree_ids[l]);
         st.add(tree_prefix[l], &d_tree_prefix[l]);
@@ -1319,6 +1324,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
     if (!ok) { return fail(c, CCS_ERR_OOM, "plan upload failed"); }
     plan->dp.gsteps = dgs;
     plan->n_tree_small = (int)tree_small.size();
+    plan->n_tree_whole = (int)tree_whole.size();
     for (size_t l = 0; l < tree_sets.size(); ++l)
       plan->tree_levels.push_back(FoldSet{d_tree_ids[l], d_tree_prefix[l], (int)tree_sets[l].size(),
                                           tree_prefix[l].back()});
@@ -1836,7 +1842,7 @@ int ccs_recombine(ccs_ctx c, ccs_plan p, ccs_res r, const ccs_recomb_opts* opts,
                    p->d_r_prefix, p->d_blk_prefix, p->d_out_prefix, p->d_z_prefix, p->max_tile_smem,
                    p->pdev.data(), (int)p->pdev.size(), r->rt_scratch, tc ? 1 : 0, stitched ? 1 : 0, KRange{0, -1},
                    p->all_star ? 0 : 1, p->tree_levels.data(), (int)p->tree_levels.size(), p->d_tree_small,
-                   p->n_tree_small};
+                   p->n_tree_small, p->d_tree_whole, p->n_tree_whole};
     if (opts && (opts->k_lo || opts->k_hi)) {
       if (opts->k_hi && opts->k_hi <= opts->k_lo) return fail(c, CCS_ERR_INVALID_ARG, "empty cut-index range");
       if (opts->k_lo > (1ull << 62) || opts->k_hi > (1ull << 62)) return fail(c, CCS_ERR_INVALID_ARG, "bad range");
@@ -2253,7 +2259,7 @@ extern "C" int ccs_recombine_noalloc(ccs_ctx c, ccs_plan p, ccs_res r, int preci
                    p->d_r_prefix, p->d_blk_prefix, p->d_out_prefix, p->d_z_prefix, p->max_tile_smem,
                    p->pdev.data(), (int)p->pdev.size(), nullptr, 0, r->ep.mode == CCS_STITCH ? 1 : 0,
                    KRange{0, -1}, p->all_star ? 0 : 1, p->tree_levels.data(), (int)p->tree_levels.size(), p->d_tree_small,
-                   p->n_tree_small};
+                   p->n_tree_small, p->d_tree_whole, p->n_tree_whole};
     e = launch_recombine(p->dp, r->dr, precision, rz, scratch, marginal_out, zexp_out, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "recombine kernel");
     return CCS_OK;

@@ -328,6 +328,8 @@ struct RecombSizes {
   int n_tree_levels;             //    step of every problem is in the final entry
   const int* tree_small;         // device list: problems whose steps but the last run in one CTA each
   int n_tree_small;
+  const int* tree_whole;         // device list: problems whose steps all run in one CTA each
+  int n_tree_whole;
 };
 cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, const RecombSizes& z,
                              float* scratch, double* marg_out, double* zexp_out, cudaStream_t s);

@@ -1141,6 +1141,18 @@ __device__ __forceinline__ double lanes_sum(double v, int lg, double* red) {
   return v;
 }
 
+// The steps of a tree contraction, read into shared memory at once (a step is a
+// chain of dependent loads otherwise): behind the 16 sums of red, 4 KB in all.
+constexpr int kRedDoubles = 512;
+static_assert((kRedDoubles - 16) * sizeof(double) >= (kMaxProblemFragments - 1) * sizeof(GStep), "steps behind the sums");
+__device__ __forceinline__ GStep* load_steps(const DevPlan& P, const ProblemDev& Pb, double* red) {
+  GStep* st = reinterpret_cast<GStep*>(red + 16);
+  const int* src = reinterpret_cast<const int*>(P.gsteps + Pb.g_first);
+  for (int i = threadIdx.x; i < Pb.g_count * (int)(sizeof(GStep) / 4); i += blockDim.x)
+    reinterpret_cast<int*>(st)[i] = src[i];
+  return st;
+}
+
 // T_f^S(zi, P) folded from the variants' Z-string values the way T_f is
 // folded from their distributions: the preparation tuples of P's input
 // Paulis (weights mu) at the output bases of P's output Paulis, each taking
@@ -1191,6 +1203,7 @@ __device__ __noinline__ void z_string_block(const DevPlan& P, const DevRes& R, c
   __syncthreads();
   if (Pb.g_zlen && kr.full()) {   // a tree of fragments: its contraction steps, without marginal bits
     double* zt = reinterpret_cast<double*>(s_tz);
+    GStep* st = load_steps(P, Pb, red);
     int tot = 0;
     for (int l = 0; l < S.nf; ++l) tot += 1 << (2 * S.ns[l]);
     for (int i = threadIdx.x; i < tot; i += blockDim.x) {
@@ -1200,7 +1213,7 @@ __device__ __noinline__ void z_string_block(const DevPlan& P, const DevRes& R, c
     }
     for (int t = 0; t < Pb.g_count; ++t) {
       __syncthreads();
-      const GStep& G = P.gsteps[Pb.g_first + t];
+      const GStep& G = st[t];
       const int le = 2 * (G.fa + G.fb), lg = tree_lanes(9, le, G.ns);      // 512 threads
       for (int g = threadIdx.x; g < (blockDim.x > (1u << le) ? (int)blockDim.x : 1 << le); g += blockDim.x) {
         const int e = g >> lg;
@@ -1512,55 +1525,6 @@ __device__ __forceinline__ void contract_item(const DevPlan& P, const DevRes& R,
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, int precision,
-                                                      const int2* direct_items, int n_direct, int stage_floats,
-                                                      const long long* z_prefix, int np, long long z_total, int z_warp,
-                                                      double* marg_out, double* zexp_out, KRange krg) {
-  extern __shared__ __align__(16) float s_buf[];   // two buffers of stage_floats
-  __shared__ double red[512];
-  __shared__ ProblemShared S;
-  __shared__ __align__(8) float s_T[kLeafStage];
-  const long long z_blocks = z_warp ? (z_total + 15) / 16 : z_total;
-  for (long long b = blockIdx.x; b < n_direct + z_blocks; b += gridDim.x) {
-    if (b >= n_direct && z_warp) {
-      const int w = threadIdx.x >> 5;
-      const long long g = (b - n_direct) * 16 + w;
-      if (g < z_total) z_string_warp(P, R, z_prefix, np, g, s_T + w * kZWarp, zexp_out, krg);
-      __syncthreads();
-      continue;
-    }
-    if (b >= n_direct) {
-      z_string_block(P, R, z_prefix, np, b - n_direct, S, red, s_T, kLeafStage, zexp_out, krg);
-      __syncthreads();
-      continue;
-    }
-    const int2 di = direct_items[b];
-    const ProblemDev& Pb = P.problems[di.x];
-    const int M = Pb.TM, lm = __ffs(M) - 1;      // this block's hub outputs; extents are powers of two
-    const int m0 = di.y * M, Mfull = Pb.M;
-    const int K = (int)Pb.K;
-    const long long klo = krg.lo_of(K), khi = krg.hi_of(K);   // cut-index terms summed
-    // the hub's Q stored transposed: K x Mfull, row-major (this slice's columns from m0),
-    // FP32 or int16 count sums: one branch per slice, none per element
-    const HubView hv = hub_view(R, P.frags[Pb.frag0 + Pb.hub], Pb.hub_T_off + m0);
-    if (hv.h)
-      contract_item(P, R, precision, Pb, hv.h, hv.scale, m0, M, lm, Mfull, K, klo, khi, S, s_buf, stage_floats, s_T,
-                    marg_out);
-    else
-      contract_item(P, R, precision, Pb, hv.f, 1.0f, m0, M, lm, Mfull, K, klo, khi, S, s_buf, stage_floats, s_T,
-                    marg_out);
-  }
-}
-
-cudaError_t launch_fold(const DevPlan& p, const DevRes& r, const EvalParams& e, const FoldSet& f,
-                        cudaStream_t s) {
-  if (f.total == 0) return cudaSuccess;
-  const long long blocks = (f.total + 255) / 256;
-  fold_kernel<<<(unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, s>>>(p, r, e, f.fidx, f.t_prefix, f.nf,
-                                                                            f.total); note_launch();
-  return cudaGetLastError();
-}
-
 // --- any topology ----------------------------------------------------------
 // A problem with no fragment on every cut (a chain or a tree of fragments,
 // Sec. V-C's general tensor network) is contracted pair by pair in an order
@@ -1617,6 +1581,79 @@ __device__ __forceinline__ void tree_entry(const DevPlan& P, const DevRes& R, co
   else R.gtmp[S.out_off + e] = acc;
 }
 
+// The first n steps of one problem by one CTA of 512 threads: the steps follow each
+// other at a block barrier instead of a launch.
+__device__ __noinline__ void tree_problem(const DevPlan& P, const DevRes& R, const ProblemDev& Pb, bool bf16, int n,
+                                          double* red, double* marg_out) {
+  const GStep* st = load_steps(P, Pb, red);
+  for (int i = 0; i < n; ++i) {
+    __syncthreads();
+    const GStep& S = st[i];
+    const int le = S.ma + S.mb + 2 * (S.fa + S.fb), lg = tree_lanes(9, le, S.ns);
+    for (long long b = 0; b < (1ll << (le + lg)); b += 512) tree_entry(P, R, S, bf16, b + threadIdx.x, lg, red, marg_out);
+  }
+}
+
+// TREES: plans with whole tree contractions (their code costs the others registers).
+template <bool TREES>
+__global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, int precision,
+                                                      const int2* direct_items, int n_direct, int stage_floats,
+                                                      const long long* z_prefix, int np, long long z_total, int z_warp,
+                                                      const int* trees, int n_trees, double* marg_out,
+                                                      double* zexp_out, KRange krg) {
+  extern __shared__ __align__(16) float s_buf[];   // two buffers of stage_floats
+  __shared__ double red[kRedDoubles];
+  __shared__ ProblemShared S;
+  __shared__ __align__(8) float s_T[kLeafStage];
+  const long long z_blocks = z_warp ? (z_total + 15) / 16 : z_total;
+  for (long long i = blockIdx.x; i < (TREES ? n_trees : 0) + n_direct + z_blocks; i += gridDim.x) {
+    if (TREES && i < n_trees) {
+      const ProblemDev& Pb = P.problems[trees[i]];
+      tree_problem(P, R, Pb, precision == CCS_BF16, Pb.g_count, red, marg_out);
+      __syncthreads();
+      continue;
+    }
+    const long long b = TREES ? i - n_trees : i;
+    if (b >= n_direct && z_warp) {
+      const int w = threadIdx.x >> 5;
+      const long long g = (b - n_direct) * 16 + w;
+      if (g < z_total) z_string_warp(P, R, z_prefix, np, g, s_T + w * kZWarp, zexp_out, krg);
+      __syncthreads();
+      continue;
+    }
+    if (b >= n_direct) {
+      z_string_block(P, R, z_prefix, np, b - n_direct, S, red, s_T, kLeafStage, zexp_out, krg);
+      __syncthreads();
+      continue;
+    }
+    const int2 di = direct_items[b];
+    const ProblemDev& Pb = P.problems[di.x];
+    const int M = Pb.TM, lm = __ffs(M) - 1;      // this block's hub outputs; extents are powers of two
+    const int m0 = di.y * M, Mfull = Pb.M;
+    const int K = (int)Pb.K;
+    const long long klo = krg.lo_of(K), khi = krg.hi_of(K);   // cut-index terms summed
+    // the hub's Q stored transposed: K x Mfull, row-major (this slice's columns from m0),
+    // FP32 or int16 count sums: one branch per slice, none per element
+    const HubView hv = hub_view(R, P.frags[Pb.frag0 + Pb.hub], Pb.hub_T_off + m0);
+    if (hv.h)
+      contract_item(P, R, precision, Pb, hv.h, hv.scale, m0, M, lm, Mfull, K, klo, khi, S, s_buf, stage_floats, s_T,
+                    marg_out);
+    else
+      contract_item(P, R, precision, Pb, hv.f, 1.0f, m0, M, lm, Mfull, K, klo, khi, S, s_buf, stage_floats, s_T,
+                    marg_out);
+  }
+}
+
+cudaError_t launch_fold(const DevPlan& p, const DevRes& r, const EvalParams& e, const FoldSet& f,
+                        cudaStream_t s) {
+  if (f.total == 0) return cudaSuccess;
+  const long long blocks = (f.total + 255) / 256;
+  fold_kernel<<<(unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, s>>>(p, r, e, f.fidx, f.t_prefix, f.nf,
+                                                                            f.total); note_launch();
+  return cudaGetLastError();
+}
+
+// --- any topology, continued -----------------------------------------------
 // One launch of independent steps (FoldSet: fidx = step, t_prefix = threads, a
 // multiple of a CTA's for each step).
 __global__ void __launch_bounds__(256) tree_level_kernel(DevPlan P, DevRes R, int precision, FoldSet f,
@@ -1629,18 +1666,11 @@ __global__ void __launch_bounds__(256) tree_level_kernel(DevPlan P, DevRes R, in
   }
 }
 
-// Every step but the last of one small problem, by one CTA: the steps follow
-// each other at a block barrier instead of a launch.
+// Every step but the last of one problem whose last step alone is large.
 __global__ void __launch_bounds__(512) tree_small_kernel(DevPlan P, DevRes R, int precision, const int* problems) {
-  __shared__ double red[16];
+  __shared__ double red[kRedDoubles];
   const ProblemDev& Pb = P.problems[problems[blockIdx.x]];
-  for (int i = 0; i + 1 < Pb.g_count; ++i) {
-    const GStep& S = P.gsteps[Pb.g_first + i];
-    const int le = S.ma + S.mb + 2 * (S.fa + S.fb), lg = tree_lanes(9, le, S.ns);
-    for (long long b = 0; b < (1ll << (le + lg)); b += 512)
-      tree_entry(P, R, S, precision == CCS_BF16, b + threadIdx.x, lg, red, nullptr);
-    __syncthreads();
-  }
+  tree_problem(P, R, Pb, precision == CCS_BF16, Pb.g_count - 1, red, nullptr);
 }
 
 // Partial cut-index ranges, which do not factor over the fragments, and
@@ -1772,22 +1802,24 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
       if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
   }
-  if ((z.has_general || (z.n_tree_levels > 0 && !z.krange.full())) && z.out_total > 0) {
+  if ((z.has_general || (z.n_tree_levels + z.n_tree_whole > 0 && !z.krange.full())) && z.out_total > 0) {
     general_contract_kernel<<<(unsigned)(z.out_total < 65535ll * 16 ? z.out_total : 65535ll * 16), 256, 0, s>>>(
         p, r, precision, z.out_prefix, p.n_problems, z.out_total, marg_out, z.krange);
     note_launch();
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  const long long blocks = z.n_direct + (z.z_warp ? (z.z_total + 15) / 16 : z.z_total);
+  const int n_trees = z.krange.full() ? z.n_tree_whole : 0;
+  const long long blocks = n_trees + z.n_direct + (z.z_warp ? (z.z_total + 15) / 16 : z.z_total);
   if (blocks > 0) {
     const size_t smem = (size_t)z.direct_stage_floats * 2 * 4;
+    auto kern = n_trees > 0 ? contract_kernel<true> : contract_kernel<false>;
     if (smem > 48 * 1024) {
-      err = cudaFuncSetAttribute(contract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (err != cudaSuccess) return err;
     }
-    contract_kernel<<<(unsigned)(blocks < 65535ll * 16 ? blocks : 65535ll * 16), 512, smem, s>>>(
+    kern<<<(unsigned)(blocks < 65535ll * 16 ? blocks : 65535ll * 16), 512, smem, s>>>(
         p, r, precision, z.direct_items, z.n_direct, z.direct_stage_floats, z.z_prefix, p.n_problems, z.z_total,
-        z.z_warp, marg_out, zexp_out, z.krange);
+        z.z_warp, z.tree_whole, n_trees, marg_out, zexp_out, z.krange);
     note_launch();
     err = cudaGetLastError();
   }
