@@ -121,7 +121,9 @@ void* dalloc(ccs_ctx c, size_t bytes) {
   void* p = nullptr;
   cudaMemPool_t pool = lib_pool(c->device);
   const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, c->stream) : cudaMallocAsync(&p, bytes, c->stream);
-  return e == cudaSuccess ? p : nullptr;
+  if (e == cudaSuccess) return p;
+  cudaGetLastError();      // reported here, not by the next launch
+  return nullptr;
 }
 
 void dfree(ccs_ctx c, void* p, size_t bytes) {
@@ -1667,8 +1669,6 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
       d.rowbasis = r->A.get<unsigned long long>(std::max<long long>((long long)kRowBasisWords * p->dp.n_cliff_frags, 1));
       d.zimg = r->A.get<unsigned long long>(std::max<long long>(p->n_zimg, 1));
       d.pbasis = r->A.get<uint32_t>(std::max<long long>(p->n_pbasis, 1));
-      d.gtmp = r->A.get<double>(std::max<long long>(p->n_gtmp, 1));
-
       d.status = r->A.get<unsigned>(4);
       r->scratch = r->A.get<float>(std::max<long long>(p->r_total + p->part_total, 1));
       {   // default launch shape before any tuning: wide tableaus take 8 words per op, 512 threads
@@ -1689,10 +1689,12 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
         r->rt_scratch = r->A.get<uint16_t>(p->rt_total);
       }
       if (!d.spaces || !d.dist || !d.qnz || !d.zval || !d.T || !d.TQ || !d.marg || !d.zexp || !d.work || !d.status ||
-          !d.body || !d.rowbasis || !d.zimg || !d.fragcnt || !d.pbasis || !d.gtmp ||
+          !d.body || !d.rowbasis || !d.zimg || !d.fragcnt || !d.pbasis ||
           !r->scratch || (p->rt_total && (!d.TQh || !r->rt_scratch))) {
         return fail(c, CCS_ERR_OOM, "result allocation failed");
       }
+      // tree contractions' intermediate tensors, last: without room for them those problems are summed directly
+      d.gtmp = r->A.get<double>(std::max<long long>(p->n_gtmp, 1));
       cudaMemsetAsync(d.status, 0, 4 * sizeof(unsigned), c->stream);
       *res = owned_r.release();
     }
@@ -1817,6 +1819,13 @@ int ccs_eval_variants(ccs_ctx c, ccs_plan p, const ccs_eval_opts* opts, ccs_res*
 
 void ccs_res_free(ccs_res r) { delete r; }
 
+// A result that found no room for the intermediate tensors sums its trees directly.
+static void no_trees_without_room(ccs_res r, RecombSizes& z) {
+  if (r->dr.gtmp) return;
+  if (z.n_tree_levels + z.n_tree_whole > 0) z.has_general = 1;
+  z.n_tree_levels = z.n_tree_small = z.n_tree_whole = 0;
+}
+
 static int check_status(ccs_ctx c, ccs_res r) {
   unsigned st[4];
   cudaError_t e = cudaMemcpyAsync(st, r->dr.status, sizeof(st), cudaMemcpyDeviceToHost, c->stream);
@@ -1843,6 +1852,7 @@ int ccs_recombine(ccs_ctx c, ccs_plan p, ccs_res r, const ccs_recomb_opts* opts,
                    p->pdev.data(), (int)p->pdev.size(), r->rt_scratch, tc ? 1 : 0, stitched ? 1 : 0, KRange{0, -1},
                    p->all_star ? 0 : 1, p->tree_levels.data(), (int)p->tree_levels.size(), p->d_tree_small,
                    p->n_tree_small, p->d_tree_whole, p->n_tree_whole};
+    no_trees_without_room(r, rz);
     if (opts && (opts->k_lo || opts->k_hi)) {
       if (opts->k_hi && opts->k_hi <= opts->k_lo) return fail(c, CCS_ERR_INVALID_ARG, "empty cut-index range");
       if (opts->k_lo > (1ull << 62) || opts->k_hi > (1ull << 62)) return fail(c, CCS_ERR_INVALID_ARG, "bad range");
@@ -2260,6 +2270,7 @@ extern "C" int ccs_recombine_noalloc(ccs_ctx c, ccs_plan p, ccs_res r, int preci
                    p->pdev.data(), (int)p->pdev.size(), nullptr, 0, r->ep.mode == CCS_STITCH ? 1 : 0,
                    KRange{0, -1}, p->all_star ? 0 : 1, p->tree_levels.data(), (int)p->tree_levels.size(), p->d_tree_small,
                    p->n_tree_small, p->d_tree_whole, p->n_tree_whole};
+    no_trees_without_room(r, rz);
     e = launch_recombine(p->dp, r->dr, precision, rz, scratch, marginal_out, zexp_out, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "recombine kernel");
     return CCS_OK;

@@ -146,7 +146,7 @@ struct DevRes {
   float* T;
   float* TQ;               // contraction operands: Q for hubs, T' for the other fragments
   uint16_t* TQh;           // bf16 copy of the hubs' Q (tensor-core path), may be null
-  double* gtmp;            // tree contractions: the intermediate tensors
+  double* gtmp;            // tree contractions: the intermediate tensors (null: no room, summed directly)
   double* marg;
   double* zexp;
   uint8_t* qnz;            // stitched results: per Clifford hub operand row, 1 unless identically zero

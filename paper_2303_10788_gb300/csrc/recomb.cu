@@ -1686,7 +1686,8 @@ __global__ void __launch_bounds__(256) general_contract_kernel(DevPlan P, DevRes
   for (long long b = blockIdx.x; b < total; b += gridDim.x) {
     const int pi = find_seg(out_prefix, np, b);
     const ProblemDev& Pb = P.problems[pi];
-    if (!Pb.general || (kr.full() && Pb.g_count)) continue;   // stars and trees: contracted by the other kernels
+    // stars and (if the result has room for their tensors) trees: contracted by the other kernels
+    if (!Pb.general || (kr.full() && Pb.g_count && R.gtmp)) continue;
     const long long o = b - out_prefix[pi];
     load_problem(P, Pb, S);
     __syncthreads();

@@ -57,6 +57,19 @@ def fat_edge(n, marginal_bits, triangle=False):
     return Workload("fat", c, cuts, ([0, p, 1, r] + a[2:])[:marginal_bits], [[0, p], [1, r], [0, 1]], 256, 3)
 
 
+def ring4():
+    """Fragments A, B, C, D joined in a ring by two cuts each, three marginal qubits
+    in each: two intermediate tensors of 2^6 outcomes x 4^4 cut digits."""
+    ab, bc, cd, ad, own = [0, 1], [2, 3], [4, 5], [6, 7], {"A": [8, 9, 10], "B": [11], "C": [12]}
+    c = Circuit(13)
+    cuts = []
+    for start, end, extra in ((ab + ad, [], own["A"]), (bc, ab, own["B"]), (cd, bc, own["C"]), ([], cd + ad, [])):
+        cuts += [(q, len(c.gates)) for q in end]
+        mixer(c, start + end + extra)
+    c.add(T, 4)
+    return Workload("ring4", c, cuts, [8, 9, 10, 0, 1, 11, 2, 3, 12, 4, 5, 6], [[0, 8], [3, 5, 6]], 256, 3)
+
+
 CASES = {
     "pair2": lambda: [fat_edge(2, 3)],
     "pair3_empty": lambda: [fat_edge(3, 0)],
@@ -67,6 +80,7 @@ CASES = {
     "triangle2": lambda: [fat_edge(2, 4, True)],
     "triangle4": lambda: [fat_edge(4, 1, True)],
     "triangle5": lambda: [fat_edge(5, 3, True)],
+    "ring4": lambda: [ring4()],
     "several": lambda: [fat_edge(2, 4, True), fat_edge(5, 2), fat_edge(3, 3, True), fat_edge(4, 0)],
 }
 
@@ -92,3 +106,32 @@ def test_fat_edges(name, mode):
         exact = [brute_force(w.circuit, w.marginal, w.zstrings) for w in ws]
         assert np.abs(m - np.concatenate([e[0] for e in exact])).max() < 1e-5
         assert np.abs(z - np.concatenate([e[1] for e in exact])).max() < 1e-5
+
+
+def test_without_room_for_the_intermediate_tensors(monkeypatch):
+    """The request for them is refused by the caller's allocator: the problems are
+    then summed directly, as they are over partial ranges."""
+    ws = [ring4()]
+    asked, refuse = [], []
+    real = ccs._TorchAllocator._alloc
+
+    def alloc(self, nbytes, stream, user):
+        asked.append(nbytes)
+        return None if len(asked) - 1 in refuse else real(self, nbytes, stream, user)
+    monkeypatch.setattr(ccs._TorchAllocator, "_alloc", alloc)
+
+    def run():
+        ctx = ccs.ccs_create(0)
+        plan = ccs.ccs_build_fragments(ctx, ws)
+        asked.clear()
+        res = ccs.ccs_eval_variants(ctx, plan, mode=ccs.CCS_EXACT)
+        out = [ccs.ccs_recombine(ctx, plan, res, use_graph=g) for g in (False, True)]
+        half = 4 ** max(len(w.cuts) for w in ws) // 2
+        parts = [ccs.ccs_recombine(ctx, plan, res, k_range=r) for r in ((0, half), (half, 0))]
+        return out, parts[0][0] + parts[1][0]
+    out, direct = run()
+    refuse.append(asked.index(2 * 4 ** 4 * 2 ** 6 * 8))
+    for m, z in run()[0]:
+        assert np.abs(m - direct).max() < 2e-6 and np.abs(m - out[0][0]).max() < 2e-6
+        assert np.abs(z - out[0][1]).max() < 2e-6
+    assert len(asked) > refuse[0]
