@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(256) build_r_kernel(DevPlan P, DevRes R, int p
                                                       int stitched, int full_range) {
   __shared__ ProblemShared S;
   const long long span = 256ll * kRPerThread;
+  total = min(total, prefix[np]);      // past the last problem there would be no stretch to step over
   for (long long base = blockIdx.x * span; base < total; base += gridDim.x * span) {
     const long long end = min(total, base + span);
     for (long long g0 = base; g0 < end;) {              // the problems this stretch crosses
