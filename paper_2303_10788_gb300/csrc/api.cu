@@ -1072,7 +1072,7 @@ int ccs_build_fragments(ccs_ctx c, const ccs_problem* probs, int n_problems, con
       if (d.nz > 0) {
         long long entries = 0;
         for (int l = 0; l < d.n_frags; ++l) entries += 1ll << (2 * plan->fdev[f0 + l].n_slots);
-        if (entries > 128 || d.k > 3) plan->z_warp = false;
+        if (entries > kZWarp || d.k > kZWarpCuts) plan->z_warp = false;
       }
       plan->out_prefix.push_back(plan->n_marg);
       plan->z_prefix.push_back(plan->n_zexp);

@@ -96,6 +96,8 @@ struct GStep {
   uint8_t pos[kMaxMarginal];        // last step: output bit of every marginal bit of A, then of B
 };
 constexpr int kZTree = 1024;        // doubles of Z-string tensors a tree contraction stages per string
+// A warp per Z-string: the string entries of all of a problem's fragments, and its cuts.
+constexpr int kZWarp = 128, kZWarpCuts = 3;
 
 // Device views of a plan + result.
 struct DevPlan {

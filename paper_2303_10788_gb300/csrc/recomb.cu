@@ -1268,10 +1268,9 @@ __device__ __noinline__ void z_string_block(const DevPlan& P, const DevRes& R, c
 }
 
 // The same by one warp per string, for plans of many strings whose fragments
-// have at most kZWarp string entries in all (k <= 3): sixteen strings a CTA and
+// have at most kZWarp string entries in all (k <= kZWarpCuts): sixteen strings a CTA and
 // no barrier (512 strings of 64 circuits: the kernel 17.7 us with a CTA per
 // string, 10.4 us so).
-constexpr int kZWarp = 128;
 __device__ __noinline__ void z_string_warp(const DevPlan& P, const DevRes& R, const long long* prefix, int np, long long g,
                                            float* s_tz, double* zexp_out, KRange kr) {
   const int lane = threadIdx.x & 31, pi = find_seg(prefix, np, g);
