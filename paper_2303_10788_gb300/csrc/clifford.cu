@@ -244,7 +244,8 @@ __device__ void prep_rows_from_body(const CliffordOp* s_prep, const int* s_qin, 
 // run in a single warp with no block barrier.  A deep narrow body (301 wires,
 // 307 moments) took 790 cycles a moment with eight lanes per op, a shuffle
 // reduction and a barrier each: 117 us for 64 such bodies,
-// 43 us so; 86 wires in 20 moments: 15 and 7.7 us.
+// 42 us so with nothing cached (34 us in a replayed evaluation); 86 wires in 20
+// moments: 15 and 7.7 us.
 namespace {
 // An op as the kernel stages it: x = the byte offsets of columns X_a (low half)
 // and X_b, y = M | sign form << 16 without the form's constant term.  Lanes
@@ -469,11 +470,6 @@ __global__ void __launch_bounds__(MODE == 0 ? 32 : MODE == 1 ? 1024 : 256) body_
 // changes H, S^+ then H, and none); k = nz + 3 qout + t is Z on marginal
 // wire t.
 namespace {
-
-__device__ __forceinline__ unsigned long long warp_xor64(unsigned long long x) {
-  for (int o = 16; o; o >>= 1) x ^= __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
 
 // One record, by one CTA: the anticommutation bits (acc, by warp 0), then
 // the phase of the ordered row product, threads over the body's columns.  Per

@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(256) ml_rebuild_kernel(DevPlan P, DevRes R, co
 // sweep.  A two-sided Jacobi in shared memory moves the whole block and its
 // eigenvectors once per round of D/2 pairs and is bound by that traffic (46%
 // bank conflicts) and two barriers a round: 768 blocks of 64 x 64 took 4.30 ms
-// and 1280 of 16 x 16 0.28 ms, here 0.89 and 0.047 ms (issue and the steps'
+// and 1280 of 16 x 16 0.28 ms, here 0.93 and 0.050 ms (issue and the steps'
 // latency: 51% of the issue slots at the four CTAs per SM the registers allow).
 // D = 16 packs two blocks into a warp (they sweep until both are done).
 template <int D>

@@ -310,7 +310,7 @@ struct ProblemShared {
   long long T_off[kMaxProblemFrags];
 };
 
-// A warp per fragment, a lane per array entry (at least as many warps as fragments).
+// The warps take the fragments in turn, a lane per array entry (27 lanes used).
 __device__ void load_problem(const DevPlan& P, const ProblemDev& Pb, ProblemShared& S) {
   const int l = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) { S.nf = Pb.n_frags; S.hub = Pb.hub; S.k = Pb.k; }
@@ -1325,7 +1325,7 @@ __device__ __forceinline__ float hub_elem(const int16_t* A, float sc, long long 
 //   Y[r][x][m] = sum_g Q^T[kr(r) | kg(g)][m0 + m] T'[x][g]
 // (r: the other leaves' digits, g: this leaf's, x: its outputs), each thread
 // VW consecutive hub outputs (one vector load per row) and two outputs x
-// (every operand load used twice), four rows in flight.
+// (every operand load used twice), kFirstRows rows in flight.
 template <class T> constexpr int first_vec() { return sizeof(T) == 2 ? 4 : 2; }   // hub outputs per thread
 constexpr int kFirstX = 2;      // leaf outputs per thread (1 or 2)
 constexpr int kFirstRows = 8;   // operand rows in flight per thread
