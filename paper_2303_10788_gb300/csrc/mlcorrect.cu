@@ -323,7 +323,9 @@ __global__ void __launch_bounds__(256, 3) ml_eig_kernel(DevPlan P, DevRes R, con
 // registers up to 16 per thread.  A pass adds the kept values in three FP32
 // parts (no fewer bits than FP64) and only the warps' sums in FP64: with FP64
 // adds and compares per value a pass was bound by the FP64 units (16 fragments
-// of 8192 values: 76 us, 32 us so; a pair of FP32 parts, of fewer bits, 25 us).
+// of 8192 values: 76 us, 33 us so; a pair of FP32 parts, of fewer bits, 25 us).
+// Warps past the last value add and shuffle nothing: corrections of a few hundred
+// values took 2 to 4 us more otherwise.
 constexpr int kThetaThreads = 1024, kThetaRegs = 16;
 
 __global__ void __launch_bounds__(kThetaThreads) ml_threshold_kernel(DevPlan P, const MlFrag* __restrict__ fr,
@@ -356,8 +358,10 @@ __global__ void __launch_bounds__(kThetaThreads) ml_threshold_kernel(DevPlan P, 
     int cnt = 0;
     if (in_regs) {
 #pragma unroll
-      for (int i = 0; i < kThetaRegs; ++i)
+      for (int i = 0; i < kThetaRegs; ++i) {
+        if (32 * warp + (long long)i * kThetaThreads >= n) break;      // the warp's values end here
         if (v[i] > cut) { s.add(v[i]); ++cnt; }
+      }
     } else {
 #pragma unroll 4
       for (long long i = tid; i < n; i += kThetaThreads) {
@@ -365,14 +369,16 @@ __global__ void __launch_bounds__(kThetaThreads) ml_threshold_kernel(DevPlan P, 
         if (x > cut) { s.add(x); ++cnt; }
       }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      Sum3 other;
-      other.s = __shfl_xor_sync(0xffffffffu, s.s, o);
-      other.c = __shfl_xor_sync(0xffffffffu, s.c, o);
-      other.e = __shfl_xor_sync(0xffffffffu, s.e, o);
-      s.add(other);
+    if (32 * warp < n) {
+      for (int o = 16; o > 0; o >>= 1) {
+        Sum3 other;
+        other.s = __shfl_xor_sync(0xffffffffu, s.s, o);
+        other.c = __shfl_xor_sync(0xffffffffu, s.c, o);
+        other.e = __shfl_xor_sync(0xffffffffu, s.e, o);
+        s.add(other);
+      }
+      cnt = __reduce_add_sync(0xffffffffu, cnt);
     }
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) {
       s_sum[warp] = s.value();
       s_cnt[warp] = cnt;
