@@ -1328,7 +1328,7 @@ __device__ __forceinline__ float hub_elem(const int16_t* A, float sc, long long 
 // (every operand load used twice), kFirstRows rows in flight.
 template <class T> constexpr int first_vec() { return sizeof(T) == 2 ? 4 : 2; }   // hub outputs per thread
 constexpr int kFirstX = 2;      // leaf outputs per thread (1 or 2)
-constexpr int kFirstRows = 8;   // operand rows in flight per thread
+constexpr int kFirstRows = 4;   // operand rows in flight per thread (divides G: a first leaf streamed has a slot)
 template <int VW, int NX, class T, class Expand>
 __device__ __forceinline__ void first_leaf_global(const T* __restrict__ At, float sc, int bf16, long long Mfull,
                                                   int lm, int lG, int ml, int lrest, long long klo, long long khi,
@@ -1347,25 +1347,24 @@ __device__ __forceinline__ void first_leaf_global(const T* __restrict__ At, floa
 #pragma unroll
     for (int v = 0; v < VW; ++v) { s0[v] = c0[v] = 0.f; if (NX == 2) s1[v] = c1[v] = 0.f; }
     const T* base = At + mv * VW;
-    for (int g0 = 0; g0 < G; g0 += kFirstRows) {      // G = 4^slots: 4, or a multiple of 8
+    for (int g0 = 0; g0 < G; g0 += kFirstRows) {
       using Raw = typename RawVec<T, VW>::type;
       Raw a[kFirstRows];
 #pragma unroll
       for (int u = 0; u < kFirstRows; ++u) {
         const int g = g0 + u;
         int kg;
-        if (kg_tab) kg = g < G ? kg_tab[g] : 0;
+        if (kg_tab) kg = kg_tab[g];
         else {
           kg = 0;
           for (int i = 0; i < S.ns[l]; ++i) kg |= ((g >> (2 * i)) & 3) << (2 * S.slot_cut[l][i]);
         }
         const long long kk = (long long)(kr | kg);
-        a[u] = (g < G && kk >= klo && kk < khi) ? __ldg(reinterpret_cast<const Raw*>(base + kk * Mfull)) : Raw{};
+        a[u] = (kk >= klo && kk < khi) ? __ldg(reinterpret_cast<const Raw*>(base + kk * Mfull)) : Raw{};
       }
 #pragma unroll
       for (int u = 0; u < kFirstRows; ++u) {
         const int g = g0 + u;
-        if (g >= G) break;                              // G = 4: half a batch
         float t0 = tv[x0 * G + g], t1 = nx == 2 ? tv[(x0 + 1) * G + g] : 0.f;
         if (bf16 && !tv_rounded) { t0 = to_bf16f(t0); t1 = to_bf16f(t1); }
 #pragma unroll
@@ -1397,24 +1396,17 @@ __device__ __forceinline__ void contract_item(const DevPlan& P, const DevRes& R,
   __syncthreads();
   float* X = s_buf;
   float* Y = s_buf + stage_floats;
-  // cut positions of the digits in leaf order (four bits each, the first leaf's
-  // lowest), and each leaf's first digit
-  unsigned long long digits = 0ull;
-  {
-    int nd = 0;
-    for (int l = 0; l < S.nf; ++l) {
-      if (l == S.hub) continue;
-      for (int i = 0; i < S.ns[l]; ++i) digits |= (unsigned long long)S.slot_cut[l][i] << (4 * nd++);
-    }
-  }
   // compact cut index (groups in leaf order, the first leaf's lowest) ->
   // cut index, for the digits of leaves from `from` on
   auto expand = [&](int kc, int from) -> int {
-    unsigned long long ps = digits;
-    for (int l = 0; l < from; ++l)
-      if (l != S.hub) ps >>= 4 * S.ns[l];
-    int k = 0;
-    for (int rem = kc; rem; rem >>= 2, ps >>= 4) k |= (rem & 3) << (2 * (int)(ps & 15ull));
+    int k = 0, rem = kc;
+    for (int l = from; l < S.nf; ++l) {
+      if (l == S.hub) continue;
+      for (int i = 0; i < S.ns[l]; ++i) {
+        k |= (rem & 3) << (2 * S.slot_cut[l][i]);
+        rem >>= 2;
+      }
+    }
     return k;
   };
   int first = 0;
@@ -1594,8 +1586,10 @@ __device__ __noinline__ void tree_problem(const DevPlan& P, const DevRes& R, con
   }
 }
 
-// TREES: plans with whole tree contractions (their code costs the others registers).
-template <bool TREES>
+// What a plan does not need is left out, as it costs the rest registers (146 bytes
+// spilled with everything in): Z, Z-strings; OP, the stars' operands (1 FP32, 2 int16
+// count sums, 0 either); TREES, whole tree contractions.
+template <int OP, bool Z, bool TREES>
 __global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, int precision,
                                                       const int2* direct_items, int n_direct, int stage_floats,
                                                       const long long* z_prefix, int np, long long z_total, int z_warp,
@@ -1605,7 +1599,7 @@ __global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, i
   __shared__ double red[kRedDoubles];
   __shared__ ProblemShared S;
   __shared__ __align__(8) float s_T[kLeafStage];
-  const long long z_blocks = z_warp ? (z_total + 15) / 16 : z_total;
+  const long long z_blocks = !Z ? 0 : z_warp ? (z_total + 15) / 16 : z_total;
   for (long long i = blockIdx.x; i < (TREES ? n_trees : 0) + n_direct + z_blocks; i += gridDim.x) {
     if (TREES && i < n_trees) {
       const ProblemDev& Pb = P.problems[trees[i]];
@@ -1614,14 +1608,14 @@ __global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, i
       continue;
     }
     const long long b = TREES ? i - n_trees : i;
-    if (b >= n_direct && z_warp) {
+    if (Z && b >= n_direct && z_warp) {
       const int w = threadIdx.x >> 5;
       const long long g = (b - n_direct) * 16 + w;
       if (g < z_total) z_string_warp(P, R, z_prefix, np, g, s_T + w * kZWarp, zexp_out, krg);
       __syncthreads();
       continue;
     }
-    if (b >= n_direct) {
+    if (Z && b >= n_direct) {
       z_string_block(P, R, z_prefix, np, b - n_direct, S, red, s_T, kLeafStage, zexp_out, krg);
       __syncthreads();
       continue;
@@ -1633,9 +1627,9 @@ __global__ void __launch_bounds__(512, 2) contract_kernel(DevPlan P, DevRes R, i
     const int K = (int)Pb.K;
     const long long klo = krg.lo_of(K), khi = krg.hi_of(K);   // cut-index terms summed
     // the hub's Q stored transposed: K x Mfull, row-major (this slice's columns from m0),
-    // FP32 or int16 count sums: one branch per slice, none per element
+    // FP32 or int16 count sums: one branch per slice at most, none per element
     const HubView hv = hub_view(R, P.frags[Pb.frag0 + Pb.hub], Pb.hub_T_off + m0);
-    if (hv.h)
+    if (OP == 2 || (OP == 0 && hv.h))
       contract_item(P, R, precision, Pb, hv.h, hv.scale, m0, M, lm, Mfull, K, klo, khi, S, s_buf, stage_floats, s_T,
                     marg_out);
     else
@@ -1813,7 +1807,15 @@ cudaError_t launch_recombine(const DevPlan& p, const DevRes& r, int precision, c
   const long long blocks = n_trees + z.n_direct + (z.z_warp ? (z.z_total + 15) / 16 : z.z_total);
   if (blocks > 0) {
     const size_t smem = (size_t)z.direct_stage_floats * 2 * 4;
-    auto kern = n_trees > 0 ? contract_kernel<true> : contract_kernel<false>;
+    int ops = 0;                       // 1: FP32 operands among the stars, 2: count sums
+    for (int i = 0; i < z.n_problems; ++i) {
+      const ProblemDev& Pb = z.host_problems[i];
+      if (Pb.direct) ops |= r.hub_i16 && Pb.hub_qrow_off >= 0 ? 2 : 1;
+    }
+    const bool zs = z.z_total > 0;
+    auto kern = n_trees > 0 || ops == 3 ? contract_kernel<0, true, true>
+                : ops == 2              ? (zs ? contract_kernel<2, true, false> : contract_kernel<2, false, false>)
+                                        : (zs ? contract_kernel<1, true, false> : contract_kernel<1, false, false>);
     if (smem > 48 * 1024) {
       err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (err != cudaSuccess) return err;
