@@ -1523,13 +1523,13 @@ __device__ __forceinline__ void contract_item(const DevPlan& P, const DevRes& R,
 // chosen when the plan is built: 4^(open cuts) entries per outcome instead of
 // a sum over all 4^k terms for every output (nine blocks in a chain, 4^8 terms
 // x 2^10 outputs: 1.80 ms as a direct sum and 0.25 ms for eight Z-strings; the
-// whole call went from 2.09 to 0.11 ms).  The steps are short sums over few
+// whole call went from 2.09 to 0.08 ms).  The steps are short sums over few
 // shared digits, so they are bound by launch and load latency; FP64 throughout
 // costs nothing there, and leaves only the tensors' own FP32 rounding.
 // Two fragments with many cuts between them make the sum long and the entries
 // few, so that up to a CTA's threads share an entry (recombination of a pair
 // joined by four cuts beside another pair: 254 us with one thread per entry,
-// 95 us so).
+// 77 us so; both with its Z-strings).
 __device__ __forceinline__ double tree_sum(const GStep& S, const float* __restrict__ T, const double* tmp, bool bf16,
                                            long long ia, long long ib, int lane, int lg) {
   double acc = 0.0;
