@@ -1192,6 +1192,40 @@ __device__ float fold_z_value(const DevRes& R, const FragDev& F, int zi, int Pi)
   return (float)acc;
 }
 
+// The same of a tree of fragments: its contraction steps, without marginal bits (a
+// function of its own: the sum over the cut index below keeps its registers).
+__device__ __noinline__ void z_tree_block(const DevPlan& P, const DevRes& R, const ProblemDev& Pb, int zi,
+                                          const ProblemShared& S, double* red, float* s_tz, double* zexp_out) {
+  double* zt = reinterpret_cast<double*>(s_tz);
+  GStep* st = load_steps(P, Pb, red);
+  int tot = 0;
+  for (int l = 0; l < S.nf; ++l) tot += 1 << (2 * S.ns[l]);
+  for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+    int l = 0, o = 0;
+    while (i >= o + (1 << (2 * S.ns[l]))) { o += 1 << (2 * S.ns[l]); ++l; }
+    zt[i] = (double)fold_z_value(R, P.frags[Pb.frag0 + l], zi, i - o);
+  }
+  for (int t = 0; t < Pb.g_count; ++t) {
+    __syncthreads();
+    const GStep& G = st[t];
+    const int le = 2 * (G.fa + G.fb), lg = tree_lanes(9, le, G.ns);      // 512 threads
+    for (int g = threadIdx.x; g < (blockDim.x > (1u << le) ? (int)blockDim.x : 1 << le); g += blockDim.x) {
+      const int e = g >> lg;
+      double acc = 0.0;
+      if (e < (1 << le)) {
+        const int ia = (int)spread(e & ((1 << (2 * G.fa)) - 1), G.fa, G.a_free);
+        const int ib = (int)spread(e >> (2 * G.fa), G.fb, G.b_free);
+        for (int q = g & ((1 << lg) - 1); q < (1 << (2 * G.ns)); q += 1 << lg)
+          acc = fma(zt[G.za + (ia | (int)spread(q, G.ns, G.a_sh))], zt[G.zb + (ib | (int)spread(q, G.ns, G.b_sh))], acc);
+      }
+      acc = lanes_sum(acc, lg, red);
+      if (e >= (1 << le) || (g & ((1 << lg) - 1))) continue;
+      if (G.last) zexp_out[Pb.zexp_off + zi] = ldexp(acc, -S.k);
+      else zt[G.zo + e] = acc;
+    }
+  }
+}
+
 // <Z_S> = 2^-k sum_P prod_f T_f^S(P|f): one block per (problem, string),
 // FP32 products, FP64 sums, fixed-order tree reduction; T_f^S is folded from
 // the variants' Z values here (no separate fold pass).
@@ -1202,58 +1236,41 @@ __device__ __noinline__ void z_string_block(const DevPlan& P, const DevRes& R, c
   const int zi = (int)(g - prefix[pi]);
   load_problem(P, Pb, S);
   __syncthreads();
-  if (Pb.g_zlen && kr.full()) {   // a tree of fragments: its contraction steps, without marginal bits
-    double* zt = reinterpret_cast<double*>(s_tz);
-    GStep* st = load_steps(P, Pb, red);
-    int tot = 0;
-    for (int l = 0; l < S.nf; ++l) tot += 1 << (2 * S.ns[l]);
-    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-      int l = 0, o = 0;
-      while (i >= o + (1 << (2 * S.ns[l]))) { o += 1 << (2 * S.ns[l]); ++l; }
-      zt[i] = (double)fold_z_value(R, P.frags[Pb.frag0 + l], zi, i - o);
-    }
-    for (int t = 0; t < Pb.g_count; ++t) {
-      __syncthreads();
-      const GStep& G = st[t];
-      const int le = 2 * (G.fa + G.fb), lg = tree_lanes(9, le, G.ns);      // 512 threads
-      for (int g = threadIdx.x; g < (blockDim.x > (1u << le) ? (int)blockDim.x : 1 << le); g += blockDim.x) {
-        const int e = g >> lg;
-        double acc = 0.0;
-        if (e < (1 << le)) {
-          const int ia = (int)spread(e & ((1 << (2 * G.fa)) - 1), G.fa, G.a_free);
-          const int ib = (int)spread(e >> (2 * G.fa), G.fb, G.b_free);
-          for (int q = g & ((1 << lg) - 1); q < (1 << (2 * G.ns)); q += 1 << lg)
-            acc = fma(zt[G.za + (ia | (int)spread(q, G.ns, G.a_sh))], zt[G.zb + (ib | (int)spread(q, G.ns, G.b_sh))], acc);
-        }
-        acc = lanes_sum(acc, lg, red);
-        if (e >= (1 << le) || (g & ((1 << lg) - 1))) continue;
-        if (G.last) zexp_out[Pb.zexp_off + zi] = ldexp(acc, -S.k);
-        else zt[G.zo + e] = acc;
-      }
-    }
+  if (Pb.g_zlen && kr.full()) {
+    z_tree_block(P, R, Pb, zi, S, red, s_tz, zexp_out);
     return;
   }
-  // every fragment's T_f^S(zi, .) folded once into shared memory when it fits
+  // the fragments' T_f^S(zi, .) folded once into shared memory, in order, each that
+  // still fits; a wide hub's entries are used once each and stay where they are
   int tz_tot = 0;
-  for (int l = 0; l < S.nf; ++l) tz_tot += 1 << (2 * S.ns[l]);
-  const bool staged = tz_tot <= tz_cap;
-  if (staged) {
-    for (int i = threadIdx.x; i < tz_tot; i += blockDim.x) {
-      int l = 0, o = 0;
-      while (i >= o + (1 << (2 * S.ns[l]))) { o += 1 << (2 * S.ns[l]); ++l; }
-      s_tz[i] = fold_z_value(R, P.frags[Pb.frag0 + l], zi, i - o);
-    }
-    __syncthreads();
+  for (int l = 0; l < S.nf; ++l) {
+    const int n = 1 << (2 * S.ns[l]);
+    if (tz_tot + n <= tz_cap) tz_tot += n;
   }
+  for (int i = threadIdx.x; i < tz_tot; i += blockDim.x) {
+    int l = 0, o = 0;
+    for (;; ++l) {
+      const int n = 1 << (2 * S.ns[l]);
+      if (o + n > tz_cap) continue;
+      if (i < o + n) break;
+      o += n;
+    }
+    s_tz[i] = fold_z_value(R, P.frags[Pb.frag0 + l], zi, i - o);
+  }
+  __syncthreads();
   const long long K = 1ll << (2 * S.k);
   double part = 0.0;
   for (long long Pp = kr.lo_of(K) + threadIdx.x; Pp < kr.hi_of(K); Pp += blockDim.x) {
     float t = 1.f;
     int o = 0;
     for (int l = 0; l < S.nf; ++l) {
-      const int pl = frag_digits(S, l, Pp);
-      t *= staged ? s_tz[o + pl] : fold_z_value(R, P.frags[Pb.frag0 + l], zi, pl);
-      o += 1 << (2 * S.ns[l]);
+      const int pl = frag_digits(S, l, Pp), n = 1 << (2 * S.ns[l]);
+      if (o + n <= tz_cap) {
+        t *= s_tz[o + pl];
+        o += n;
+      } else {
+        t *= fold_z_value(R, P.frags[Pb.frag0 + l], zi, pl);
+      }
     }
     part += (double)t;
   }
